@@ -15,6 +15,7 @@
 // a cell's Gaussians are copied into the warp's shared memory asynchronously
 // two cells ahead and broadcast from there to the warp's 128 pixels.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -54,11 +55,14 @@ constexpr int WT = 32;  // threads per work unit
 constexpr int NSTAGE = 3;
 
 // Issue the copy of the records of cell `id` (per float4s) into dst.
+// KT > 0: K at compile time (one or two pieces a lane for the common ones).
+template <int KT>
 __device__ __forceinline__ void issue_cell(float4 *dst, const float4 *__restrict__ vrec, uint32_t id, int per,
                                            int lane) {
     const float4 *src = vrec + (long long)id * per;
+    constexpr int PIECES = ((KT > 0 ? KT : kMaxK) * kRecF4 + 31) / 32;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
+    for (int q = 0; q < PIECES; ++q) {
         const int i = lane + 32 * q;
         if (i < per) cp_async16(dst + i, src + i);
     }
@@ -165,7 +169,7 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
     CellFeed feed{cells, rg.x, rg.y, 0u};
 #pragma unroll
     for (int b = 0; b < NSTAGE - 1; ++b) {
-        if (rg.x + b < rg.y) issue_cell(s_rec[b], vrec, feed.id(rg.x + b, lane), per, lane);
+        if (rg.x + b < rg.y) issue_cell<KT>(s_rec[b], vrec, feed.id(rg.x + b, lane), per, lane);
         cp_async_commit();
     }
     int buf = 0;
@@ -179,7 +183,7 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
         }
         if (__all_sync(0xffffffffu, all)) break;
         const int fill = buf == 0 ? NSTAGE - 1 : buf - 1;  // the buffer of entry e - 1, read by now
-        if (e + NSTAGE - 1 < rg.y) issue_cell(s_rec[fill], vrec, feed.id(e + NSTAGE - 1, lane), per, lane);
+        if (e + NSTAGE - 1 < rg.y) issue_cell<KT>(s_rec[fill], vrec, feed.id(e + NSTAGE - 1, lane), per, lane);
         cp_async_commit();
         cp_async_wait<NSTAGE - 1>();
         __syncwarp();
@@ -224,7 +228,10 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
                     // outside the box along a column or a row: an offset far off
                     // the Gaussian, so exp2 gives alpha = +0 exactly (in-box pixels
                     // compute as before; a done pixel's sums are not used)
-                    any = (hx[0] || hx[1]) && (hy[0] || hy[NR - 1]);
+                    bool anyy = hy[0];
+#pragma unroll
+                    for (int rr = 1; rr < NR; ++rr) anyy = anyy || hy[rr];
+                    any = (hx[0] || hx[1]) && anyy;
 #pragma unroll
                     for (int c = 0; c < 2; ++c) dx[c] = hx[c] ? dx[c] : kFar;
 #pragma unroll
@@ -484,33 +491,28 @@ void launch_count_pairs(const ViewDesc *views, int n_views, int total_tiles, con
 // values a lane carries) and adds the totals to global memory (one atomic
 // add per value per sub-tile).
 
-// Sum v[0..7] over the warp.  On return lane L holds the total of value
-// 4 b2 + 2 b3 + b4 (b_i = bit i of L; transposed_owner8); the four lanes that
-// differ only in b0 and b1 hold the same total.
-// Transposed warp reduction of eight per-lane values: three halving steps
-// (offsets 16, 8, 4) in which each lane keeps half of its slots and receives
-// its partner's other half, then two butterfly steps (offsets 2, 1).  Every
-// lane ends with the warp total of slot transposed_owner8(lane): 9 shuffles
-// instead of 8 x 5.
-__device__ __forceinline__ float transposed_warp_sum8(float v[8], int lane) {
+// Sums of eight per-lane values over the eight lanes of a group (lanes that
+// differ in bits 0..2): three halving steps (offsets 4, 2, 1) in which each
+// lane keeps half of its values and receives its partner's other half, so
+// lane L ends with the group's total of value group_owner8(L): 7 shuffles
+// instead of 8 x 3.
+__device__ __forceinline__ float group_sum8(float v[8], int lane) {
 #pragma unroll
     for (int step = 0; step < 3; ++step) {
-        const int bit = 16 >> step;
+        const int bit = 4 >> step;
         const bool hi = lane & bit;
-        const int n = 4 >> step;  // pairs at this step
 #pragma unroll
-        for (int i = 0; i < n; ++i) {
+        for (int i = 0; i < (4 >> step); ++i) {
             const float keep = hi ? v[2 * i + 1] : v[2 * i];
             const float send = hi ? v[2 * i] : v[2 * i + 1];
             v[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
         }
     }
-    const float t = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 2);
-    return t + __shfl_xor_sync(0xffffffffu, t, 1);
+    return v[0];
 }
 
-__device__ __forceinline__ int transposed_owner8(int lane) {
-    return ((lane >> 2) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 4) & 1);
+__device__ __forceinline__ int group_owner8(int lane) {
+    return ((lane >> 2) & 1) + ((lane >> 1) & 1) * 2 + (lane & 1) * 4;
 }
 
 __device__ __forceinline__ float warp_sum(float a) {
@@ -526,64 +528,56 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
-// Screen-space gradient terms of (pixel, Gaussian) pairs for the two pixels
-// of one lane row at once (one f32x2 operation per pixel pair), with the
-// constant factors left to the caller (applied once per reduced total):
-//   acc[1], acc[4] = sum dq' dy, sum dq' dy^2 per column (column_terms forms
-//   the lane's moments sum dq' (dx, dy), which mean_terms makes the mean's,
-//   and sum dq' (dx^2, dx dy, dy^2): da, db, dc = -1/2, -1, -1/2 x acc)
-//   acc[5..7] = sum v T alpha e       (drgb)
-//   dop       = sum dalpha G          (dsigma)
-//   pv       += alpha / (1 - v alpha)  (per pixel; times -S_n, dL/dv's share)
-// with dq' = G dalpha sigma = -2 dL/dq.  cA = v T_n and nvS = -v S_n are the
-// pixels' per-cell factors (formed once per cell); dx the lane's column
-// offsets (shared by its rows).  A pixel with G' = 0 (not reached, or inactive) adds
-// exactly 0, and the opacity-clamped branch is a select, so no per-pixel
-// branch remains.
-template <bool WV>
-__device__ __forceinline__ void pair_grad2(float2 acc[8], float2 &dop, float2 &pv, float2 Gv, float4 r0, float4 r1,
-                                           float4 r2, float2 dx, float py, float2 cA, float2 nvS,
-                                           float2 e0, float2 e1, float2 e2, float2 eD, float alpha_max) {
-    const float v = r2.w, op = r1.w;
-    const float2 raw = __fmul2_rn(make_float2(op, op), Gv);
-    const float2 al = make_float2(fminf(raw.x, alpha_max), fminf(raw.y, alpha_max));
-    const float2 om = __ffma2_rn(make_float2(-v, -v), al, make_float2(1.0f, 1.0f));
-    const float2 rom = make_float2(rcp_approx(om.x), rcp_approx(om.y));
-    const float2 inner = __ffma2_rn(
-        e0, make_float2(r2.x, r2.x),
-        __ffma2_rn(e1, make_float2(r2.y, r2.y), __ffma2_rn(e2, make_float2(r2.z, r2.z), eD)));
-    const float2 dal = __ffma2_rn(nvS, rom, __fmul2_rn(cA, inner));
-    const float2 ca_al = __fmul2_rn(cA, al);
-    acc[5] = __ffma2_rn(ca_al, e0, acc[5]);
-    acc[6] = __ffma2_rn(ca_al, e1, acc[6]);
-    acc[7] = __ffma2_rn(ca_al, e2, acc[7]);
-    if (WV) pv = __ffma2_rn(al, rom, pv);
-    float2 dG = __fmul2_rn(dal, Gv);
-    dG.x = raw.x < alpha_max ? dG.x : 0.f;
-    dG.y = raw.y < alpha_max ? dG.y : 0.f;
-    dop = __fadd2_rn(dop, dG);
-    // per column of the lane (dx is the same for its rows): sum dq' dy and
-    // sum dq' dy^2; the dx-weighted sums follow from dop (dq' = sigma dG)
-    // and these in column_terms
-    const float dys = py - r0.y, opdy = op * dys;
-    const float2 dqy = __fmul2_rn(dG, make_float2(opdy, opdy));
-    acc[1] = __fadd2_rn(acc[1], dqy);
-    acc[4] = __ffma2_rn(dqy, make_float2(dys, dys), acc[4]);
-}
+// One lane's sums of a Gaussian's screen-space gradient terms over its pixels
+// (components x, y: its two columns; e the pixel's dL/dN):
+//   dop = sum dG                 (dsigma)
+//   Y, Q = sum dG dy, sum dG dy^2  (times sigma: the moments of dq' = -2 dL/dq;
+//          the dx-weighted ones follow per column at the end)
+//   C    = sum v T alpha e, less the factor `colour` (drgb)
+//   dv   = sum -S_n alpha / (1 - v alpha), less the same factor (dL/dv_n's share)
+struct LaneGrad {
+    float2 dop, Y, Q, C0, C1, C2, dv;
+};
 
-// A lane's totals of slots 0..4 from its per-column sums (components x, y:
-// its two columns, offsets dx from the Gaussian's centre): with D = sigma dop
-// = sum dq' per column and Y = acc[1] = sum dq' dy per column,
-//   sum dq' dx = D.dx, sum dq' dy = sum Y, sum dq' dx^2 = D.dx^2,
-//   sum dq' dx dy = Y.dx, sum dq' dy^2 = sum acc[4].
-__device__ __forceinline__ void column_terms(const float2 acc2[8], float2 dop, float op, float2 dx, float acc[8]) {
-    const float2 D = __fmul2_rn(dop, make_float2(op, op));
-    const float2 t = __fmul2_rn(D, dx);
-    acc[0] = t.x + t.y;
-    acc[1] = acc2[1].x + acc2[1].y;
-    acc[2] = fmaf(t.x, dx.x, t.y * dx.y);
-    acc[3] = fmaf(acc2[1].x, dx.x, acc2[1].y * dx.y);
-    acc[4] = acc2[4].x + acc2[4].y;
+// A Gaussian's terms at one pixel pair of a row: G' = Gv, F = v T_n (e0, e1,
+// e2, eD), nS = -v S_n (WV: -S_n) of the pixels.  With dalpha = v T_n (e.c +
+// eD) - v S_n / (1 - v alpha):  dG = dalpha G', zero where alpha is clamped.
+// CLAMP = false: sigma < alpha_max, so alpha = sigma G' nowhere reaches the
+// clamp; sigma is then applied to the sums instead of to each pixel.
+template <bool CLAMP, bool WV>
+__device__ __forceinline__ void pair_grad2(LaneGrad &a, float2 Gv, float2 F0, float2 F1, float2 F2, float2 FD, float2 nS,
+                                           float dy, float op, float v, float nvop, float4 r2, float alpha_max) {
+    float2 al = Gv, om, raw;
+    if (CLAMP) {
+        raw = __fmul2_rn(make_float2(op, op), Gv);
+        al = make_float2(fminf(raw.x, alpha_max), fminf(raw.y, alpha_max));
+        om = __ffma2_rn(make_float2(-v, -v), al, make_float2(1.0f, 1.0f));
+    } else {
+        om = __ffma2_rn(make_float2(nvop, nvop), Gv, make_float2(1.0f, 1.0f));
+    }
+    const float2 rom = make_float2(rcp_approx(om.x), rcp_approx(om.y));
+    const float2 u = __ffma2_rn(F0, make_float2(r2.x, r2.x),
+                                __ffma2_rn(F1, make_float2(r2.y, r2.y), __ffma2_rn(F2, make_float2(r2.z, r2.z), FD)));
+    float2 dal;
+    if (WV) {
+        const float2 w = __fmul2_rn(nS, rom);
+        a.dv = __ffma2_rn(w, al, a.dv);
+        dal = __ffma2_rn(make_float2(v, v), w, u);
+    } else {
+        dal = __ffma2_rn(nS, rom, u);
+    }
+    a.C0 = __ffma2_rn(F0, al, a.C0);
+    a.C1 = __ffma2_rn(F1, al, a.C1);
+    a.C2 = __ffma2_rn(F2, al, a.C2);
+    float2 dG = __fmul2_rn(dal, Gv);
+    if (CLAMP) {
+        dG.x = raw.x < alpha_max ? dG.x : 0.f;
+        dG.y = raw.y < alpha_max ? dG.y : 0.f;
+    }
+    const float dy2 = dy * dy;
+    a.dop = __fadd2_rn(a.dop, dG);
+    a.Y = __ffma2_rn(dG, make_float2(dy, dy), a.Y);
+    a.Q = __ffma2_rn(dG, make_float2(dy2, dy2), a.Q);
 }
 
 // The mean's terms of a lane, from its moments m = sum dq' (dx, dy): with the
@@ -599,7 +593,7 @@ __device__ __forceinline__ void mean_terms(float4 r1, float &a0, float &a1) {
     a1 = b1;
 }
 
-// Constant factor of reduction slot j (see pair_grad2): dL/dq = -dq'/2, so
+// Constant factor of reduction slot j: dL/dq = -dq'/2, so
 // dmu = -(4 ln 2)(-1/2) acc = 2 ln 2 acc, da = -acc/2, db = -acc (the 2 dx dy
 // term), dc = -acc/2; rgb unchanged.
 __device__ __forceinline__ float slot_scale(int j) {
@@ -610,34 +604,64 @@ __device__ __forceinline__ float slot_scale(int j) {
 __device__ __forceinline__ int grad_slot(int j) { return j < 5 ? j : j + 1; }
 
 // The adjoint's work unit: one warp per 16 x (2 PPL) sub-tile, pixels of a
-// lane as in the forward (lane_col, lane_row).  Per cell: pass 1 replays the forward (keeping G' of the Gaussians
-// that reach the sub-tile in warp-private shared memory) and updates T and
-// S; pass 2 forms each such Gaussian's screen-space gradient over the
-// sub-tile's pixels and adds the warp total with global atomics.
+// lane as in the forward (lane_col, lane_row).  Per cell:
+//   pass 1, pixel-major (a lane owns four pixels): replays the forward, keeping
+//     G' of the Gaussians that reach the sub-tile in warp-private shared memory
+//     (one row of 128 pixels each), and updates T and S; then the lanes leave
+//     their pixels' factors v T_n e and -v S_n there too;
+//   pass 2, Gaussian-major: four Gaussians at a time, eight lanes each; a lane
+//     takes columns w and w + 8 of all eight rows (16 pixels) of its Gaussian
+//     and sums its terms in registers, so one reduction over eight lanes (7 + 3
+//     shuffles) serves four Gaussians and 32 totals leave in one atomic add per
+//     lane.  Of the last one or two Gaussians of a cell each gets 32 or 16 lanes.
+// Bound by instruction issue and the shared-memory data path together (189
+// warp instructions and 58 wavefronts per (sub-tile, Gaussian), 66% and 75% of
+// their peaks before the split of the last round).  A pixel-major pass 2 needs
+// a 32-lane reduction of nine values per Gaussian (229 instructions): 6.33 ms
+// on the 1M-Gaussian 8-view step against 5.17 ms; always four groups: 5.72 ms
+// there, and 1.50 against 1.27 ms where cells have few hits (neural cells, 1.6
+// per cell and sub-tile); two Gaussians per lane (half the factor loads): 5.62 ms,
+// its registers leave 16 warps an SM.
 constexpr int BWD_PPL = 4;
-constexpr int BWD_SUB = kTile / (2 * BWD_PPL);  // sub-tiles per tile
-constexpr int BWD_MINB = 24;  // resident one-warp CTAs per SM the register budget is set for
+constexpr int BWD_ROWS = 2 * BWD_PPL;
+constexpr int BWD_SUB = kTile / BWD_ROWS;  // sub-tiles per tile
+// Resident one-warp CTAs per SM the register budget is set for: 22 are what the
+// shared memory of K = 10 admits (80 registers; 20 at 96 registers is 4% slower
+// on the 1M-Gaussian step).  With dL/dv_n's sums 80 registers spill: 20 there
+// (0.43 against 0.47 ms on 20,011 cells x 5, three 641 x 479 views).
+constexpr int bwd_minb(bool wv) { return wv ? 20 : 22; }
 
-template <int KT, int PPL, bool VAR, bool WV>
-__global__ void __launch_bounds__(WT, BWD_MINB) k_blend_bwd(const ViewDesc *__restrict__ views, int n_views,
+// float4s of shared memory: records [NSTAGE][3 K], G' rows [K][32] (a lane's
+// pixels q = 0..3), v T_n (e0, e1) and v T_n (e2, eD) [2][32] each, -v S_n
+// [32], and the Gaussian of every row (K ints)
+__host__ __device__ constexpr int bwd_smem_f4(int K) {
+    return NSTAGE * kRecF4 * K + WT * K + 4 * WT + WT + (K + 3) / 4;
+}
+
+template <int KT, bool VAR, bool WV>
+__global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *__restrict__ views, int n_views,
                                                   const uint2 *__restrict__ ranges, const uint32_t *__restrict__ cells,
                                                   const float4 *__restrict__ rec, BlendParams bp,
                                                   const float *__restrict__ rgb, const float *__restrict__ Dpix,
                                                   const int *__restrict__ ndpix, const float *__restrict__ dL_drgb,
                                                   float *__restrict__ g2d, float *__restrict__ g_cell_v) {
-    constexpr int ROWS = 2 * PPL, NSUB = kTile / ROWS;
-    constexpr int KRS = KT > 0 ? KT : kMaxK;
-    __shared__ float4 s_rec[NSTAGE][kRecF4 * KRS];
-    static_assert(PPL == 4, "G' of a lane's four pixels is kept as one float4");
-    __shared__ float4 s_G[KRS][WT];  // G' of hit i at the lane's pixels q = 0..3
+    extern __shared__ float4 s_bwd[];
     const int lane = threadIdx.x;
-    const int tile = blockIdx.x / NSUB, sub = blockIdx.x % NSUB;
+    const int tile = blockIdx.x / BWD_SUB, sub = blockIdx.x % BWD_SUB;
     const int vi = find_view(views, n_views, tile);
     const ViewDesc &V = views[vi];
+    const int K = KT > 0 ? KT : V.K;
+    const int per = kRecF4 * K;
+    float4 *const s_rec = s_bwd;                    // [NSTAGE][per]
+    float4 *const s_G = s_rec + NSTAGE * per;       // [K][WT]
+    float4 *const s_F01 = s_G + WT * K;             // [2][WT]
+    float4 *const s_F2D = s_F01 + 2 * WT;           // [2][WT]
+    float4 *const s_nS = s_F2D + 2 * WT;            // [WT]
+    int *const s_k = reinterpret_cast<int *>(s_nS + WT);  // [K]
     const int local = tile - V.tile_base;
     const int tx = local % V.Tx, ty = local / V.Tx;
-    const float bx0 = (float)(tx * kTile), by0 = (float)(ty * kTile + ROWS * sub);
-    constexpr int NR = PPL / 2;  // rows per lane (pixel mapping as in the forward)
+    const float bx0 = (float)(tx * kTile), by0 = (float)(ty * kTile + BWD_ROWS * sub);
+    constexpr int PPL = BWD_PPL, NR = PPL / 2;  // rows per lane (pixel mapping as in the forward)
     int xs[2], ys[NR];
     float pxs[2], pys[NR];
 #pragma unroll
@@ -647,12 +671,10 @@ __global__ void __launch_bounds__(WT, BWD_MINB) k_blend_bwd(const ViewDesc *__re
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-        ys[r] = ty * kTile + ROWS * sub + lane_row(lane, r);
+        ys[r] = ty * kTile + BWD_ROWS * sub + lane_row(lane, r);
         pys[r] = (float)ys[r] + 0.5f;
     }
     const long long HW = (long long)V.W * V.H;
-    const int K = KT > 0 ? KT : V.K;
-    const int per = kRecF4 * K;
 
     // Per pixel: dL/dN = e, dL/dD = eD, and S's start value, the sum of x_n
     // over the processed cells: 0 for C = N / D (degree-0 homogeneity), else
@@ -688,228 +710,245 @@ __global__ void __launch_bounds__(WT, BWD_MINB) k_blend_bwd(const ViewDesc *__re
         }
         ndm = max(ndm, nd[q]);
     }
-    // the lane's pixels as row pairs (columns 0 and 1 of lane row rr); half of
-    // the per-pixel factors, (e2, eD), wait in warp-private shared memory
-    // (registers are the adjoint's limit: this keeps it from spilling)
-    __shared__ float4 s_E[NR][WT];
-    float2 e0r[NR], e1r[NR];
-    const float2 px2 = make_float2(pxs[0], pxs[1]);
+    // the lane's pixels as row pairs (columns 0 and 1 of lane row rr)
+    float2 e0[NR], e1[NR], e2[NR], eD[NR], T[NR], S[NR];
 #pragma unroll
     for (int rr = 0; rr < NR; ++rr) {
-        e0r[rr] = make_float2(e0s[2 * rr], e0s[2 * rr + 1]);
-        e1r[rr] = make_float2(e1s[2 * rr], e1s[2 * rr + 1]);
-        s_E[rr][lane] = make_float4(e2s[2 * rr], e2s[2 * rr + 1], eDs[2 * rr], eDs[2 * rr + 1]);
+        e0[rr] = make_float2(e0s[2 * rr], e0s[2 * rr + 1]);
+        e1[rr] = make_float2(e1s[2 * rr], e1s[2 * rr + 1]);
+        e2[rr] = make_float2(e2s[2 * rr], e2s[2 * rr + 1]);
+        eD[rr] = make_float2(eDs[2 * rr], eDs[2 * rr + 1]);
+        T[rr] = make_float2(nd[2 * rr] > 0 ? 1.0f : 0.f, nd[2 * rr + 1] > 0 ? 1.0f : 0.f);
+        S[rr] = make_float2(S0[2 * rr], S0[2 * rr + 1]);
     }
-    auto efac = [&](int rr, float2 &e0, float2 &e1, float2 &e2, float2 &eD) {
-        const float4 b = s_E[rr][lane];
-        e0 = e0r[rr]; e1 = e1r[rr];
-        e2 = make_float2(b.x, b.y); eD = make_float2(b.z, b.w);
-    };
-    __shared__ int4 s_nd[WT];  // the lane's per-pixel cell counts, read once per cell
-    s_nd[lane] = make_int4(nd[0], nd[1], nd[2], nd[3]);
     const int ndmax = __reduce_max_sync(0xffffffffu, ndm);
     const uint2 rg = ranges[tile];
     const uint32_t end = rg.x + min((uint32_t)ndmax, rg.y - rg.x);
     const float4 *vrec = rec + V.rec_base * kRecF4;
-    constexpr bool want_v = WV;  // dL/dv_n requested (g_cell_v): else its per-pixel sums are not formed
 
-    float2 T[NR], S[NR];
-#pragma unroll
-    for (int rr = 0; rr < NR; ++rr) { T[rr] = make_float2(1.0f, 1.0f); S[rr] = make_float2(S0[2 * rr], S0[2 * rr + 1]); }
+    // pass 2's lane: group (Gaussian of four) and columns; the reduction slot it ends up with
+    const int grp = lane >> 3, w8 = lane & 7;
+    const float2 px2 = make_float2(bx0 + (float)w8 + 0.5f, bx0 + (float)w8 + 8.5f);
+    const int slot = group_owner8(lane);
+
     CellFeed feed{cells, rg.x, end, 0u};
 #pragma unroll
     for (int b = 0; b < NSTAGE - 1; ++b) {
-        if (rg.x + b < end) issue_cell(s_rec[b], vrec, feed.id(rg.x + b, lane), per, lane);
+        if (rg.x + b < end) issue_cell<KT>(s_rec + b * per, vrec, feed.id(rg.x + b, lane), per, lane);
         cp_async_commit();
     }
     int buf = 0;
     for (uint32_t e = rg.x; e < end; ++e) {
         const int fill = buf == 0 ? NSTAGE - 1 : buf - 1;  // the buffer of entry e - 1, read by now
-        if (e + NSTAGE - 1 < end) issue_cell(s_rec[fill], vrec, feed.id(e + NSTAGE - 1, lane), per, lane);
+        if (e + NSTAGE - 1 < end) issue_cell<KT>(s_rec + fill * per, vrec, feed.id(e + NSTAGE - 1, lane), per, lane);
         cp_async_commit();
         cp_async_wait<NSTAGE - 1>();
         __syncwarp();
         const int n = (int)(e - rg.x);
-        bool act[PPL];
-        {
-            const int4 nd4 = s_nd[lane];
-            act[0] = n < nd4.x; act[1] = n < nd4.y; act[2] = n < nd4.z; act[3] = n < nd4.w;
-        }
-        const float4 *r = s_rec[buf];
+        const float4 *r = s_rec + buf * per;
+        buf = buf == NSTAGE - 1 ? 0 : buf + 1;
         const float v = r[2].w;
-        unsigned mask = __ballot_sync(0xffffffffu, lane < K && touches_rows(r[kRecF4 * lane], bx0, by0, (float)ROWS));
-        const unsigned mask0 = mask;
-        const int nhit = __popc(mask);
+        // the Gaussians that reach the sub-tile: row i of G' belongs to the i-th
+        const unsigned hits = __ballot_sync(0xffffffffu, lane < K && touches_rows(r[kRecF4 * lane], bx0, by0, (float)BWD_ROWS));
+        const int rows = __popc(hits);
+        if ((hits >> lane) & 1u) s_k[__popc(hits & ((1u << lane) - 1u))] = lane;
+        // With v <= 1 every 1 - v alpha is at least 1 - alpha_max, and the zero
+        // factors of a finished pixel (T = S = 0) alone keep it out of pass 2;
+        // otherwise the reciprocal may be infinite and its G' is zeroed too.
+        const bool mask_G = !VAR && !(v <= 1.0f);
+        if (rows == 0) {  // (uniform) X = 0, P = 1: only a finished pixel changes
+#pragma unroll
+            for (int rr = 0; rr < NR; ++rr) {
+                T[rr].x = n + 1 < nd[2 * rr] ? T[rr].x : 0.f;
+                T[rr].y = n + 1 < nd[2 * rr + 1] ? T[rr].y : 0.f;
+            }
+            __syncwarp();  // every lane is done with the records before they are refilled
+            continue;
+        }
         // pass 1: replay the cell, keep G'; per pixel P_n and
         // X_n = dN.A_n + dD B_n = sum_k alpha_k (dN.c_k + dD)
         float2 X[NR], P[NR];
         const float2 v2 = make_float2(v, v);
         const float amin = VAR && (bp.flags & DGS_FLAG_ALPHA_SKIP) ? 1.0f / 255.0f : 0.0f;
-        {
 #pragma unroll
-            for (int rr = 0; rr < NR; ++rr) { X[rr] = make_float2(0.f, 0.f); P[rr] = make_float2(1.0f, 1.0f); }
+        for (int rr = 0; rr < NR; ++rr) { X[rr] = make_float2(0.f, 0.f); P[rr] = make_float2(1.0f, 1.0f); }
+        float4 *row = s_G + lane;
 #pragma unroll 1
-            for (int i = 0; i < nhit; ++i) {
-                const int k = __ffs(mask) - 1;
-                mask &= mask - 1;
-                const float4 r0 = r[3 * k];
-                float dx[2], dy[NR];
-                bool hx[2], hy[NR];
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    dx[c] = pxs[c] - r0.x;
-                    hx[c] = fabsf(dx[c]) <= r0.z;
-                }
-#pragma unroll
-                for (int rr = 0; rr < NR; ++rr) {
-                    dy[rr] = pys[rr] - r0.y;
-                    hy[rr] = fabsf(dy[rr]) <= r0.w;
-                }
-                bool h[PPL], any = false;
-                if (VAR) {
-#pragma unroll
-                    for (int q = 0; q < PPL; ++q) {
-                        h[q] = act[q] && hx[q & 1] && hy[q >> 1];
-                        any = any || h[q];
-                    }
-                } else {
-                    // outside the box along a column or a row: an offset far off the
-                    // Gaussian (G' = +0 exactly, as in the forward); inactive pixels
-                    // get G' = 0 when it is stored (their X and P are not used)
-                    any = (hx[0] || hx[1]) && (hy[0] || hy[NR - 1]);
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) dx[c] = hx[c] ? dx[c] : kFar;
-#pragma unroll
-                    for (int rr = 0; rr < NR; ++rr) dy[rr] = hy[rr] ? dy[rr] : kFar;
-                }
-                if (!any) {
-                    s_G[i][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    continue;
-                }
-                const float4 r1 = r[3 * k + 1];
-                const float4 r2 = r[3 * k + 2];
-                const float2 pdx = __fmul2_rn(make_float2(r1.x, r1.x), make_float2(dx[0], dx[1]));
-                float2 gq[NR];
-#pragma unroll
-                for (int rr = 0; rr < NR; ++rr) {
-                    const float dyq = dy[rr];
-                    const float s2 = r1.z * dyq, s22 = s2 * s2;
-                    const float2 s1 = __ffma2_rn(make_float2(r1.y, r1.y), make_float2(dyq, dyq), pdx);
-                    const float2 qd = __ffma2_rn(s1, s1, make_float2(s22, s22));
-                    float2 Gv = make_float2(ex2_approx(-qd.x), ex2_approx(-qd.y));
-                    float2 rw = __fmul2_rn(make_float2(r1.w, r1.w), Gv);
-                    if (VAR) {  // not reached (or alpha skipped as in the forward): G' = 0 leaves X and P as they are
-                        if (!h[2 * rr] || rw.x < amin) Gv.x = rw.x = 0.f;
-                        if (!h[2 * rr + 1] || rw.y < amin) Gv.y = rw.y = 0.f;
-                        gq[rr] = Gv;
-                    } else {
-                        gq[rr] = make_float2(act[2 * rr] ? Gv.x : 0.f, act[2 * rr + 1] ? Gv.y : 0.f);
-                    }
-                    const float2 al = make_float2(fminf(rw.x, bp.alpha_max), fminf(rw.y, bp.alpha_max));
-                    float2 e0, e1, e2, eD;
-                    efac(rr, e0, e1, e2, eD);
-                    const float2 inner = __ffma2_rn(
-                        e0, make_float2(r2.x, r2.x),
-                        __ffma2_rn(e1, make_float2(r2.y, r2.y), __ffma2_rn(e2, make_float2(r2.z, r2.z), eD)));
-                    X[rr] = __ffma2_rn(al, inner, X[rr]);
-                    P[rr] = __ffma2_rn(make_float2(-P[rr].x, -P[rr].y), __fmul2_rn(v2, al), P[rr]);
-                }
-                s_G[i][lane] = make_float4(gq[0].x, gq[0].y, gq[1].x, gq[1].y);
-            }
-        }
-        // per-pixel transmittance bookkeeping (S_n includes x_n); the cell
-        // term of dL/dv, sum over pixels of T_n X_n, joins the Gaussians'
-        // terms below so one reduction per cell carries dL/dv
-        float2 Tn[NR];
-        float dv = 0.f;
-#pragma unroll
-        for (int rr = 0; rr < NR; ++rr) {
-            Tn[rr] = T[rr];
-            if (act[2 * rr]) {
-                S[rr].x -= v * Tn[rr].x * X[rr].x;
-                T[rr].x *= P[rr].x;
-                dv += Tn[rr].x * X[rr].x;
-            }
-            if (act[2 * rr + 1]) {
-                S[rr].y -= v * Tn[rr].y * X[rr].y;
-                T[rr].y *= P[rr].y;
-                dv += Tn[rr].y * X[rr].y;
-            }
-        }
-        // per pixel: sum alpha / (1 - v alpha) of the cell's Gaussians; v T_n; -v S_n
-        float2 pv[NR], cA[NR], nvS[NR];
-#pragma unroll
-        for (int rr = 0; rr < NR; ++rr) {
-            pv[rr] = make_float2(0.f, 0.f);
-            cA[rr] = __fmul2_rn(v2, Tn[rr]);
-            nvS[rr] = __fmul2_rn(make_float2(-v, -v), S[rr]);
-        }
-        const uint32_t cellid = __ldg(cells + e);
-        float *gbase = g2d + (V.rec_base + (long long)cellid * K) * kGradF;
-        // pass 2: gradient terms per Gaussian reaching the sub-tile, two
-        // Gaussians per loop trip (fully unrolled over K the body overflows the
-        // instruction cache; by two it is 2% faster than not unrolled)
-        unsigned m2 = mask0;
-#pragma unroll 2
-        for (int i = 0; m2; ++i, m2 &= m2 - 1) {
-            const float4 g4 = s_G[i][lane];
-            const float2 gv[NR] = {make_float2(g4.x, g4.y), make_float2(g4.z, g4.w)};
-            const bool any = g4.x > 0.f || g4.y > 0.f || g4.z > 0.f || g4.w > 0.f;
-            if (!__any_sync(0xffffffffu, any)) continue;
-            const int k = __ffs(m2) - 1;
+        for (unsigned mask = hits; mask; mask &= mask - 1, row += WT) {
+            const int k = __ffs(mask) - 1;
             const float4 r0 = r[3 * k], r1 = r[3 * k + 1], r2 = r[3 * k + 2];
-            float2 acc2[8];
+            float dx[2], dy[NR];
+            bool hx[2], hy[NR];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc2[j] = make_float2(0.f, 0.f);
-            float2 dop2 = make_float2(0.f, 0.f);
-            const float2 gdx = __fadd2_rn(px2, make_float2(-r0.x, -r0.x));
+            for (int c = 0; c < 2; ++c) {
+                dx[c] = pxs[c] - r0.x;
+                hx[c] = fabsf(dx[c]) <= r0.z;
+                // outside the box along a column or a row: an offset far off the
+                // Gaussian (G' = +0 exactly, as in the forward)
+                if (!VAR) dx[c] = hx[c] ? dx[c] : kFar;
+            }
 #pragma unroll
             for (int rr = 0; rr < NR; ++rr) {
-                float2 e0, e1, e2, eD;
-                efac(rr, e0, e1, e2, eD);
-                pair_grad2<WV>(acc2, dop2, pv[rr], gv[rr], r0, r1, r2, gdx, pys[rr], cA[rr], nvS[rr], e0, e1, e2, eD,
-                               bp.alpha_max);
+                dy[rr] = pys[rr] - r0.y;
+                hy[rr] = fabsf(dy[rr]) <= r0.w;
+                if (!VAR) dy[rr] = hy[rr] ? dy[rr] : kFar;
             }
-            float acc[8];
-            column_terms(acc2, dop2, r1.w, gdx, acc);
+            const float2 pdx = __fmul2_rn(make_float2(r1.x, r1.x), make_float2(dx[0], dx[1]));
+            float2 gq[NR];
 #pragma unroll
-            for (int j = 5; j < 8; ++j) acc[j] = acc2[j].x + acc2[j].y;
-            mean_terms(r1, acc[0], acc[1]);
-            const float tot = transposed_warp_sum8(acc, lane);
-            const float dop_tot = warp_sum(dop2.x + dop2.y);
-            float *gk = gbase + k * kGradF;
-            const int slot = transposed_owner8(lane);
-            if ((lane & 3) == 0 && tot != 0.f) atomicAdd(gk + grad_slot(slot), tot * slot_scale(slot));
-            if (lane == 1 && dop_tot != 0.f) atomicAdd(gk + 5, dop_tot);
+            for (int rr = 0; rr < NR; ++rr) {
+                const float dyq = dy[rr];
+                const float s2 = r1.z * dyq, s22 = s2 * s2;
+                const float2 s1 = __ffma2_rn(make_float2(r1.y, r1.y), make_float2(dyq, dyq), pdx);
+                const float2 qd = __ffma2_rn(s1, s1, make_float2(s22, s22));
+                float2 Gv = make_float2(ex2_approx(-qd.x), ex2_approx(-qd.y));
+                float2 rw = __fmul2_rn(make_float2(r1.w, r1.w), Gv);
+                if (VAR) {  // not reached (or alpha skipped as in the forward): G' = 0 leaves X and P as they are
+                    if (!(n < nd[2 * rr] && hx[0] && hy[rr]) || rw.x < amin) Gv.x = rw.x = 0.f;
+                    if (!(n < nd[2 * rr + 1] && hx[1] && hy[rr]) || rw.y < amin) Gv.y = rw.y = 0.f;
+                }
+                gq[rr] = Gv;
+                const float2 al = make_float2(fminf(rw.x, bp.alpha_max), fminf(rw.y, bp.alpha_max));
+                const float2 inner = __ffma2_rn(
+                    e0[rr], make_float2(r2.x, r2.x),
+                    __ffma2_rn(e1[rr], make_float2(r2.y, r2.y), __ffma2_rn(e2[rr], make_float2(r2.z, r2.z), eD[rr])));
+                X[rr] = __ffma2_rn(al, inner, X[rr]);
+                P[rr] = __ffma2_rn(make_float2(-P[rr].x, -P[rr].y), __fmul2_rn(v2, al), P[rr]);
+            }
+            if (mask_G) {
+#pragma unroll
+                for (int rr = 0; rr < NR; ++rr) {
+                    gq[rr].x = n < nd[2 * rr] ? gq[rr].x : 0.f;
+                    gq[rr].y = n < nd[2 * rr + 1] ? gq[rr].y : 0.f;
+                }
+            }
+            *row = make_float4(gq[0].x, gq[0].y, gq[1].x, gq[1].y);
         }
-        if (want_v) {  // per (view, cell) entry: v_n may differ between views
-            float2 dv2 = make_float2(0.f, 0.f);
+        // per-pixel transmittance bookkeeping (S_n includes x_n; a pixel past its
+        // last cell has T = S = 0), and the factors of pass 2.  The cell term of
+        // dL/dv, sum over pixels of T_n X_n, joins the Gaussians' terms below so
+        // one reduction per cell carries dL/dv.
+        float2 dv2 = make_float2(0.f, 0.f), nS[NR];
 #pragma unroll
-            for (int rr = 0; rr < NR; ++rr) dv2 = __ffma2_rn(make_float2(-S[rr].x, -S[rr].y), pv[rr], dv2);
-            dv = warp_sum(dv + (dv2.x + dv2.y));
+        for (int rr = 0; rr < NR; ++rr) {
+            const float2 cA = __fmul2_rn(v2, T[rr]);
+            const float2 F0 = __fmul2_rn(cA, e0[rr]), F1 = __fmul2_rn(cA, e1[rr]);
+            const float2 F2 = __fmul2_rn(cA, e2[rr]), FD = __fmul2_rn(cA, eD[rr]);
+            s_F01[rr * WT + lane] = make_float4(F0.x, F0.y, F1.x, F1.y);
+            s_F2D[rr * WT + lane] = make_float4(F2.x, F2.y, FD.x, FD.y);
+            if (WV) {
+                const float2 TX = __fmul2_rn(T[rr], X[rr]);
+                dv2.x += n < nd[2 * rr] ? TX.x : 0.f;
+                dv2.y += n < nd[2 * rr + 1] ? TX.y : 0.f;
+            }
+            const float2 Sn = __ffma2_rn(make_float2(-cA.x, -cA.y), X[rr], S[rr]), Tn = __fmul2_rn(T[rr], P[rr]);
+            S[rr].x = n < nd[2 * rr] ? Sn.x : 0.f;
+            S[rr].y = n < nd[2 * rr + 1] ? Sn.y : 0.f;
+            T[rr].x = n + 1 < nd[2 * rr] ? Tn.x : 0.f;
+            T[rr].y = n + 1 < nd[2 * rr + 1] ? Tn.y : 0.f;
+            nS[rr] = WV ? make_float2(-S[rr].x, -S[rr].y) : __fmul2_rn(make_float2(-v, -v), S[rr]);
+        }
+        float dv = dv2.x + dv2.y;
+        s_nS[lane] = make_float4(nS[0].x, nS[0].y, nS[1].x, nS[1].y);
+        __syncwarp();
+        const uint32_t cellid = __ldg(cells + e);
+        float *gbase = g2d + (V.rec_base + (long long)cellid * K) * kGradF;
+        // pass 2: the gradient terms of the rows [c, c + 4 / SPLIT); SPLIT groups of
+        // eight lanes share a Gaussian, each taking 8 / SPLIT of the sub-tile's rows
+        auto round = [&](auto split, int c) {
+            constexpr int SPLIT = decltype(split)::value;
+            const int g = grp / SPLIT, part = grp % SPLIT;
+            // (three rows left: the fourth group repeats the round's first and drops its sums)
+            const bool live = SPLIT > 1 || c + g < rows;
+            const int i = live ? c + g : c;
+            const int k = s_k[i];
+            const float4 *Gr = s_G + i * WT + w8;
+            const float4 r0 = r[3 * k], r1 = r[3 * k + 1], r2 = r[3 * k + 2];
+            const float op = r1.w;
+            const float py0 = by0 + 0.5f + (float)part;
+            LaneGrad a;
+            a.dop = a.Y = a.Q = a.C0 = a.C1 = a.C2 = a.dv = make_float2(0.f, 0.f);
+            auto sweep = [&](auto clamp) {
+#pragma unroll
+                for (int t = 0; t < 4 / SPLIT; ++t) {  // rows j and j + 4
+                    const int at = 8 * (SPLIT * t + part) + w8;
+                    const float4 g4 = Gr[at - w8], n4 = s_nS[at];
+#pragma unroll
+                    for (int rr = 0; rr < NR; ++rr) {
+                        const float4 fa = s_F01[rr * WT + at], fb = s_F2D[rr * WT + at];
+                        pair_grad2<decltype(clamp)::value, WV>(
+                            a, rr == 0 ? make_float2(g4.x, g4.y) : make_float2(g4.z, g4.w), make_float2(fa.x, fa.y),
+                            make_float2(fa.z, fa.w), make_float2(fb.x, fb.y), make_float2(fb.z, fb.w),
+                            rr == 0 ? make_float2(n4.x, n4.y) : make_float2(n4.z, n4.w),
+                            (py0 + (float)(SPLIT * t + 4 * rr)) - r0.y, op, v, -v * op, r2, bp.alpha_max);
+                    }
+                }
+            };
+            // (not op < alpha_max: a NaN opacity takes the clamp, as in the forward)
+            const bool clamp = __any_sync(0xffffffffu, !(op < bp.alpha_max));
+            if (clamp) sweep(std::true_type{}); else sweep(std::false_type{});
+            const float cs = clamp ? 1.0f : op;
+            const float2 dx = __fadd2_rn(px2, make_float2(-r0.x, -r0.x));
+            // the lane's totals of slots 0..4 from its per-column sums: with D =
+            // sigma dop = sum dq' and Y = sigma Y per column, sum dq' dx = D.dx,
+            // sum dq' dx^2 = D.dx^2, sum dq' dx dy = Y.dx
+            float acc[8];
+            const float2 D = __fmul2_rn(a.dop, make_float2(op, op)), t = __fmul2_rn(D, dx);
+            const float2 Y = __fmul2_rn(a.Y, make_float2(op, op));
+            acc[0] = t.x + t.y;
+            acc[1] = Y.x + Y.y;
+            acc[2] = fmaf(t.x, dx.x, t.y * dx.y);
+            acc[3] = fmaf(Y.x, dx.x, Y.y * dx.y);
+            acc[4] = (a.Q.x + a.Q.y) * op;
+            acc[5] = (a.C0.x + a.C0.y) * cs;
+            acc[6] = (a.C1.x + a.C1.y) * cs;
+            acc[7] = (a.C2.x + a.C2.y) * cs;
+            mean_terms(r1, acc[0], acc[1]);
+            if (WV) dv += live ? (a.dv.x + a.dv.y) * cs : 0.f;
+            float tot = group_sum8(acc, lane), dop = a.dop.x + a.dop.y;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) dop += __shfl_xor_sync(0xffffffffu, dop, o);
+#pragma unroll
+            for (int o = 8; o < 8 * SPLIT; o <<= 1) {
+                tot += __shfl_xor_sync(0xffffffffu, tot, o);
+                dop += __shfl_xor_sync(0xffffffffu, dop, o);
+            }
+            float *gk = gbase + k * kGradF;
+            if (live && part == 0) {
+                if (tot != 0.f) atomicAdd(gk + grad_slot(slot), tot * slot_scale(slot));
+                if (w8 == 0 && dop != 0.f) atomicAdd(gk + 5, dop);
+            }
+        };
+        int c = 0;
+#pragma unroll 1
+        for (; rows - c > 2; c += 4) round(std::integral_constant<int, 1>{}, c);
+        if (rows - c == 2) round(std::integral_constant<int, 2>{}, c);
+        if (rows - c == 1) round(std::integral_constant<int, 4>{}, c);
+        if (WV) {  // per (view, cell) entry: v_n may differ between views
+            dv = warp_sum(dv);
             if (lane == 0 && dv != 0.f) atomicAdd(g_cell_v + V.cell_base + cellid, dv);
         }
-        __syncwarp();  // every lane is done with s_rec[buf] and s_G before they are refilled
-        buf = buf == NSTAGE - 1 ? 0 : buf + 1;
+        __syncwarp();  // every lane is done with the records and rows before they are refilled
     }
     cp_async_wait<0>();
 }
 
-// K_all: K of the chain's scene (compile-time loop for common values)
+// K_all: K of the chain's scene (compile-time loop for common values; sizes the shared memory)
 void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, int K_all, const uint2 *ranges,
                       const uint32_t *tile_cells, const float4 *rec, const BlendParams &bp, const float *rgb,
                       const float *D, const int *nd, const float *dL_drgb, float *g2d, float *g_cell_v,
                       cudaStream_t st) {
     if (total_tiles == 0) return;
     const unsigned grid = (unsigned)total_tiles * BWD_SUB;
+    const size_t smem = sizeof(float4) * bwd_smem_f4(K_all);
 #define DGS_BWD(KV, VV)                                                                                          \
     do {                                                                                                        \
         if (g_cell_v)                                                                                           \
-            k_blend_bwd<KV, BWD_PPL, VV, true><<<grid, WT, 0, st>>>(views, n_views, ranges, tile_cells, rec, bp,  \
-                                                                    rgb, D, nd, dL_drgb, g2d, g_cell_v);        \
+            k_blend_bwd<KV, VV, true><<<grid, WT, smem, st>>>(views, n_views, ranges, tile_cells, rec, bp, rgb, D, nd, \
+                                                              dL_drgb, g2d, g_cell_v);                          \
         else                                                                                                    \
-            k_blend_bwd<KV, BWD_PPL, VV, false><<<grid, WT, 0, st>>>(views, n_views, ranges, tile_cells, rec, bp, \
-                                                                     rgb, D, nd, dL_drgb, g2d, nullptr);        \
+            k_blend_bwd<KV, VV, false><<<grid, WT, smem, st>>>(views, n_views, ranges, tile_cells, rec, bp, rgb, D, nd, \
+                                                               dL_drgb, g2d, nullptr);                          \
     } while (0)
     if (blend_variants(bp)) {
         switch (K_all) {

@@ -166,3 +166,33 @@ def test_gradients_beyond_the_jacobian_clamp(rctx):
     for k_gpu, k_ref in (("g_mean", "mean"), ("g_scale", "scale"), ("g_quat", "quat"), ("g_logit", "logit"),
                          ("g_sh", "sh")):
         assert_close_group(k_ref, gr[k_gpu].cpu(), ref[k_ref])
+
+
+@pytest.mark.parametrize("K", [1, 2, 3, 5, 6, 7, 8, 10, 13, 32])
+@pytest.mark.parametrize("opaque", [False, True])
+def test_gradients_per_cell_row_counts(rctx, K, opaque):
+    """The adjoint's second pass takes a cell's Gaussians four at a time, the
+    last one or two with more lanes each: every remainder, the compiled and the
+    run-time K, with opacities below the alpha clamp and beyond it (their pixels
+    below the clamp keep a gradient), and with dL/dv_n requested and not."""
+    sc = synth.make_scene(24, K, synth._box(-0.5, 0.5), 0.1, 0.4, 1, seed=100 + K)
+    sc.cell_v[:] = np.random.default_rng(K).uniform(0.3, 1.0, sc.N).astype(np.float32)
+    if opaque:
+        sc.g_logit[::2] = 7.0  # sigma = 0.9991
+    cams = synth.sphere_cameras(1, 3.0, 61, 43, seed0=9)
+    _, dl, gr, gs, _ = _grads(rctx, sc, cams, seed=K)
+    ref, _ = _oracle_grads(sc, cams, dl, gs)
+    names = (("g_mean", "mean"), ("g_scale", "scale"), ("g_quat", "quat"), ("g_logit", "logit"), ("g_sh", "sh"))
+    for k_gpu, k_ref in names + (("g_cell_v", "cell_v"),):
+        assert_close_group(k_ref, gr[k_gpu].cpu(), ref[k_ref])
+    # without dL/dv_n: the same terms by the other instantiation; only the FP32
+    # roundings of v S differ (a few ulp of sums of up to 1e3 terms)
+    sid = rctx.upload_scene(sc)
+    flat, state, _ = rctx.render(sid, cams, want_state=True)
+    g = {k: torch.empty_like(gr[k]) for k, _ in names}
+    rctx.backward(state, torch.from_numpy(dl).cuda(), g)
+    torch.cuda.synchronize()
+    for k, _ in names:
+        assert (g[k] - gr[k]).norm() <= 1e-4 * gr[k].norm(), k
+    rctx.release_state(state)
+    rctx.release_scene(sid)
