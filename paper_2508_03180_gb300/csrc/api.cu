@@ -295,7 +295,10 @@ extern "C" void dgs_destroy(dgs_ctx *ctx) {
         for (auto *st : ctx->live_states) delete st;
         ctx->live_states.clear();
         ctx->pool.clear();
-        ctx->scenes.clear();
+        {
+            std::lock_guard<std::mutex> ls(ctx->scene_mu);
+            ctx->scenes.clear();
+        }
         ctx->aux.release();
         ctx->sort_ws.reset();
     }
@@ -606,7 +609,10 @@ extern "C" dgs_status dgs_scene_upload(dgs_ctx *ctx, const dgs_scene_desc *d, ui
     if ((s = fill_scene(ctx, *sc, d, st, true))) return s;
     CK(cudaStreamSynchronize(st));
     const uint32_t id = ctx->next_scene++;
-    ctx->scenes[id] = std::move(sc);
+    {
+        std::lock_guard<std::mutex> ls(ctx->scene_mu);
+        ctx->scenes[id] = std::move(sc);
+    }
     *scene_id = id;
     return DGS_OK;
 }
@@ -636,7 +642,10 @@ extern "C" dgs_status dgs_scene_release(dgs_ctx *ctx, uint32_t scene_id) {
     for (auto *st : ctx->live_states)
         if (st->scene_id == scene_id) return set_error(DGS_ERR_BUSY, "a forward state still refers to this scene");
     CK(cudaDeviceSynchronize());
-    ctx->scenes.erase(it);
+    {
+        std::lock_guard<std::mutex> ls(ctx->scene_mu);
+        ctx->scenes.erase(it);
+    }
     ++ctx->scene_epoch;  // captured serving graphs may hold its pointers
     return DGS_OK;
 }

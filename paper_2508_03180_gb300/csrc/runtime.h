@@ -230,7 +230,11 @@ struct StageTimer {
 struct dgs_ctx {
     dgs_config cfg;
     dgs::Profiler prof;
-    std::mutex mu;  // serialises every ABI call (and the serving worker's launches)
+    std::mutex mu;  // serialises every ABI call but submit, poll and cancel (and the serving worker's launches)
+    // The scene table itself: taken, after mu, by the calls that add or remove a
+    // scene, and alone by dgs_submit, whose look-up of the scene's sizes then does
+    // not wait for a launch of the worker (a scene's sizes never change).
+    std::mutex scene_mu;
     std::map<uint32_t, std::unique_ptr<dgs::Scene>> scenes;
     uint32_t next_scene = 1;
     std::vector<dgs_camera> cams;

@@ -605,7 +605,7 @@ extern "C" dgs_status dgs_submit(dgs_ctx *ctx, const dgs_request *req, uint64_t 
         return set_error(DGS_ERR_INVALID_ARG, "bad camera");
     int64_t bytes;
     {
-        std::lock_guard<std::mutex> lk(ctx->mu);
+        std::lock_guard<std::mutex> lk(ctx->scene_mu);
         auto it = ctx->scenes.find(req->scene_id);
         if (it == ctx->scenes.end()) return set_error(DGS_ERR_NOT_FOUND, "unknown scene id");
         bytes = request_bytes(*it->second, c);
