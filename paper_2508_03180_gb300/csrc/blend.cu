@@ -12,8 +12,8 @@
 //
 // GB300 mapping: one one-warp CTA per 16x8 half of a 16x16 tile, four
 // pixels per lane in packed pairs (f32x2 arithmetic).  The 48-byte records of
-// a cell's Gaussians are copied into the warp's shared memory asynchronously
-// two cells ahead and broadcast from there to the warp's 128 pixels.
+// the cells' Gaussians are copied into the warp's shared memory asynchronously,
+// ahead of their use, and broadcast from there to the warp's 128 pixels.
 #include <algorithm>
 #include <type_traits>
 
@@ -110,18 +110,67 @@ __device__ __forceinline__ bool covers_rows(float4 r0, float x0, float y0, float
 __device__ __forceinline__ int lane_col(int lane, int c) { return (lane & 7) + 8 * c; }
 __device__ __forceinline__ int lane_row(int lane, int r) { return (lane >> 3) + 4 * r; }
 
+// Cells of a tile list in batches: the 32 / K cells (one at least) whose Gaussians a
+// warp's lanes test in one ballot.  Lane l copies the float4s l, l + 32, l + 64
+// of a batch (at most 32 records), whose cell within the batch and place within the
+// cell stay the same for the whole list; the ids of a batch's cells are read one
+// batch before its copies are issued, so no copy waits for its address.
+constexpr int FSTAGE = 2;          // batches in shared memory: one blended, one on its way
+constexpr int kBatchF4 = 32 * kRecF4;
+__host__ __device__ constexpr int batch_cells(int K) { return 32 / K; }
+
+struct CellBatches {
+    const uint32_t *__restrict__ cells;
+    const float4 *__restrict__ vrec;
+    uint32_t end;
+    uint32_t id;            // lane l: cell l of the next batch to copy
+    uint32_t pos;           // byte q: the cell (of the batch) of the lane's q-th piece
+    __device__ __forceinline__ CellBatches(const uint32_t *c, const float4 *v, uint32_t list_end, int K, int lane)
+        : cells(c), vrec(v + lane), end(list_end), id(0u), pos(0u) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) pos |= (uint32_t)((lane + 32 * q) / (kRecF4 * K)) << (8 * q);
+    }
+    // cells of the batch at entry e
+    __device__ __forceinline__ uint32_t count(uint32_t e, int K) const {
+        return e < end ? min(end - e, (uint32_t)batch_cells(K)) : 0u;
+    }
+    __device__ __forceinline__ void read_ids(uint32_t e, int K, int lane) {
+        if (lane < count(e, K)) id = __ldg(cells + e + lane);
+    }
+    // the copies of the batch at entry e (its ids read before)
+    __device__ __forceinline__ void issue(float4 *dst, uint32_t e, int K, int lane) const {
+        const uint32_t n = count(e, K);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const uint32_t j = (pos >> (8 * q)) & 255u, from = __shfl_sync(0xffffffffu, id, j);
+            // piece lane + 32 q of the batch is piece lane + 32 q - j per of its cell
+            if (j < n) cp_async16(dst + lane + 32 * q, vrec + ((long long)from - j) * (kRecF4 * K) + 32 * q);
+        }
+    }
+};
+
 // The forward's work unit: one warp per 16 x (2 PPL) sub-tile.  FWD_PPL = 4
 // (16x8 sub-tiles, the adjoint's): with the pixel math in packed pairs, the
-// per-Gaussian work of a lane (ballot, record loads, AABB tests) spread over
-// four pixels outweighs the register cost; the kernels are held to 64
-// registers (32 one-warp CTAs per SM; 1% faster than 72 registers and 28).
+// per-Gaussian work of a lane (record loads, AABB tests) spread over four
+// pixels outweighs the register cost; the kernels are held to 64 registers
+// (32 one-warp CTAs per SM).
+//
+// Bound by instruction issue.  A (sub-tile, cell) pair has two Gaussians in reach
+// on average, about 90 of the 200 warp instructions that a cell cost when it was
+// copied, tested and added up by itself: a batch's copies, wait and ballots now
+// serve 32 / K cells, and a cell with no Gaussian in reach (P = 1, sums 0) leaves
+// the pixels as they are and costs nothing more.  1M Gaussians, eight 1080p views:
+// 2.16 -> 1.97 ms; two views of neural cells, fewer hits per cell: 0.65 -> 0.52 ms;
+// 2,048 cells x 8 at 256 x 256, one warp a scheduler: 74 -> 46 us.  Weighting every
+// alpha by v_n T_n instead of the cell's sums (no sums to clear and add) takes
+// another 3%, but rounds N and D more often; 72 registers and 28 CTAs an SM: 2.00 ms.
 constexpr int FWD_PPL = 4;
 // an offset from the Gaussian's centre that no box reaches: s1 or s2 then
 // squares to at least ~1e18 (the record's L entries are far above 1e-9), and
 // exp2 of its negation is +0
 constexpr float kFar = 1e18f;
 constexpr int FWD_SUB = kTile / (2 * FWD_PPL);  // sub-tiles per tile
-constexpr int FWD_MINB = 32;
+constexpr int fwd_minb(bool var) { return var ? 24 : 32; }  // (the variants spill at 64 registers)
 
 // VAR: the variant flags and background weight are live (dgs_config.flags,
 // w_bg); without it the kernels are the paper's reading with no check left.
@@ -131,7 +180,7 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
                                                const float4 *__restrict__ rec, const BlendParams &bp,
                                                float *__restrict__ out_rgb, float *__restrict__ out_rgb2,
                                                float *__restrict__ out_D, int *__restrict__ out_nd,
-                                               float4 (*s_rec)[kRecF4 * (KT > 0 ? KT : kMaxK)]) {
+                                               float4 (*s_rec)[kBatchF4]) {
     constexpr int ROWS = 2 * PPL, NSUB = kTile / ROWS;
     const int lane = threadIdx.x;
     const int tile = unit / NSUB, sub = unit % NSUB;
@@ -154,140 +203,132 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
         pys[r] = (float)ys[r] + 0.5f;
     }
     const int K = KT > 0 ? KT : V.K;
-    const int per = kRecF4 * K;
-    const float4 *vrec = rec + V.rec_base * kRecF4;
+    const uint32_t CB = batch_cells(K);
+    const unsigned kmask = K == 32 ? 0xffffffffu : (1u << K) - 1u;
     const uint2 rg = ranges[tile];
 
-    float T[PPL], N0[PPL], N1[PPL], N2[PPL], D[PPL];
-    int n[PPL];
-    bool done[PPL];
+    // A pixel is done once T < eps (eps >= 0): T is then not needed any more and holds,
+    // as a negative number, how many cells were blended (done_after).
+    // A lane's two pixels of a row as packed pairs (one f32x2 operation per pair;
+    // per component the same IEEE operations as one pixel).
+    float T[PPL];
+    float2 N0[NR], N1[NR], N2[NR], D[NR];
+    auto done_after = [](int cells_blended) { return __int_as_float((int)0x80000000 | (cells_blended + 1)); };
 #pragma unroll
-    for (int q = 0; q < PPL; ++q) {
-        T[q] = 1.0f; N0[q] = N1[q] = N2[q] = D[q] = 0.f; n[q] = 0;
-        done[q] = !(xs[q & 1] < V.W && ys[q >> 1] < V.H);
-    }
-    CellFeed feed{cells, rg.x, rg.y, 0u};
+    for (int q = 0; q < PPL; ++q)
+        T[q] = xs[q & 1] < V.W && ys[q >> 1] < V.H && !(1.0f < bp.eps) ? 1.0f : done_after(0);
 #pragma unroll
-    for (int b = 0; b < NSTAGE - 1; ++b) {
-        if (rg.x + b < rg.y) issue_cell<KT>(s_rec[b], vrec, feed.id(rg.x + b, lane), per, lane);
-        cp_async_commit();
-    }
+    for (int rr = 0; rr < NR; ++rr) N0[rr] = N1[rr] = N2[rr] = D[rr] = make_float2(0.f, 0.f);
+    CellBatches feed(cells, rec + V.rec_base * kRecF4, rg.y, K, lane);
+    feed.read_ids(rg.x, K, lane);
+    feed.issue(s_rec[0], rg.x, K, lane);
+    cp_async_commit();
+    feed.read_ids(rg.x + CB, K, lane);
     int buf = 0;
-    for (uint32_t e = rg.x; e < rg.y; ++e) {
+    for (uint32_t e = rg.x; e < rg.y; e += CB, buf ^= 1) {
         // before cell n a pixel stops if T_n < eps (Sec. V-B)
         bool all = true;
 #pragma unroll
-        for (int q = 0; q < PPL; ++q) {
-            done[q] = done[q] || T[q] < bp.eps;
-            all = all && done[q];
-        }
+        for (int q = 0; q < PPL; ++q) all = all && T[q] < bp.eps;
         if (__all_sync(0xffffffffu, all)) break;
-        const int fill = buf == 0 ? NSTAGE - 1 : buf - 1;  // the buffer of entry e - 1, read by now
-        if (e + NSTAGE - 1 < rg.y) issue_cell<KT>(s_rec[fill], vrec, feed.id(e + NSTAGE - 1, lane), per, lane);
+        feed.issue(s_rec[buf ^ 1], e + CB, K, lane);  // (that buffer's batch was read in the last iteration)
         cp_async_commit();
-        cp_async_wait<NSTAGE - 1>();
+        feed.read_ids(e + 2 * CB, K, lane);
+        cp_async_wait<1>();
         __syncwarp();
         const float4 *r = s_rec[buf];
-        const float v = r[2].w;
-        unsigned mask = __ballot_sync(0xffffffffu, lane < K && touches_rows(r[kRecF4 * lane], bx0, by0, (float)ROWS));
+        const bool mine = lane < K * feed.count(e, K);  // lane l: the batch's l-th Gaussian
+        const float4 rl = r[kRecF4 * lane];
+        unsigned hits = __ballot_sync(0xffffffffu, mine && touches_rows(rl, bx0, by0, (float)ROWS));
         // Gaussians whose box holds the whole sub-tile: no per-pixel test
-        const unsigned full = VAR ? 0u : __ballot_sync(0xffffffffu, lane < K && covers_rows(r[kRecF4 * lane], bx0, by0,
-                                                                                            (float)ROWS));
-        // the lane's two pixels of a row as packed pairs (one f32x2 operation
-        // per pair; per component the same IEEE operations as one pixel)
-        float2 A0[NR], A1[NR], A2[NR], B[NR], P[NR];
-#pragma unroll
-        for (int rr = 0; rr < NR; ++rr) {
-            A0[rr] = A1[rr] = A2[rr] = B[rr] = make_float2(0.f, 0.f);
-            P[rr] = make_float2(1.0f, 1.0f);
-        }
-        const float2 v2 = make_float2(v, v);
+        const unsigned full = VAR ? 0u : __ballot_sync(0xffffffffu, mine && covers_rows(rl, bx0, by0, (float)ROWS));
         const float amin = VAR && (bp.flags & DGS_FLAG_ALPHA_SKIP) ? 1.0f / 255.0f : 0.0f;
-        for (; mask; mask &= mask - 1) {
-            const int k = __ffs(mask) - 1;
-            const float4 r0 = r[3 * k];
-            float dx[2], dy[NR];
-#pragma unroll
-            for (int c = 0; c < 2; ++c) dx[c] = pxs[c] - r0.x;
-#pragma unroll
-            for (int rr = 0; rr < NR; ++rr) dy[rr] = pys[rr] - r0.y;
-            bool h[PPL];
-            if (VAR || !((full >> k) & 1u)) {  // (else every pixel of the sub-tile is in the box)
-                bool hx[2], hy[NR], any = false;
-#pragma unroll
-                for (int c = 0; c < 2; ++c) hx[c] = fabsf(dx[c]) <= r0.z;
-#pragma unroll
-                for (int rr = 0; rr < NR; ++rr) hy[rr] = fabsf(dy[rr]) <= r0.w;
-                if (VAR) {
-#pragma unroll
-                    for (int q = 0; q < PPL; ++q) {
-                        h[q] = !done[q] && hx[q & 1] && hy[q >> 1];
-                        any = any || h[q];
-                    }
-                } else {
-                    // outside the box along a column or a row: an offset far off
-                    // the Gaussian, so exp2 gives alpha = +0 exactly (in-box pixels
-                    // compute as before; a done pixel's sums are not used)
-                    bool anyy = hy[0];
-#pragma unroll
-                    for (int rr = 1; rr < NR; ++rr) anyy = anyy || hy[rr];
-                    any = (hx[0] || hx[1]) && anyy;
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) dx[c] = hx[c] ? dx[c] : kFar;
-#pragma unroll
-                    for (int rr = 0; rr < NR; ++rr) dy[rr] = hy[rr] ? dy[rr] : kFar;
-                }
-                // warp-uniform skip: lanes without a hit run the body with alpha = 0
-                if (!__any_sync(0xffffffffu, any)) continue;
-            }
-            const float4 r1 = r[3 * k + 1];
-            const float4 r2 = r[3 * k + 2];
-            const float2 pdx = __fmul2_rn(make_float2(r1.x, r1.x), make_float2(dx[0], dx[1]));
+        while (hits) {
+            // the next cell with a Gaussian in reach: cell c of the batch, its Gaussians' lanes in mask
+            const int c = (__ffs(hits) - 1) / K;
+            unsigned mask = hits & (kmask << (c * K));
+            hits ^= mask;
+            const float v = r[kRecF4 * (c * K) + 2].w;
+            float2 A0[NR], A1[NR], A2[NR], B[NR], P[NR];
 #pragma unroll
             for (int rr = 0; rr < NR; ++rr) {
-                const float dyq = dy[rr];
-                const float s2 = r1.z * dyq, s22 = s2 * s2;
-                const float2 s1 = __ffma2_rn(make_float2(r1.y, r1.y), make_float2(dyq, dyq), pdx);
-                const float2 qd = __ffma2_rn(s1, s1, make_float2(s22, s22));
-                float2 al = __fmul2_rn(make_float2(r1.w, r1.w), make_float2(ex2_approx(-qd.x), ex2_approx(-qd.y)));
-                // a pixel the Gaussian does not reach (or, with the alpha skip, an
-                // alpha below 1/255) takes alpha 0: every update below leaves it unchanged
-                if (VAR) {
-                    al.x = h[2 * rr] && al.x >= amin ? fminf(al.x, bp.alpha_max) : 0.f;
-                    al.y = h[2 * rr + 1] && al.y >= amin ? fminf(al.y, bp.alpha_max) : 0.f;
-                } else {
-                    al.x = fminf(al.x, bp.alpha_max);
-                    al.y = fminf(al.y, bp.alpha_max);
-                }
-                A0[rr] = __ffma2_rn(al, make_float2(r2.x, r2.x), A0[rr]);
-                A1[rr] = __ffma2_rn(al, make_float2(r2.y, r2.y), A1[rr]);
-                A2[rr] = __ffma2_rn(al, make_float2(r2.z, r2.z), A2[rr]);
-                B[rr] = __fadd2_rn(B[rr], al);
-                P[rr] = __ffma2_rn(make_float2(-P[rr].x, -P[rr].y), __fmul2_rn(v2, al), P[rr]);
+                A0[rr] = A1[rr] = A2[rr] = B[rr] = make_float2(0.f, 0.f);
+                P[rr] = make_float2(1.0f, 1.0f);
             }
-        }
-        const bool exclude = VAR && (bp.flags & DGS_FLAG_TERM_EXCLUDE) != 0;
+            const float2 nv2 = make_float2(-v, -v);
+            for (; mask; mask &= mask - 1) {
+                const int k = __ffs(mask) - 1;
+                const float4 r0 = r[3 * k], r1 = r[3 * k + 1], r2 = r[3 * k + 2];
+                float dx[2], dy[NR];
 #pragma unroll
-        for (int q = 0; q < PPL; ++q) {
-            if (!done[q]) {
-                const int rr = q >> 1;
-                const bool hi = q & 1;
-                const float Tnext = T[q] * (hi ? P[rr].y : P[rr].x);
-                if (exclude && Tnext < bp.eps) {  // the 3DGS rule: this cell is not blended
-                    done[q] = true;
-                    continue;
+                for (int c2 = 0; c2 < 2; ++c2) dx[c2] = pxs[c2] - r0.x;
+#pragma unroll
+                for (int rr = 0; rr < NR; ++rr) dy[rr] = pys[rr] - r0.y;
+                bool h[PPL];
+                if (VAR || !((full >> k) & 1u)) {  // (else every pixel of the sub-tile is in the box)
+                    bool hx[2], hy[NR];
+#pragma unroll
+                    for (int c2 = 0; c2 < 2; ++c2) hx[c2] = fabsf(dx[c2]) <= r0.z;
+#pragma unroll
+                    for (int rr = 0; rr < NR; ++rr) hy[rr] = fabsf(dy[rr]) <= r0.w;
+                    if (VAR) {
+#pragma unroll
+                        for (int q = 0; q < PPL; ++q) h[q] = !(T[q] < bp.eps) && hx[q & 1] && hy[q >> 1];
+                    } else {
+                        // outside the box along a column or a row: an offset far off
+                        // the Gaussian, so exp2 gives alpha = +0 exactly (in-box pixels
+                        // compute as before; a done pixel's sums are not used)
+#pragma unroll
+                        for (int c2 = 0; c2 < 2; ++c2) dx[c2] = hx[c2] ? dx[c2] : kFar;
+#pragma unroll
+                        for (int rr = 0; rr < NR; ++rr) dy[rr] = hy[rr] ? dy[rr] : kFar;
+                    }
                 }
-                const float w = v * T[q];
-                N0[q] = fmaf(w, hi ? A0[rr].y : A0[rr].x, N0[q]);
-                N1[q] = fmaf(w, hi ? A1[rr].y : A1[rr].x, N1[q]);
-                N2[q] = fmaf(w, hi ? A2[rr].y : A2[rr].x, N2[q]);
-                D[q] = fmaf(w, hi ? B[rr].y : B[rr].x, D[q]);
-                T[q] = Tnext;
-                ++n[q];
+                const float2 pdx = __fmul2_rn(make_float2(r1.x, r1.x), make_float2(dx[0], dx[1]));
+#pragma unroll
+                for (int rr = 0; rr < NR; ++rr) {
+                    const float dyq = dy[rr];
+                    const float s2 = r1.z * dyq, s22 = s2 * s2;
+                    const float2 s1 = __ffma2_rn(make_float2(r1.y, r1.y), make_float2(dyq, dyq), pdx);
+                    const float2 qd = __ffma2_rn(s1, s1, make_float2(s22, s22));
+                    float2 al = __fmul2_rn(make_float2(r1.w, r1.w), make_float2(ex2_approx(-qd.x), ex2_approx(-qd.y)));
+                    // a pixel the Gaussian does not reach (or, with the alpha skip, an
+                    // alpha below 1/255) takes alpha 0: every update below leaves it unchanged
+                    if (VAR) {
+                        al.x = h[2 * rr] && al.x >= amin ? fminf(al.x, bp.alpha_max) : 0.f;
+                        al.y = h[2 * rr + 1] && al.y >= amin ? fminf(al.y, bp.alpha_max) : 0.f;
+                    } else {
+                        al.x = fminf(al.x, bp.alpha_max);
+                        al.y = fminf(al.y, bp.alpha_max);
+                    }
+                    A0[rr] = __ffma2_rn(al, make_float2(r2.x, r2.x), A0[rr]);
+                    A1[rr] = __ffma2_rn(al, make_float2(r2.y, r2.y), A1[rr]);
+                    A2[rr] = __ffma2_rn(al, make_float2(r2.z, r2.z), A2[rr]);
+                    B[rr] = __fadd2_rn(B[rr], al);
+                    P[rr] = __ffma2_rn(P[rr], __fmul2_rn(nv2, al), P[rr]);
+                }
+            }
+            const float now_done = done_after((int)(e - rg.x) + c + 1);
+            const bool exclude = VAR && (bp.flags & DGS_FLAG_TERM_EXCLUDE) != 0;
+#pragma unroll
+            for (int rr = 0; rr < NR; ++rr) {
+                const float2 Tr = make_float2(T[2 * rr], T[2 * rr + 1]);
+                float2 w = __fmul2_rn(make_float2(v, v), Tr);
+                const float2 Tn = __fmul2_rn(Tr, P[rr]);
+                const bool d0 = Tr.x < bp.eps, d1 = Tr.y < bp.eps;      // done before this cell
+                const bool n0 = Tn.x < bp.eps, n1 = Tn.y < bp.eps;      // (or with it)
+                w.x = d0 || (exclude && n0) ? 0.f : w.x;  // exclude, the 3DGS rule: that cell is not blended
+                w.y = d1 || (exclude && n1) ? 0.f : w.y;
+                N0[rr] = __ffma2_rn(w, A0[rr], N0[rr]);
+                N1[rr] = __ffma2_rn(w, A1[rr], N1[rr]);
+                N2[rr] = __ffma2_rn(w, A2[rr], N2[rr]);
+                D[rr] = __ffma2_rn(w, B[rr], D[rr]);
+                const float end = exclude ? done_after((int)(e - rg.x) + c) : now_done;
+                T[2 * rr] = d0 ? Tr.x : n0 ? end : Tn.x;
+                T[2 * rr + 1] = d1 ? Tr.y : n1 ? end : Tn.y;
             }
         }
         __syncwarp();  // every lane is done with s_rec[buf] before it is refilled
-        buf = buf == NSTAGE - 1 ? 0 : buf + 1;
     }
     cp_async_wait<0>();  // copies of entries past an early stop land before the buffers are reused
     __syncwarp();
@@ -298,20 +339,22 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
     for (int q = 0; q < PPL; ++q) {
         if (!(xs[q & 1] < V.W && ys[q >> 1] < V.H)) continue;
         const long long pin = (long long)ys[q >> 1] * V.W + xs[q & 1];
+        const float m0 = q & 1 ? N0[q >> 1].y : N0[q >> 1].x, m1 = q & 1 ? N1[q >> 1].y : N1[q >> 1].x;
+        const float m2 = q & 1 ? N2[q >> 1].y : N2[q >> 1].x, Dq = q & 1 ? D[q >> 1].y : D[q >> 1].x;
         float c0, c1, c2;
         if (VAR && (bp.flags & DGS_FLAG_NUMERATOR)) {  // the numerator of Eq. 12
-            c0 = N0[q]; c1 = N1[q]; c2 = N2[q];
+            c0 = m0; c1 = m1; c2 = m2;
         } else if (VAR) {  // Eq. 12, with a background weight (N + w_bg bg) / (D + w_bg)
-            const float Dp = D[q] + bp.w_bg;
+            const float Dp = Dq + bp.w_bg;
             const bool hit = Dp > bp.d_min;
-            c0 = hit ? (N0[q] + bp.w_bg * bp.bg0) / Dp : bp.bg0;
-            c1 = hit ? (N1[q] + bp.w_bg * bp.bg1) / Dp : bp.bg1;
-            c2 = hit ? (N2[q] + bp.w_bg * bp.bg2) / Dp : bp.bg2;
+            c0 = hit ? (m0 + bp.w_bg * bp.bg0) / Dp : bp.bg0;
+            c1 = hit ? (m1 + bp.w_bg * bp.bg1) / Dp : bp.bg1;
+            c2 = hit ? (m2 + bp.w_bg * bp.bg2) / Dp : bp.bg2;
         } else {  // Eq. 12
-            const bool hit = D[q] > bp.d_min;
-            c0 = hit ? N0[q] / D[q] : bp.bg0;
-            c1 = hit ? N1[q] / D[q] : bp.bg1;
-            c2 = hit ? N2[q] / D[q] : bp.bg2;
+            const bool hit = Dq > bp.d_min;
+            c0 = hit ? m0 / Dq : bp.bg0;
+            c1 = hit ? m1 / Dq : bp.bg1;
+            c2 = hit ? m2 / Dq : bp.bg2;
         }
         img[pin] = c0;
         img[HW + pin] = c1;
@@ -321,18 +364,18 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
             im2[HW + pin] = c1;
             im2[2 * HW + pin] = c2;
         }
-        out_D[V.pix_base + pin] = D[q];
-        out_nd[V.pix_base + pin] = n[q];
+        out_D[V.pix_base + pin] = Dq;
+        out_nd[V.pix_base + pin] = T[q] < bp.eps ? (__float_as_int(T[q]) & 0x7fffffff) - 1 : (int)(rg.y - rg.x);
     }
 }
 
 template <int KT, bool VAR>
-__global__ void __launch_bounds__(WT, FWD_MINB) k_blend_fwd(const ViewDesc *__restrict__ views, int n_views,
+__global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd(const ViewDesc *__restrict__ views, int n_views,
                                                   const uint2 *__restrict__ ranges, const uint32_t *__restrict__ cells,
                                                   const float4 *__restrict__ rec, BlendParams bp,
                                                   float *__restrict__ out_rgb, float *__restrict__ out_rgb2,
                                                   float *__restrict__ out_D, int *__restrict__ out_nd) {
-    __shared__ float4 s_rec[NSTAGE][kRecF4 * (KT > 0 ? KT : kMaxK)];
+    __shared__ float4 s_rec[FSTAGE][kBatchF4];
     blend_fwd_unit<KT, FWD_PPL, VAR>(blockIdx.x, views, n_views, ranges, cells, rec, bp, out_rgb, out_rgb2, out_D, out_nd,
                                 s_rec);
 }
@@ -343,14 +386,14 @@ __global__ void __launch_bounds__(WT, FWD_MINB) k_blend_fwd(const ViewDesc *__re
 // dense and the empty regions of the images balance dynamically.  One
 // atomic per sub-tile: their rate is bounded by the blend work between them.
 template <int KT, bool VAR>
-__global__ void __launch_bounds__(WT, FWD_MINB) k_blend_fwd_pull(const ViewDesc *__restrict__ views,
+__global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd_pull(const ViewDesc *__restrict__ views,
                                                        const uint2 *__restrict__ ranges,
                                                        const uint32_t *__restrict__ cells,
                                                        const float4 *__restrict__ rec, BlendParams bp,
                                                        float *__restrict__ out_rgb, float *__restrict__ out_D,
                                                        int *__restrict__ out_nd, const ChainSizes *__restrict__ dsz,
                                                        uint32_t *__restrict__ work) {
-    __shared__ float4 s_rec[NSTAGE][kRecF4 * (KT > 0 ? KT : kMaxK)];
+    __shared__ float4 s_rec[FSTAGE][kBatchF4];
     const int n_views = dsz->n_views;
     const uint32_t units = (uint32_t)dsz->total_tiles * FWD_SUB;
     for (;;) {
@@ -364,9 +407,14 @@ __global__ void __launch_bounds__(WT, FWD_MINB) k_blend_fwd_pull(const ViewDesc 
     }
 }
 
-// Do the blend kernels need their variant form (a flag or a background weight)?
+// Do the blend kernels need their variant form (a flag, a background weight, or
+// no dilation)?  The default form gives a pixel outside a Gaussian's box an offset of
+// kFar, and needs L's entries finite for it: with the screen covariance dilated they
+// are at most 1/sqrt(dilation), without, a Gaussian of no extent has infinite ones.
+// The variant form masks every pixel's alpha instead.
 static bool blend_variants(const BlendParams &bp) {
-    return (bp.flags & (DGS_FLAG_ALPHA_SKIP | DGS_FLAG_TERM_EXCLUDE | DGS_FLAG_NUMERATOR)) != 0 || bp.w_bg != 0.f;
+    return (bp.flags & (DGS_FLAG_ALPHA_SKIP | DGS_FLAG_TERM_EXCLUDE | DGS_FLAG_NUMERATOR)) != 0 || bp.w_bg != 0.f ||
+           bp.dilation < 1e-12f;
 }
 
 template <int KT, bool VAR>

@@ -121,6 +121,35 @@ def test_gaussians_per_cell(rctx, K):
     _render_and_check(rctx, sc, [synth.small_camera(80, 72)])
 
 
+@pytest.mark.parametrize("K", [2, 5, 8, 11, 16, 17, 31])
+def test_cell_batches(rctx, K):
+    """The forward blends 32 // K cells per batch: list lengths around the
+    batch's, lanes without a Gaussian (K not dividing 32), lists that end or
+    whose pixels finish within a batch (opaque cells)."""
+    sc = synth.make_scene(max(8, 900 // K), K, synth._box(-1, 1), 0.05, 0.4, 1, seed=40 + K)
+    sc.g_logit[:] += 2.0
+    _render_and_check(rctx, sc, [synth.small_camera(75, 50), synth.small_camera(64, 48)])
+
+
+def test_no_dilation_and_a_gaussian_of_no_extent():
+    """Without dilation a Gaussian of no extent has an infinite conic: it is
+    drawn nowhere but at its centre, and its neighbours as if it were absent."""
+    cam = synth.small_camera(64, 48)
+    from paper_2508_03180_gb300.renderer import Context
+    images = []
+    for hidden in (False, True):
+        sc = synth.make_scene(40, 4, synth._box(-0.5, 0.5), 0.2, 0.4, 0, seed=9)
+        sc.g_scale[::7] = 0.0
+        if hidden:
+            sc.g_logit[::7] = -100.0
+            sc.g_scale[::7] = 0.05
+        ctx = Context(dilation=0.0)
+        images.append(ctx.render(ctx.upload_scene(sc), [cam])[0].cpu().numpy())
+        ctx.close()
+    assert np.isfinite(images[0]).all()
+    assert np.abs(images[0] - images[1]).max() <= 1e-6
+
+
 def test_multiscale_subset_480x270(rctx):
     sc = synth.scene_multiscale(n_cells=20_000, K=10)
     _render_and_check(rctx, sc, synth.sphere_cameras(2, 15.0, 480, 270))
