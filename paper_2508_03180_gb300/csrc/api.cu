@@ -107,6 +107,13 @@ dgs_status DevBuf::ensure(size_t bytes) {
     return DGS_OK;
 }
 
+void DevBuf::swap(DevBuf &o) {
+    std::swap(p, o.p);
+    std::swap(cap, o.cap);
+    std::swap(guarded, o.guarded);
+    std::swap(dev, o.dev);
+}
+
 void DevBuf::release() {
     if (p) {
         if (guarded) {
@@ -134,7 +141,7 @@ Workspace::~Workspace() {
 }
 
 std::vector<DevBuf *> Workspace::all() {
-    return {&views, &scenes, &zkey, &zval, &rect, &depth, &count, &cnt_sorted, &offs, &tkey, &tval, &ranges, &rec,
+    return {&views, &scenes, &zkey, &zval, &rect, &depth, &count, &offs, &tkey, &tval, &ranges, &rec,
             &Dpix, &ndpix, &rgb, &g2d, &gstage, &sort_k, &sort_v, &sort_hist, &sort_status, &sort_ctr, &small, &scan, &sizes, &vview, &gvview, &dec};
 }
 
@@ -168,6 +175,28 @@ SortScratch sort_scratch_of(Workspace &ws) {
     s.cap_items = (long long)(ws.sort_k.cap / 4);
     s.cap_parts = (long long)(ws.sort_status.cap / 2048);
     return s;
+}
+
+SortScratch chain_sort_scratch(Workspace &ws, int which) {
+    SortScratch s = sort_scratch_of(ws);
+    s.hist = (uint32_t *)ws.small.p + kSmallHist + 1024 * which;
+    s.counters = (uint32_t *)ws.small.p + kSmallCounters + 4 * which;
+    return s;
+}
+
+BinPrep chain_prep(Workspace &ws, int which, long long n, long long n_tiles) {
+    BinPrep p{};
+    const SortScratch s = chain_sort_scratch(ws, which);
+    p.hist = s.hist;
+    p.status = s.status;
+    p.status_words = sort_status_words(n);
+    if (which == 0) {
+        p.scan = (uint32_t *)ws.scan.p;
+        p.scan_words = scan_scratch_words(n);
+        p.ranges = (uint2 *)ws.ranges.p;
+        p.n_tiles = n_tiles;
+    }
+    return p;
 }
 
 cudaEvent_t Profiler::take() {
@@ -769,111 +798,103 @@ static long long pair_capacity(const dgs_ctx *ctx, const Workspace &ws) {
     return std::max<long long>(1LL << 16, (long long)std::ceil(want));
 }
 
+void sort_tiles(Workspace &ws, long long L, int bits, const uint32_t *d_L, cudaStream_t st) {
+    if (!radix_sort_counted((uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, L, bits, chain_sort_scratch(ws, 1), st, d_L,
+                            nullptr, false))
+        return;
+    // an odd number of passes: the alternate buffers hold the result
+    if (ws.tkey.guarded == ws.sort_k.guarded && ws.tval.guarded == ws.sort_v.guarded) {
+        ws.tkey.swap(ws.sort_k);
+        ws.tval.swap(ws.sort_v);
+    } else {
+        cudaMemcpyAsync(ws.tkey.p, ws.sort_k.p, 4 * (size_t)L, cudaMemcpyDeviceToDevice, st);
+        cudaMemcpyAsync(ws.tval.p, ws.sort_v.p, 4 * (size_t)L, cudaMemcpyDeviceToDevice, st);
+    }
+}
+
 // Binning of all views of the chain (steps a1-a5): cell projection and cull,
 // depth sort over cells, count scan, key emission, tile sort, tile ranges.
 // Synchronises the stream once to learn the sort length L, unless
 // device_sized: then the pair count stays on the device, the pair buffers
-// are sized by pair_capacity and the kernels stop at that capacity (a
-// k_clamp_pairs flag records an overflow).
+// are sized by pair_capacity and the kernels stop at that capacity (the
+// offsets' scan records an overflow).
 static dgs_status run_binning(dgs_ctx *ctx, Workspace &ws, cudaStream_t st, bool device_sized) {
     Profiler &pf = ctx->prof;
     const int V = ws.V;
     const long long n = ws.n_entries;
     const long long n1 = std::max(1LL, n);
     dgs_status s;
-    if ((s = ws.small.ensure(256))) return s;
-    CK(cudaMemsetAsync(ws.small.p, 0, 256, st));
+    if ((s = ws.small.ensure(kSmallBytes))) return s;
+    CK(cudaMemsetAsync(ws.small.p, 0, kSmallBytes, st));
     if ((s = ws.zkey.ensure(4 * n1)) || (s = ws.zval.ensure(4 * n1)) || (s = ws.rect.ensure(8 * n1)) ||
-        (s = ws.depth.ensure(4 * n1)) || (s = ws.count.ensure(4 * n1)) || (s = ws.cnt_sorted.ensure(4 * n1)) ||
-        (s = ws.offs.ensure(4 * n1)) || (s = ws.scan.ensure(4 * scan_scratch_words(n1))) ||
-        (s = ws.vview.ensure(4 * n1)))
+        (s = ws.depth.ensure(4 * n1)) || (s = ws.count.ensure(4 * n1)) || (s = ws.offs.ensure(4 * n1)) ||
+        (s = ws.scan.ensure(4 * scan_scratch_words(n1))) || (s = ws.vview.ensure(4 * n1)) ||
+        (s = ws.ranges.ensure(8 * (size_t)std::max(1, ws.total_tiles))))
         return s;
     if ((s = ensure_sort_scratch(ws, n))) return s;
     // a device-sized chain sizes every buffer before its first launch, so no
     // buffer is reallocated under the kernels in flight
     const long long cap = device_sized ? pair_capacity(ctx, ws) : 0;
     if (device_sized &&
-        ((s = ws.tkey.ensure(4 * cap)) || (s = ws.tval.ensure(4 * cap)) || (s = ensure_sort_scratch(ws, cap)) ||
-         (s = ws.ranges.ensure(8 * (size_t)std::max(1, ws.total_tiles))) || (s = ws.sizes.ensure(sizeof(ChainSizes)))))
+        ((s = ws.tkey.ensure(4 * cap)) || (s = ws.tval.ensure(4 * cap)) || (s = ensure_sort_scratch(ws, cap))))
         return s;
     uint32_t *small = (uint32_t *)ws.small.p;
+    const uint32_t *d_vis = small + kSmallVisible;  // entries that survive culling: the depth sort keeps those
     const ViewDesc *dv = (const ViewDesc *)ws.views.p;
     {
         StageTimer t(pf, DGS_STAGE_CELL_PROJECT, st);
         launch_cell_project(dv, V, (const SceneDev *)ws.scenes.p, n, (uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p,
                             (short4 *)ws.rect.p, (float *)ws.depth.p, (uint32_t *)ws.count.p, small + kSmallVisible,
-                            (float *)ws.vview.p, ctx->cfg.flags, st);
+                            (float *)ws.vview.p, ctx->cfg.flags, chain_prep(ws, 0, n, ws.total_tiles), st);
     }
     {
         StageTimer t(pf, DGS_STAGE_DEPTH_SORT, st);
-        radix_sort_pairs((uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p, n, 32, sort_scratch_of(ws), st);
+        radix_sort_counted((uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p, n, 32, chain_sort_scratch(ws, 0), st, nullptr,
+                           d_vis, false);
     }
     {
         StageTimer t(pf, DGS_STAGE_COUNT_SCAN, st);
-        launch_gather_counts((const uint32_t *)ws.zval.p, (const uint32_t *)ws.count.p, n, (uint32_t *)ws.cnt_sorted.p,
-                             st);
-        exclusive_scan_u32((const uint32_t *)ws.cnt_sorted.p, (uint32_t *)ws.offs.p, n, small + kSmallTotal,
-                           (uint32_t *)ws.scan.p, st);
+        launch_pair_offsets((const uint32_t *)ws.zval.p, (const uint32_t *)ws.count.p, n, nullptr, d_vis,
+                            (uint32_t *)ws.offs.p, (uint32_t *)ws.scan.p, small + kSmallCounters + 8, small, kPairSlots,
+                            device_sized ? (uint32_t)cap : 0xFFFFFFFFu, nullptr, st);
     }
     CK(cudaGetLastError());
     int bits = 1;
     while ((1LL << bits) < ws.total_tiles) ++bits;
+    long long L = cap;              // pairs, or (device-sized) their capacity
+    const uint32_t *d_L = nullptr;  // and then the count min(pairs, cap) on the device
     if (device_sized) {
         ws.L_cap = cap;
         ws.L = -1;
         ws.n_vis = -1;
-        *ws.h_sizes = ChainSizes{};
-        ws.h_sizes->n_entries = (uint32_t)n;
-        ws.h_sizes->n_views = V;
-        ws.h_sizes->total_tiles = ws.total_tiles;
-        ws.h_sizes->L_cap = (uint32_t)cap;
-        ws.h_sizes->n_scenes = (int32_t)ws.scene_ids.size();
-        CK(cudaMemcpyAsync(ws.sizes.p, ws.h_sizes, sizeof(ChainSizes), cudaMemcpyHostToDevice, st));
-        const uint32_t *d_L = small + kSmallPairs;  // min(L, cap), written on the device
-        launch_clamp_pairs(small, kSmallTotal, kSmallPairs, kSmallOverflow, (const ChainSizes *)ws.sizes.p, st);
-        {
-            StageTimer t(pf, DGS_STAGE_EMIT, st);
-            launch_emit((const uint32_t *)ws.offs.p, (const uint32_t *)ws.zval.p, (const short4 *)ws.rect.p, dv, V,
-                        n, cap, (uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, st, nullptr, d_L);
-        }
-        {
-            StageTimer t(pf, DGS_STAGE_TILE_SORT, st);
-            radix_sort_pairs((uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, cap, bits, sort_scratch_of(ws), st, d_L);
-        }
-        {
-            StageTimer t(pf, DGS_STAGE_TILE_RANGES, st);
-            CK(cudaMemsetAsync(ws.ranges.p, 0, 8 * (size_t)std::max(1, ws.total_tiles), st));
-            launch_tile_ranges((const uint32_t *)ws.tkey.p, cap, (uint2 *)ws.ranges.p, st, d_L);
-        }
-        CK(cudaGetLastError());
-        ws.async_pending = true;
-        return DGS_OK;
+        d_L = small + kSmallPairs;
+    } else {
+        CK(cudaMemcpyAsync(ws.h_small, small, 64, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        if (ws.h_small[kSmallSortErr]) return set_error(DGS_ERR_TIMEOUT, "radix sort look-back wait gave up");
+        L = ws.h_small[kSmallTotal];
+        ws.L = L;
+        ws.n_vis = ws.h_small[kSmallVisible];
+        if (ws.total_tiles > 0) ctx->pairs_per_tile = std::max(ctx->pairs_per_tile, (double)L / ws.total_tiles);
+        if ((s = ws.tkey.ensure(4 * std::max(1LL, L))) || (s = ws.tval.ensure(4 * std::max(1LL, L)))) return s;
+        if ((s = ensure_sort_scratch(ws, L))) return s;
     }
-    CK(cudaMemcpyAsync(ws.h_small, small, 64, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (ws.h_small[kSmallSortErr]) return set_error(DGS_ERR_TIMEOUT, "radix sort look-back wait gave up");
-    const long long L = ws.h_small[kSmallTotal];
-    ws.L = L;
-    ws.n_vis = ws.h_small[kSmallVisible];
-    if (ws.total_tiles > 0) ctx->pairs_per_tile = std::max(ctx->pairs_per_tile, (double)L / ws.total_tiles);
-    if ((s = ws.tkey.ensure(4 * std::max(1LL, L))) || (s = ws.tval.ensure(4 * std::max(1LL, L)))) return s;
-    if ((s = ensure_sort_scratch(ws, L))) return s;
-    if ((s = ws.ranges.ensure(8 * (size_t)std::max(1, ws.total_tiles)))) return s;
     {
         StageTimer t(pf, DGS_STAGE_EMIT, st);
-        launch_emit((const uint32_t *)ws.offs.p, (const uint32_t *)ws.zval.p, (const short4 *)ws.rect.p, dv, V, n, L,
-                    (uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, st);
+        launch_emit((const uint32_t *)ws.offs.p, (const uint32_t *)ws.zval.p, (const short4 *)ws.rect.p, dv, V, n, n, L,
+                    ws.total_tiles, (uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, (bits + 7) / 8,
+                    chain_prep(ws, 1, L, 0), st, nullptr, d_vis, d_L);
     }
     {
         StageTimer t(pf, DGS_STAGE_TILE_SORT, st);
-        radix_sort_pairs((uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, L, bits, sort_scratch_of(ws), st);
+        sort_tiles(ws, L, bits, d_L, st);
     }
     {
         StageTimer t(pf, DGS_STAGE_TILE_RANGES, st);
-        CK(cudaMemsetAsync(ws.ranges.p, 0, 8 * (size_t)std::max(1, ws.total_tiles), st));
-        launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, st);
+        launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, st, d_L);
     }
     CK(cudaGetLastError());
+    if (device_sized) ws.async_pending = true;
     return DGS_OK;
 }
 

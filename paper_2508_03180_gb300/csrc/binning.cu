@@ -2,6 +2,8 @@
 // proxy of every view, cull it to the frustum, bound its screen footprint,
 // and emit one (tile, cell) pair per covered tile.  Depth ordering comes from
 // a radix sort over cells (sort.cu); a second stable sort groups by tile.
+#include <algorithm>
+
 #include "internal.cuh"
 #include "sh.cuh"
 
@@ -20,8 +22,12 @@ __global__ void __launch_bounds__(256) k_cell_project(const ViewDesc *__restrict
                                                       uint32_t *__restrict__ zkey, uint32_t *__restrict__ zval,
                                                       short4 *__restrict__ rect, float *__restrict__ depth,
                                                       uint32_t *__restrict__ count, uint32_t *__restrict__ visible,
-                                                      float *__restrict__ vview, int flags,
+                                                      float *__restrict__ vview, int flags, BinPrep prep,
                                                       const ChainSizes *__restrict__ dsz) {
+    __shared__ uint32_t s_hist[4][256];  // the depth keys' digits
+    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) (&s_hist[0][0])[i] = 0u;
+    __syncthreads();
+    prep_clear(prep, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
     if (dsz) n_views = dsz->n_views;
     uint32_t nvis = 0;
     for (int v = 0; v < n_views; ++v) {
@@ -107,16 +113,26 @@ __global__ void __launch_bounds__(256) k_cell_project(const ViewDesc *__restrict
         }
         vview[i] = vn;
         // depth key: positive float bits order like the floats; culled last
-        zkey[i] = vis ? __float_as_uint(dz) : 0xFFFFFFFFu;
+        const uint32_t key = vis ? __float_as_uint(dz) : 0xFFFFFFFFu;
+        zkey[i] = key;
         zval[i] = (uint32_t)i;
         count[i] = vis ? (uint32_t)((r.z - r.x + 1) * (r.w - r.y + 1)) : 0u;
         nvis += vis ? 1u : 0u;
+        if (vis) {
+#pragma unroll
+            for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p][(key >> (8 * p)) & 255u], 1u);
+        }
     }
     }
     // one atomic per warp for the visible-cell statistic
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nvis += __shfl_xor_sync(0xffffffffu, nvis, o);
     if ((threadIdx.x & 31) == 0 && nvis) atomicAdd(visible, nvis);
+    __syncthreads();
+    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) {
+        const uint32_t c = (&s_hist[0][0])[i];
+        if (c) atomicAdd(prep.hist + i, c);
+    }
 }
 
 static int grid_for(long long n, int threads) {
@@ -128,108 +144,172 @@ static int grid_for(long long n, int threads) {
 
 void launch_cell_project(const ViewDesc *views, int n_views, const SceneDev *scenes, long long n_entries,
                          uint32_t *zkey, uint32_t *zval, short4 *rect, float *depth, uint32_t *count,
-                         uint32_t *visible, float *vview, int flags, cudaStream_t st, const ChainSizes *dsz) {
-    if (n_entries == 0) return;
-    k_cell_project<<<grid_for(n_entries / n_views + 1, 256), 256, 0, st>>>(views, n_views, scenes, zkey, zval, rect,
-                                                                          depth, count, visible, vview, flags, dsz);
-}
-
-__global__ void k_gather_counts(const uint32_t *__restrict__ idx, const uint32_t *__restrict__ count, long long n,
-                                const uint32_t *__restrict__ d_n, uint32_t *__restrict__ out) {
-    if (d_n) n = *d_n;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = count[idx[i]];
-}
-
-void launch_gather_counts(const uint32_t *zval_sorted, const uint32_t *count, long long n, uint32_t *out,
-                          cudaStream_t st, const uint32_t *d_n) {
-    if (n == 0) return;
-    k_gather_counts<<<grid_for(n, 256), 256, 0, st>>>(zval_sorted, count, n, d_n, out);
+                         uint32_t *visible, float *vview, int flags, const BinPrep &prep, cudaStream_t st,
+                         const ChainSizes *dsz) {
+    // eight blocks an SM at most: each adds its digit counts to the global ones once
+    k_cell_project<<<std::min(grid_for(n_entries / n_views + 1, 256), 152 * 8), 256, 0, st>>>(
+        views, n_views, scenes, zkey, zval, rect, depth, count, visible, vview, flags, prep, dsz);
 }
 
 // Output slot j belongs to the last entry e with offs[e] <= j.  A block takes
-// runs of EM_TB consecutive slots: thread 0 finds the run's first and last
-// owners by binary search in global memory; when at most EM_TB entries lie
-// between them (always for the depth-sorted cell entries, whose culled ones
-// come last, so every entry in a run owns a slot) their offsets are staged
-// in shared memory and each thread finds its slots' owners there, otherwise
-// (entries that own no slot interleaved, as in the weighted-sum comparator's
-// index order) it searches the run's entries in global memory.  Consecutive
-// threads write consecutive addresses whatever the footprints.  Entries are in depth order, so the emitted sequence is
-// (depth, cell)-ordered within every tile; the stable tile sort keeps that order.
+// runs of EM_TB consecutive slots.  Two warps find the run's first and last owners
+// in global memory, 32 probes at a time (four dependent reads for a million
+// entries; one thread's two binary searches were 40, most of a small view's 19 us
+// in here).  When at most EM_TB entries lie between them (always for the
+// depth-sorted entries, of which each owns a slot) their offsets are staged in
+// shared memory, otherwise (entries that own no slot interleaved, as in the
+// weighted-sum comparator's index order) they are searched in global memory.  A
+// thread finds the owner of the first of its eight consecutive slots and walks on from
+// there, one division for its tile, and writes the eight keys and cells as vectors.
+// Entries are in depth order, so the emitted sequence is (depth, cell)-ordered
+// within every tile; the stable tile sort keeps that order.  The keys' digits are
+// counted on the way, runs of equal digits of a thread at once.
 constexpr int EM_THREADS = 256, EM_ITEMS = 8, EM_TB = EM_THREADS * EM_ITEMS;
+
+// Last entry e in [0, n) with offs[e] <= j (0 if there is none), by one warp.
+__device__ __forceinline__ long long warp_owner(const uint32_t *__restrict__ offs, long long n, long long j, int lane) {
+    long long lo = 0, hi = n;  // offs[lo] <= j (or lo = 0), offs[hi] > j (or hi = n)
+    while (hi - lo > 1) {
+        const long long step = (hi - lo + 31) / 32, at = lo + (lane + 1) * step;  // probes above lo
+        const bool le = at < hi && (long long)offs[at] <= j;
+        const int m = __popc(__ballot_sync(0xffffffffu, le));  // (offs is sorted: the first m probes)
+        const long long nlo = lo + m * step;
+        hi = min(hi, nlo + step);
+        lo = nlo;
+    }
+    return lo;
+}
+
 __global__ void __launch_bounds__(EM_THREADS) k_emit(const uint32_t *__restrict__ offs,
                                                      const uint32_t *__restrict__ zval,
                                                      const short4 *__restrict__ rect,
                                                      const ViewDesc *__restrict__ views, int n_views,
-                                                     long long n_entries, long long L, uint32_t *__restrict__ tkey,
-                                                     uint32_t *__restrict__ tval,
-                                                     const ChainSizes *__restrict__ dsz,
+                                                     long long n_entries, long long n_all, long long L, int n_tiles,
+                                                     uint32_t *__restrict__ tkey, uint32_t *__restrict__ tval,
+                                                     int passes, BinPrep prep, const ChainSizes *__restrict__ dsz,
+                                                     const uint32_t *__restrict__ d_n,
                                                      const uint32_t *__restrict__ d_L) {
-    __shared__ uint32_t s_off[EM_TB];
-    __shared__ long long s_e0, s_ne;
+    __shared__ uint32_t s_off[EM_TB + 1];
+    __shared__ uint32_t s_hist[4][256];
+    __shared__ long long s_own[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < passes * 256; i += EM_THREADS) (&s_hist[0][0])[i] = 0u;
+    prep_clear(prep, blockIdx.x * (long long)EM_THREADS + tid, (long long)gridDim.x * EM_THREADS);
     if (dsz) {
         n_views = dsz->n_views;
-        n_entries = dsz->n_entries;
+        n_all = dsz->n_entries;
+        n_tiles = dsz->total_tiles;
     }
+    if (d_n) n_entries = *d_n;
     if (d_L) L = *d_L;
     for (long long j0 = blockIdx.x * (long long)EM_TB; j0 < L; j0 += (long long)gridDim.x * EM_TB) {
         const long long j1 = min(j0 + (long long)EM_TB, L);  // this run: [j0, j1)
-        if (threadIdx.x == 0) {
-            auto owner = [&](long long j) {
-                long long lo = 0, hi = n_entries;
-                while (hi - lo > 1) {
-                    const long long mid = (lo + hi) >> 1;
-                    if ((long long)offs[mid] <= j) lo = mid; else hi = mid;
-                }
-                return lo;
-            };
-            const long long e0 = owner(j0);
-            s_e0 = e0;
-            s_ne = owner(j1 - 1) - e0 + 1;
+        __syncthreads();  // s_off and s_own of the last run are read (and s_hist is clear)
+        if (warp < 2) {
+            const long long o = warp_owner(offs, n_entries, warp == 0 ? j0 : j1 - 1, lane);
+            if (lane == 0) s_own[warp] = o;
         }
         __syncthreads();
-        const long long e0 = s_e0, ne = s_ne;  // the run's owners are entries [e0, e0 + ne)
+        const long long e0 = s_own[0], ne = s_own[1] - e0 + 1;  // the run's owners are entries [e0, e0 + ne)
         const bool staged = ne <= EM_TB;
         if (staged)
-            for (int i = threadIdx.x; i < (int)ne; i += EM_THREADS) s_off[i] = offs[e0 + i];
+            for (int i = tid; i < (int)ne; i += EM_THREADS) s_off[i] = offs[e0 + i];
         __syncthreads();
-#pragma unroll 2
-        for (int it = 0; it < EM_ITEMS; ++it) {
-            const long long j = j0 + it * EM_THREADS + threadIdx.x;
-            if (j >= j1) break;
-            long long lo = 0, hi = ne;  // last i in [0, ne) with offs[e0 + i] <= j
-            while (hi - lo > 1) {
-                const long long mid = (lo + hi) >> 1;
-                const uint32_t o = staged ? s_off[mid] : offs[e0 + mid];
-                if ((long long)o <= j) lo = mid; else hi = mid;
-            }
-            const uint32_t base = staged ? s_off[lo] : offs[e0 + lo];
-            const uint32_t vi = zval[e0 + lo];
-            int vlo = 0, vhi = n_views;  // view owning entry vi
-            while (vhi - vlo > 1) {
-                const int mid = (vlo + vhi) >> 1;
-                if (views[mid].cell_base <= (long long)vi) vlo = mid; else vhi = mid;
-            }
-            const ViewDesc &V = views[vlo];
-            const uint32_t cellid = (uint32_t)((long long)vi - V.cell_base);
-            const short4 r = rect[vi];
-            const int w = r.z - r.x + 1;
-            const int local = (int)(j - base);
-            const int ty = r.y + local / w, tx = r.x + local % w;
-            tkey[j] = (uint32_t)(V.tile_base + ty * V.Tx + tx);
-            tval[j] = cellid;
+        const long long j = j0 + (long long)tid * EM_ITEMS;
+        if (j >= j1) continue;
+        auto off = [&](long long i) { return (long long)(staged ? s_off[i] : offs[e0 + i]); };
+        long long lo = 0, hi = ne;  // last i in [0, ne) with off(i) <= j
+        while (hi - lo > 1) {
+            const long long mid = (lo + hi) >> 1;
+            if (off(mid) <= j) lo = mid; else hi = mid;
         }
-        __syncthreads();  // s_off is refilled for the next run
+        uint32_t key[EM_ITEMS], cell[EM_ITEMS];
+        long long own = lo, next = -1;  // the current owner; its slots end before `next`
+        int x = 0, y = 0, x0 = 0, x1 = 0, Tx = 0, tile_base = 0;
+        uint32_t cellid = 0;
+#pragma unroll
+        for (int i = 0; i < EM_ITEMS; ++i) {
+            const long long ji = j + i;
+            key[i] = cell[i] = 0u;
+            if (ji < j1) {
+                if (ji >= next) {  // enter the owner of slot ji
+                    if (i > 0)
+                        while (own + 1 < ne && off(own + 1) <= ji) ++own;
+                    next = own + 1 < ne ? off(own + 1) : j1;
+                    // (bounds: only a sort that gave up can leave an entry outside the arrays)
+                    const uint32_t vi = (uint32_t)min((long long)zval[e0 + own], n_all - 1);
+                    int vlo = 0, vhi = n_views;  // view owning entry vi
+                    while (vhi - vlo > 1) {
+                        const int mid = (vlo + vhi) >> 1;
+                        if (views[mid].cell_base <= (long long)vi) vlo = mid; else vhi = mid;
+                    }
+                    const ViewDesc &V = views[vlo];
+                    cellid = (uint32_t)((long long)vi - V.cell_base);
+                    const short4 r = rect[vi];
+                    const int w = r.z - r.x + 1, local = (int)(ji - off(own));
+                    x0 = r.x;
+                    x1 = r.z;
+                    y = r.y + local / w;
+                    x = x0 + local % w;
+                    Tx = V.Tx;
+                    tile_base = V.tile_base;
+                }
+                key[i] = min((uint32_t)(tile_base + y * Tx + x), (uint32_t)(n_tiles - 1));
+                cell[i] = cellid;
+                if (++x > x1) {
+                    x = x0;
+                    ++y;
+                }
+            }
+        }
+        if (j + EM_ITEMS <= j1) {
+#pragma unroll
+            for (int i = 0; i < EM_ITEMS; i += 4) {
+                *reinterpret_cast<uint4 *>(tkey + j + i) = make_uint4(key[i], key[i + 1], key[i + 2], key[i + 3]);
+                *reinterpret_cast<uint4 *>(tval + j + i) = make_uint4(cell[i], cell[i + 1], cell[i + 2], cell[i + 3]);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < EM_ITEMS; ++i)
+                if (j + i < j1) {
+                    tkey[j + i] = key[i];
+                    tval[j + i] = cell[i];
+                }
+        }
+        const int n = (int)min((long long)EM_ITEMS, j1 - j);
+        for (int p = 0; p < passes; ++p) {
+            uint32_t d = (key[0] >> (8 * p)) & 255u, run = 1;
+#pragma unroll
+            for (int i = 1; i < EM_ITEMS; ++i) {
+                const uint32_t di = (key[i] >> (8 * p)) & 255u;
+                if (i < n) {
+                    if (di != d) {
+                        atomicAdd(&s_hist[p][d], run);
+                        d = di;
+                        run = 0;
+                    }
+                    ++run;
+                }
+            }
+            atomicAdd(&s_hist[p][d], run);
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < passes * 256; i += EM_THREADS) {
+        const uint32_t c = (&s_hist[0][0])[i];
+        if (c) atomicAdd(prep.hist + i, c);
     }
 }
 
 void launch_emit(const uint32_t *offs, const uint32_t *zval_sorted, const short4 *rect, const ViewDesc *views,
-                 int n_views, long long n_entries, long long L, uint32_t *tkey, uint32_t *tval, cudaStream_t st,
-                 const ChainSizes *dsz, const uint32_t *d_L) {
+                 int n_views, long long n_entries, long long n_all, long long L, int n_tiles, uint32_t *tkey,
+                 uint32_t *tval, int passes, const BinPrep &prep, cudaStream_t st, const ChainSizes *dsz,
+                 const uint32_t *d_n, const uint32_t *d_L) {
     if (L == 0) return;
-    k_emit<<<grid_for((L + EM_ITEMS - 1) / EM_ITEMS, EM_THREADS), EM_THREADS, 0, st>>>(
-        offs, zval_sorted, rect, views, n_views, n_entries, L, tkey, tval, dsz, d_L);
+    // eight blocks an SM at most: each adds its digit counts to the global ones once
+    const long long runs = (L + EM_TB - 1) / EM_TB;
+    k_emit<<<(unsigned)std::min<long long>(runs, 152 * 8), EM_THREADS, 0, st>>>(
+        offs, zval_sorted, rect, views, n_views, n_entries, n_all, L, n_tiles, tkey, tval, passes, prep, dsz, d_n, d_L);
 }
 
 // [start, end) of every non-empty tile from the tile-sorted keys; empty
@@ -248,17 +328,6 @@ void launch_tile_ranges(const uint32_t *tkey_sorted, long long L, uint2 *ranges,
                         const uint32_t *d_L) {
     if (L == 0) return;
     k_tile_ranges<<<grid_for(L, 256), 256, 0, st>>>(tkey_sorted, L, d_L, ranges);
-}
-
-__global__ void k_clamp_pairs(uint32_t *small, int total, int clamped, int overflow, const ChainSizes *dsz) {
-    const uint32_t L = small[total], cap = dsz->L_cap;
-    small[clamped] = L < cap ? L : cap;
-    small[overflow] = L > cap ? 1u : 0u;
-}
-
-void launch_clamp_pairs(uint32_t *small, int total, int clamped, int overflow, const ChainSizes *dsz,
-                        cudaStream_t st) {
-    k_clamp_pairs<<<1, 1, 0, st>>>(small, total, clamped, overflow, dsz);
 }
 
 }  // namespace dgs

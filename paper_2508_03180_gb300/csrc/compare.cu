@@ -183,9 +183,9 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
     ws.n_records = n;
     const long long n1 = std::max(1LL, n);
     dgs_status s;
-    if ((s = ws.views.ensure(sizeof(ViewDesc) * V)) || (s = ws.small.ensure(256)) || (s = ws.zkey.ensure(4 * n1)) ||
+    if ((s = ws.views.ensure(sizeof(ViewDesc) * V)) || (s = ws.small.ensure(kSmallBytes)) || (s = ws.zkey.ensure(4 * n1)) ||
         (s = ws.zval.ensure(4 * n1)) || (s = ws.rect.ensure(8 * n1)) || (s = ws.count.ensure(4 * n1)) ||
-        (s = ws.cnt_sorted.ensure(4 * n1)) || (s = ws.offs.ensure(4 * n1)) ||
+        (s = ws.offs.ensure(4 * n1)) ||
         (s = ws.scan.ensure(4 * scan_scratch_words(n1))) || (s = ensure_sort_scratch(ws, n)) ||
         (s = ws.rec.ensure(sizeof(float4) * kRecF4 * n1)) || (s = ws.ranges.ensure(8 * (size_t)std::max(1, tiles))))
         return s;
@@ -199,19 +199,20 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
     memcpy(ws.h_views, hv.data(), sizeof(ViewDesc) * V);
     CK(cudaMemcpyAsync(ws.views.p, ws.h_views, sizeof(ViewDesc) * V, cudaMemcpyHostToDevice, st));
     uint32_t *small = (uint32_t *)ws.small.p;
-    CK(cudaMemsetAsync(small, 0, 256, st));
+    CK(cudaMemsetAsync(small, 0, kSmallBytes, st));
     const ViewDesc *dv = (const ViewDesc *)ws.views.p;
     const BlendParams bp = blend_params(ctx->cfg);
     const float tau = std::isfinite(cfg.tau) && cfg.tau > 0.f ? cfg.tau : 0.f;
     launch_gauss_bin(dv, V, sc.dev(), bp, wsr, tau, (float4 *)ws.rec.p, (uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p,
-                     (short4 *)ws.rect.p, (uint32_t *)ws.count.p, small + kSmallVisible, st);
-    const uint32_t *counts = (const uint32_t *)ws.count.p;
-    if (!wsr) {  // global depth order over every (view, Gaussian) entry
-        radix_sort_pairs((uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p, n, 32, sort_scratch_of(ws), st);
-        launch_gather_counts((const uint32_t *)ws.zval.p, counts, n, (uint32_t *)ws.cnt_sorted.p, st);
-        counts = (const uint32_t *)ws.cnt_sorted.p;
-    }  // weighted sums: entries stay in index order (zval is the identity)
-    exclusive_scan_u32(counts, (uint32_t *)ws.offs.p, n, small + kSmallTotal, (uint32_t *)ws.scan.p, st);
+                     (short4 *)ws.rect.p, (uint32_t *)ws.count.p, small + kSmallVisible, chain_prep(ws, 0, n, tiles), st);
+    const uint32_t *d_vis = wsr ? nullptr : small + kSmallVisible;
+    if (!wsr)  // global depth order over every visible (view, Gaussian) entry
+        radix_sort_counted((uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p, n, 32, chain_sort_scratch(ws, 0), st, nullptr,
+                           d_vis, false);
+    // weighted sums: entries stay in index order (zval is the identity)
+    launch_pair_offsets((const uint32_t *)ws.zval.p, (const uint32_t *)ws.count.p, n, nullptr, d_vis,
+                        (uint32_t *)ws.offs.p, (uint32_t *)ws.scan.p, small + kSmallCounters + 8, small, kPairSlots,
+                        0xFFFFFFFFu, nullptr, st);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(ws.h_small, small, 64, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -221,12 +222,12 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
     if ((s = ws.tkey.ensure(4 * std::max(1LL, L))) || (s = ws.tval.ensure(4 * std::max(1LL, L))) ||
         (s = ensure_sort_scratch(ws, L)))
         return s;
-    launch_emit((const uint32_t *)ws.offs.p, (const uint32_t *)ws.zval.p, (const short4 *)ws.rect.p, dv, V, n, L,
-                (uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, st);
     int bits = 1;
     while ((1LL << bits) < tiles) ++bits;
-    radix_sort_pairs((uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, L, bits, sort_scratch_of(ws), st);
-    CK(cudaMemsetAsync(ws.ranges.p, 0, 8 * (size_t)std::max(1, tiles), st));
+    launch_emit((const uint32_t *)ws.offs.p, (const uint32_t *)ws.zval.p, (const short4 *)ws.rect.p, dv, V, n, n, L, tiles,
+                (uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, (bits + 7) / 8, chain_prep(ws, 1, L, 0), st, nullptr,
+                d_vis, nullptr);
+    sort_tiles(ws, L, bits, nullptr, st);
     launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, st);
     if (tiles > 0) {
         const unsigned grid = (unsigned)tiles * CSUB;

@@ -117,27 +117,35 @@ __device__ __forceinline__ void xform_s(const float R[9], const float t[3], floa
 // vview[entry]: v_n as rendered in that view (the scalar, or the clamped SH
 // value of a view-dependent v_n).
 // flags: dgs_config.flags (DGS_FLAG_NEAR_FULL changes the footprint of cells at the near plane).
+// The binning kernels also prepare their successors, so that a chain needs one
+// memset and no kernel that only counts: they add up the digit counts of
+// the sort that follows (hist, zeroed before) and clear the words listed here.
+struct BinPrep {
+    uint32_t *hist;          // of the sort that follows: [passes][256]
+    uint32_t *status;        // look-back words of its first pass
+    long long status_words;
+    uint32_t *scan;          // look-back words of launch_pair_offsets (cell / Gaussian binning)
+    long long scan_words;
+    uint2 *ranges;           // tile ranges (empty tiles stay (0, 0))
+    long long n_tiles;
+};
 void launch_cell_project(const ViewDesc *views, int n_views, const SceneDev *scenes, long long n_entries,
                          uint32_t *zkey, uint32_t *zval, short4 *rect, float *depth, uint32_t *count,
-                         uint32_t *visible, float *vview, int flags, cudaStream_t st,
+                         uint32_t *visible, float *vview, int flags, const BinPrep &prep, cudaStream_t st,
                          const ChainSizes *dsz = nullptr);
-void launch_gather_counts(const uint32_t *zval_sorted, const uint32_t *count, long long n, uint32_t *out,
-                          cudaStream_t st, const uint32_t *d_n = nullptr);
+// n_entries: the sorted entries (capacity with d_n); n_all: (view, cell) entries.
+// Keys are below n_tiles.
 void launch_emit(const uint32_t *offs, const uint32_t *zval_sorted, const short4 *rect, const ViewDesc *views,
-                 int n_views, long long n_entries, long long L, uint32_t *tkey, uint32_t *tval, cudaStream_t st,
-                 const ChainSizes *dsz = nullptr, const uint32_t *d_L = nullptr);
+                 int n_views, long long n_entries, long long n_all, long long L, int n_tiles, uint32_t *tkey,
+                 uint32_t *tval, int passes, const BinPrep &prep, cudaStream_t st, const ChainSizes *dsz,
+                 const uint32_t *d_n, const uint32_t *d_L);
 void launch_tile_ranges(const uint32_t *tkey_sorted, long long L, uint2 *ranges, cudaStream_t st,
                         const uint32_t *d_L = nullptr);
-// small[total] = pairs needed; writes small[clamped] = min(total, L_cap) and
-// small[overflow] = (total > L_cap), for chains whose pair buffers are
-// sized in advance.
-void launch_clamp_pairs(uint32_t *small, int total, int clamped, int overflow, const ChainSizes *dsz,
-                        cudaStream_t st);
 
 // sort.cu
 struct SortScratch {
     uint32_t *keys_alt, *vals_alt;   // n each
-    uint32_t *hist;                  // 4 * 256
+    uint32_t *hist;                  // 4 * 256 digit counts
     uint32_t *status;                // 2 * parts * 256 (alternate passes)
     uint32_t *counters;              // 4 (one per pass)
     uint32_t *err;                   // 1
@@ -147,11 +155,27 @@ long long sort_parts_for(long long n);
 // Stable LSD radix sort of (key, val) by the low `bits` bits.  Results end in
 // keys/vals.  Returns the number of passes.
 int radix_sort_pairs(uint32_t *keys, uint32_t *vals, long long n, int bits, const SortScratch &s,
-                     cudaStream_t st, const uint32_t *d_n = nullptr);
-// Exclusive scan; total written to *total (device).  scratch >= scan_scratch_words(n).
+                     cudaStream_t st);
+// The same with s.hist holding the digits' counts, s.counters zeroed and the first
+// pass's sort_status_words(n) look-back words cleared already (BinPrep).  Returns
+// true if the result is in the alternate buffers.  d_n: the count in device memory,
+// n being the capacity.  d_live: items with key 0xFFFFFFFF, in no count, are left
+// out and *d_live remain.  skip_trivial: passes whose digit is 0 in every key are
+// skipped on the device, and the result is copied back (false returned).
+bool radix_sort_counted(uint32_t *keys, uint32_t *vals, long long n, int bits, const SortScratch &s, cudaStream_t st,
+                        const uint32_t *d_n, const uint32_t *d_live, bool skip_trivial);
+long long sort_status_words(long long n);
+// offs[i] = sum over the entries before i of count[idx[i]], and the total, its clamp
+// to the pair capacity (cap, or dsz->L_cap) and the overflow flag in `small`.
+// n: entries (capacity with d_all / d_n; d_n: how many of them idx lists).
+// scratch: scan_scratch_words(n) words, zeroed; counter: one zeroed word.
+struct PairSlots {
+    int total, clamped, overflow, err;  // words of `small`
+};
 long long scan_scratch_words(long long n);
-void exclusive_scan_u32(const uint32_t *in, uint32_t *out, long long n, uint32_t *total, uint32_t *scratch,
-                        cudaStream_t st, const uint32_t *d_n = nullptr);
+void launch_pair_offsets(const uint32_t *idx, const uint32_t *count, long long n, const uint32_t *d_all,
+                         const uint32_t *d_n, uint32_t *offs, uint32_t *scratch, uint32_t *counter, uint32_t *small,
+                         const PairSlots &slots, uint32_t cap, const ChainSizes *dsz, cudaStream_t st);
 
 // project.cu  (one launch per distinct scene of the chain: views whose
 // scene_slot differs from `slot` are skipped)
@@ -173,7 +197,7 @@ struct CellGrads {
 // (views with N = G, K = 1 entries); wsr selects the LC-WSR weight in r2.w.
 void launch_gauss_bin(const ViewDesc *views, int n_views, const SceneDev &sc, const BlendParams &bp, bool wsr,
                       float tau, float4 *rec, uint32_t *zkey, uint32_t *zval, short4 *rect, uint32_t *count,
-                      uint32_t *visible, cudaStream_t st);
+                      uint32_t *visible, const BinPrep &prep, cudaStream_t st);
 // Neural scenes: decode the Gaussians of the (view, cell) entries
 // samples[0 .. nsamp) (entry e = cell_base of its view + cell; NULL: entry q
 // for sample q) of scene `slot` into dec [rec_base + g][kDecF] and, with rec
@@ -251,6 +275,13 @@ long long resident_ctas(const void *kernel, int threads);
 // Test-only: make the radix sort's look-back waits run out (see sort.cu).
 cudaError_t set_sort_fault(bool on);
 cudaError_t set_tc_fault(bool on);  // the tensor-core decode's completion wait runs out (DGS_FAULT_TC_WAIT)
+
+// Clear the words of a BinPrep (all threads of the grid).
+__device__ __forceinline__ void prep_clear(const BinPrep &p, long long thread, long long threads) {
+    for (long long i = thread; i < p.status_words; i += threads) p.status[i] = 0u;
+    for (long long i = thread; i < p.scan_words; i += threads) p.scan[i] = 0u;
+    for (long long i = thread; i < p.n_tiles; i += threads) p.ranges[i] = make_uint2(0u, 0u);
+}
 
 // Asynchronous 16-byte global-to-shared copies (cp.async, cached in L2
 // only): both addresses 16-byte aligned.  A copy is complete for the issuing

@@ -71,7 +71,11 @@ __global__ void __launch_bounds__(128) k_gauss_bin(const ViewDesc *__restrict__ 
                                                    BlendParams bp, bool wsr, float tau, float4 *__restrict__ rec,
                                                    uint32_t *__restrict__ zkey, uint32_t *__restrict__ zval,
                                                    short4 *__restrict__ rect, uint32_t *__restrict__ count,
-                                                   uint32_t *__restrict__ visible) {
+                                                   uint32_t *__restrict__ visible, BinPrep prep) {
+    __shared__ uint32_t s_hist[4][256];  // the depth keys' digits
+    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) (&s_hist[0][0])[i] = 0u;
+    __syncthreads();
+    prep_clear(prep, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
     const long long G = sc.G, N = sc.N;
     const int K = sc.K;
     uint32_t nvis = 0;
@@ -108,15 +112,25 @@ __global__ void __launch_bounds__(128) k_gauss_bin(const ViewDesc *__restrict__ 
             float4 *o = rec + (Vw.rec_base + g) * kRecF4;
             o[0] = r0; o[1] = r1; o[2] = r2;
             rect[e] = r;
-            zkey[e] = vis ? __float_as_uint(c.t[2]) : 0xFFFFFFFFu;
+            const uint32_t key = vis ? __float_as_uint(c.t[2]) : 0xFFFFFFFFu;
+            zkey[e] = key;
             zval[e] = (uint32_t)e;
             count[e] = vis ? (uint32_t)((r.z - r.x + 1) * (r.w - r.y + 1)) : 0u;
             nvis += vis ? 1u : 0u;
+            if (vis && !wsr) {
+#pragma unroll
+                for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p][(key >> (8 * p)) & 255u], 1u);
+            }
         }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nvis += __shfl_xor_sync(0xffffffffu, nvis, o);
     if ((threadIdx.x & 31) == 0 && nvis) atomicAdd(visible, nvis);
+    __syncthreads();
+    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) {
+        const uint32_t cnt = (&s_hist[0][0])[i];
+        if (cnt) atomicAdd(prep.hist + i, cnt);
+    }
 }
 
 __global__ void __launch_bounds__(128) k_project_fwd(const ViewDesc *__restrict__ views, int n_views, int slot,
@@ -212,10 +226,10 @@ void launch_cell_v_grad(const ViewDesc *views, int n_views, const SceneDev &sc, 
 
 void launch_gauss_bin(const ViewDesc *views, int n_views, const SceneDev &sc, const BlendParams &bp, bool wsr,
                       float tau, float4 *rec, uint32_t *zkey, uint32_t *zval, short4 *rect, uint32_t *count,
-                      uint32_t *visible, cudaStream_t st) {
-    if (sc.G == 0 || n_views == 0) return;
+                      uint32_t *visible, const BinPrep &prep, cudaStream_t st) {
+    if (n_views == 0) return;
     k_gauss_bin<<<grid_for(sc.G, 128), 128, 0, st>>>(views, n_views, sc, bp, wsr, tau, rec, zkey, zval, rect, count,
-                                                     visible);
+                                                     visible, prep);
 }
 
 void launch_project_fwd_table(const ViewDesc *views, const SceneDev *scenes, long long G_cap, const uint32_t *count,

@@ -29,6 +29,12 @@ constexpr int kSmallPairs = 3;    // L clamped to the pair capacity (captured ch
 constexpr int kSmallOverflow = 4; // L exceeded the pair capacity (captured chains)
 constexpr int kSmallWork = 5;     // work counter of the pulling blend (captured chains)
 constexpr int kSmallTcErr = 6;    // a tensor-core product's completion wait gave up (decode)
+// and after its first 64 words what the binning kernels need zeroed, so that one
+// memset clears all of it: partition counters of the depth sort, the tile sort (4
+// each) and the offsets' scan, and the two sorts' digit counts
+constexpr int kSmallCounters = 64, kSmallHist = 128;
+constexpr size_t kSmallBytes = 4 * (kSmallHist + 2 * 4 * 256);
+constexpr PairSlots kPairSlots{kSmallTotal, kSmallPairs, kSmallOverflow, kSmallSortErr};
 
 dgs_status set_error(dgs_status code, const std::string &msg);
 dgs_status cuda_error(cudaError_t e, const char *what);
@@ -50,6 +56,7 @@ struct DevBuf {
     int dev = 0;
     dgs_status ensure(size_t bytes);
     void release();
+    void swap(DevBuf &o);  // (both guarded or neither)
     ~DevBuf() { release(); }
 };
 
@@ -76,7 +83,7 @@ struct ChainView {
 // a pool and are reused once their `done` event has fired.
 struct Workspace {
     DevBuf views, scenes;
-    DevBuf zkey, zval, rect, depth, count, cnt_sorted, offs;  // per (view, cell)
+    DevBuf zkey, zval, rect, depth, count, offs;             // per (view, cell)
     DevBuf tkey, tval;                                       // per (tile, cell) pair
     DevBuf ranges;                                           // per tile
     DevBuf rec, g2d;                                         // per (view, Gaussian)
@@ -117,6 +124,13 @@ struct Workspace {
 
 dgs_status ensure_sort_scratch(Workspace &ws, long long n);
 SortScratch sort_scratch_of(Workspace &ws);
+// Of a chain's depth sort (0) or tile sort (1): counters and counts in ws.small.
+SortScratch chain_sort_scratch(Workspace &ws, int which);
+// What the binning kernel (0: cells or Gaussians, of n entries) or the emission (1: n
+// pairs) prepares for the sort that follows it.
+BinPrep chain_prep(Workspace &ws, int which, long long n, long long n_tiles);
+// Tile sort of a chain's L emitted pairs (d_L: their count on the device, L the capacity).
+void sort_tiles(Workspace &ws, long long L, int bits, const uint32_t *d_L, cudaStream_t st);
 BlendParams blend_params(const dgs_config &c);
 
 // ---------------------------------------------------------------- serving

@@ -112,7 +112,7 @@ dgs_status plan_batch(dgs_ctx *ctx, const std::vector<PendingReq> &reqs, BatchPl
 // Device bytes of a slot workspace with capacities c.
 long long slot_bytes(const ChainCaps &c) {
     const long long n = std::max(c.E, c.L);
-    return (long long)sizeof(ViewDesc) * c.V + (long long)sizeof(SceneDev) * c.S + 36 * c.E + 4 * c.E / 1024 +
+    return (long long)sizeof(ViewDesc) * c.V + (long long)sizeof(SceneDev) * c.S + 32 * c.E + 4 * c.E / 1024 +
            8 * n + 1024 * (n / 4096 + 1) + 8 * c.L + 8 * c.T + 48 * c.R + 20 * c.P +
            (c.W > 0 ? 4 * c.W + 4LL * kDecF * c.R : 0);
 }
@@ -182,9 +182,9 @@ dgs_status fit_slot(dgs_ctx *ctx, ServeState &S, GraphSlot &g, const BatchPlan &
     if (e != cudaSuccess) return cuda_error(e, "serving stream");
     Workspace &ws = *g.ws;
     if ((s = ws.views.ensure(sizeof(ViewDesc) * c.V)) || (s = ws.scenes.ensure(sizeof(SceneDev) * c.S)) ||
-        (s = ws.sizes.ensure(sizeof(ChainSizes))) || (s = ws.small.ensure(256)) || (s = ws.zkey.ensure(4 * c.E)) ||
+        (s = ws.sizes.ensure(sizeof(ChainSizes))) || (s = ws.small.ensure(kSmallBytes)) || (s = ws.zkey.ensure(4 * c.E)) ||
         (s = ws.zval.ensure(4 * c.E)) || (s = ws.rect.ensure(8 * c.E)) || (s = ws.depth.ensure(4 * c.E)) ||
-        (s = ws.count.ensure(4 * c.E)) || (s = ws.cnt_sorted.ensure(4 * c.E)) || (s = ws.offs.ensure(4 * c.E)) ||
+        (s = ws.count.ensure(4 * c.E)) || (s = ws.offs.ensure(4 * c.E)) ||
         (s = ws.scan.ensure(4 * scan_scratch_words(c.E))) || (s = ensure_sort_scratch(ws, std::max(c.E, c.L))) ||
         (s = ws.tkey.ensure(4 * c.L)) || (s = ws.tval.ensure(4 * c.L)) || (s = ws.ranges.ensure(8 * c.T)) ||
         (s = ws.rec.ensure(sizeof(float4) * kRecF4 * c.R)) || (s = ws.Dpix.ensure(4 * c.P)) ||
@@ -227,26 +227,26 @@ dgs_status record_chain(dgs_ctx *ctx, Workspace &ws, const ChainCaps &c, const B
     const uint32_t *d_E = (const uint32_t *)ws.sizes.p;  // ChainSizes::n_entries
     const uint32_t *d_L = small + kSmallPairs;
     const ViewDesc *dv = (const ViewDesc *)ws.views.p;
-    const SortScratch sc = sort_scratch_of(ws);
+    const uint32_t *d_vis = small + kSmallVisible;
     CKR(cudaMemcpyAsync(ws.views.p, ws.h_views, sizeof(ViewDesc) * c.V, cudaMemcpyHostToDevice, st));
     CKR(cudaMemcpyAsync(ws.scenes.p, ws.h_scenes, sizeof(SceneDev) * c.S, cudaMemcpyHostToDevice, st));
     CKR(cudaMemcpyAsync(ws.sizes.p, ws.h_sizes, sizeof(ChainSizes), cudaMemcpyHostToDevice, st));
-    CKR(cudaMemsetAsync(small, 0, 256, st));
+    CKR(cudaMemsetAsync(small, 0, kSmallBytes, st));
     launch_cell_project(dv, c.V, (const SceneDev *)ws.scenes.p, c.E, (uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p,
                         (short4 *)ws.rect.p, (float *)ws.depth.p, (uint32_t *)ws.count.p, small + kSmallVisible,
-                        (float *)ws.vview.p, ctx->cfg.flags, st, dsz);
-    radix_sort_pairs((uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p, c.E, 32, sc, st, d_E);
-    launch_gather_counts((const uint32_t *)ws.zval.p, (const uint32_t *)ws.count.p, c.E, (uint32_t *)ws.cnt_sorted.p,
-                         st, d_E);
-    exclusive_scan_u32((const uint32_t *)ws.cnt_sorted.p, (uint32_t *)ws.offs.p, c.E, small + kSmallTotal,
-                       (uint32_t *)ws.scan.p, st, d_E);
-    launch_clamp_pairs(small, kSmallTotal, kSmallPairs, kSmallOverflow, dsz, st);
-    launch_emit((const uint32_t *)ws.offs.p, (const uint32_t *)ws.zval.p, (const short4 *)ws.rect.p, dv, c.V, c.E,
-                c.L, (uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, st, dsz, d_L);
+                        (float *)ws.vview.p, ctx->cfg.flags, chain_prep(ws, 0, c.E, c.T), st, dsz);
+    radix_sort_counted((uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p, c.E, 32, chain_sort_scratch(ws, 0), st, d_E, d_vis,
+                       false);
+    launch_pair_offsets((const uint32_t *)ws.zval.p, (const uint32_t *)ws.count.p, c.E, d_E, d_vis,
+                        (uint32_t *)ws.offs.p, (uint32_t *)ws.scan.p, small + kSmallCounters + 8, small, kPairSlots, 0,
+                        dsz, st);
     int bits = 1;
     while ((1LL << bits) < c.T) ++bits;
-    radix_sort_pairs((uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, c.L, bits, sc, st, d_L);
-    CKR(cudaMemsetAsync(ws.ranges.p, 0, 8 * (size_t)c.T, st));
+    launch_emit((const uint32_t *)ws.offs.p, (const uint32_t *)ws.zval.p, (const short4 *)ws.rect.p, dv, c.V, c.E, c.E,
+                c.L, (int)c.T, (uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, (bits + 7) / 8, chain_prep(ws, 1, c.L, 0),
+                st, dsz, d_vis, d_L);
+    radix_sort_counted((uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, c.L, bits, chain_sort_scratch(ws, 1), st, d_L,
+                       nullptr, true);
     launch_tile_ranges((const uint32_t *)ws.tkey.p, c.L, (uint2 *)ws.ranges.p, st, d_L);
     // neural scenes: the decode writes their records (slot k's samples of the
     // visible entries, counted on the device); the table projection skips them

@@ -233,6 +233,28 @@ def test_radix_sort_pairs_stable(rctx, n, bits):
     assert np.array_equal(kd.cpu().numpy(), k32.numpy()[order])
 
 
+@pytest.mark.parametrize("n", [2, 1023, 1024, 1025, 9 * 1024 + 1, 65536, 65537])
+def test_radix_sort_partition_edges(rctx, n):
+    """Around a small partition, one look-back of eight partitions, and the
+    size at which the partitions grow."""
+    test_radix_sort_pairs_stable(rctx, n, 32)
+
+
+@pytest.mark.parametrize("n_cells", [1, 1023, 2048, 2049, 70_000])
+def test_binning_with_most_cells_culled(rctx, n_cells):
+    """The depth sort leaves the culled cells out: entry counts around a scan
+    partition and a sort partition, a camera inside the scene."""
+    sc = synth.make_scene(n_cells, 1, synth._box(-1, 1), 0.002, 0.1, 0, seed=n_cells)
+    cams = [synth.look_at((0.1, 0.0, 0.0), (1.0, 0.2, 0.1), 64, 48, 60.0), synth.small_camera(40, 56)]
+    _render_and_check(rctx, sc, cams)
+
+
+def test_more_than_65536_tiles(rctx):
+    """An odd number of tile-sort passes (17 bits of tile number)."""
+    sc = synth.scene_small(n_cells=400)
+    _render_and_check(rctx, sc, [synth.small_camera(4112, 4112)], tile_rows=(128, 130))
+
+
 def test_loss_l1_matches_definition(rctx):
     g = torch.Generator().manual_seed(0)
     a = torch.rand(1_000_003, generator=g).cuda()
