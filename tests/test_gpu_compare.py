@@ -62,6 +62,24 @@ def test_alpha_blend_matches_oracle(rctx, sh):
         rctx.release_scene(sid)
 
 
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 64, 97])
+def test_alpha_blend_batch_edges(rctx, n):
+    """Lists around one and two batches of 32: all n Gaussians reach every pixel
+    of a small image, whose right and lower edges cut sub-tiles."""
+    sc = synth.make_scene(n, 1, synth._box(-0.2, 0.2), 1.0, 1.5, 0, seed=n)
+    sc.g_logit[:] -= 2.0
+    sid = rctx.upload_scene(sc)
+    try:
+        for cam in (synth.small_camera(23, 13), synth.small_camera(16, 9)):
+            img, nd, _ = rctx.render_compare(sid, [cam], "alpha", want_ndone=True)
+            _alpha_check(sc, cam, img.cpu().numpy(), nd.cpu().numpy())
+            img, _, _ = rctx.render_compare(sid, [cam], "wsr")
+            ref = oracle.render_wsr(sc, cam.as_array())
+            assert np.abs(img.cpu().numpy().reshape(3, cam.H, cam.W) - ref["C"]).max() <= IMG_TOL
+    finally:
+        rctx.release_scene(sid)
+
+
 def test_alpha_blend_terminates(rctx):
     # an opaque scene: many pixels stop early, the counts still validate
     s = synth.scene_small(seed=2, n_cells=4000)
