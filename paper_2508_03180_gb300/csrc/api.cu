@@ -354,12 +354,12 @@ static const void *mapped_host(const void *h) {
 }
 
 // One parameter array (rows x cols, row-major, in `location` memory) into
-// its structure-of-arrays planes.  Mapped host arrays are read by the
-// transposing kernel over the host link; other host arrays go through
-// `stage` (device, rows x cols floats).  The caller synchronises before the
-// host memory or the staging is reused.
+// its structure-of-arrays planes, as one of the launch's copies.  Mapped host
+// arrays are read by the transposing kernel over the host link; other host arrays
+// go through `stage` (device, rows x cols floats).  The caller synchronises before
+// the host memory or the staging is reused.
 static dgs_status upload_param(const float *src, int location, int64_t rows, int cols, float *dst_planes,
-                               int64_t plane_stride, float *stage, cudaStream_t st) {
+                               int64_t plane_stride, float *stage, PlaneCopies &copies, cudaStream_t st) {
     const size_t bytes = sizeof(float) * (size_t)rows * cols;
     if (bytes == 0) return DGS_OK;
     const float *dsrc = src;
@@ -371,8 +371,7 @@ static dgs_status upload_param(const float *src, int location, int64_t rows, int
             dsrc = stage;
         }
     }
-    launch_aos_to_soa(dsrc, rows, cols, dst_planes, plane_stride, st);
-    CK(cudaGetLastError());
+    copies.add(dsrc, rows, cols, dst_planes, plane_stride);
     return DGS_OK;
 }
 
@@ -421,13 +420,15 @@ static dgs_status fill_scene(dgs_ctx *ctx, Scene &sc, const dgs_scene_desc *d, c
         }
     }
     if (!d->cell_v && cells_too) launch_fill_f32(cell + 10 * N, N, 1.0f, st);
+    PlaneCopies copies;
     for (auto &p : parts) {
         if (!p.src) continue;
         const bool staged = d->location == DGS_HOST && !mapped_host(p.src);
-        dgs_status s = upload_param(p.src, d->location, p.rows, p.cols, p.dst, p.stride, stage, st);
+        dgs_status s = upload_param(p.src, d->location, p.rows, p.cols, p.dst, p.stride, stage, copies, st);
         if (s) return s;
         if (staged) stage += p.rows * p.cols;
     }
+    launch_rows_to_planes(copies, st);
     CK(cudaGetLastError());
     if (d->location == DGS_HOST) CK(cudaStreamSynchronize(st));  // host arrays and staging free again
     return DGS_OK;

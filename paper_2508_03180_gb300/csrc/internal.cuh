@@ -257,8 +257,23 @@ void launch_count_pairs(const ViewDesc *views, int n_views, int total_tiles, con
                         cudaStream_t st);
 
 // misc.cu
-void launch_aos_to_soa(const float *src, int64_t rows, int cols, float *dst, int64_t dst_stride,
-                       cudaStream_t st);
+// Arrays [rows][cols] (at most 64 columns, or one row) that one launch turns into planes.
+struct PlaneCopy {
+    const float *src;
+    float *dst;
+    int64_t rows, stride, first_task;
+    int cols;
+};
+struct PlaneCopies {
+    static constexpr int kMax = 12;
+    PlaneCopy a[kMax];
+    int n = 0;
+    int64_t tasks = 0;
+    void add(const float *src, int64_t rows, int cols, float *dst, int64_t stride);
+};
+// rows of a tile: about 4096 elements in 32-row groups
+__host__ __device__ constexpr int plane_tile_rows(int cols) { return 4096 / cols / 32 * 32; }
+void launch_rows_to_planes(const PlaneCopies &c, cudaStream_t st);
 void launch_soa_to_aos(const float *src, int64_t rows, int cols, int64_t src_stride, float *dst,
                        cudaStream_t st);
 void launch_fill_f32(float *dst, int64_t n, float v, cudaStream_t st);

@@ -249,6 +249,32 @@ def test_binning_with_most_cells_culled(rctx, n_cells):
     _render_and_check(rctx, sc, cams)
 
 
+@pytest.mark.parametrize("n_cells,sh,offset", [(1, 0, 0), (21, 1, 1), (64, 2, 2), (65, 3, 3), (683, 3, 0)])
+def test_update_from_arrays_at_any_alignment(rctx, n_cells, sh, offset):
+    """The rows become planes whatever the arrays' widths, row counts (tiles of
+    64 rows and more) and alignment: the updated scene renders as the uploaded one."""
+    sc = synth.make_scene(n_cells, 3, synth._box(-1, 1), 0.1, 0.4, sh, seed=n_cells)
+    other = synth.make_scene(n_cells, 3, synth._box(-1, 1), 0.1, 0.4, sh, seed=n_cells)
+    for a in (other.g_mean, other.g_scale, other.g_quat, other.g_logit, other.g_sh):
+        a[:] = 0.5
+    cam = synth.small_camera(96, 80)
+
+    def shifted(a):
+        buf = torch.empty(a.size + 8, device="cuda")
+        t = buf[offset:offset + a.size].view(a.shape)
+        t.copy_(torch.from_numpy(np.ascontiguousarray(a)))
+        return t
+
+    sid, oid = rctx.upload_scene(sc), rctx.upload_scene(other)
+    ref = rctx.render(sid, [cam])[0].clone()
+    rctx.update_scene(oid, sc.N, sc.K, sh, **{k: shifted(getattr(sc, k)) for k in
+                                              ("g_mean", "g_scale", "g_quat", "g_logit", "g_sh")})
+    img = rctx.render(oid, [cam])[0]
+    assert torch.equal(img, ref)
+    rctx.release_scene(sid)
+    rctx.release_scene(oid)
+
+
 def test_more_than_65536_tiles(rctx):
     """An odd number of tile-sort passes (17 bits of tile number)."""
     sc = synth.scene_small(n_cells=400)
