@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(EM_THREADS) k_emit(const uint32_t *__restrict_
     __shared__ long long s_own[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i < passes * 256; i += EM_THREADS) (&s_hist[0][0])[i] = 0u;
+    chain_begin();
     prep_clear(prep, blockIdx.x * (long long)EM_THREADS + tid, (long long)gridDim.x * EM_THREADS);
     if (dsz) {
         n_views = dsz->n_views;
@@ -308,7 +309,7 @@ void launch_emit(const uint32_t *offs, const uint32_t *zval_sorted, const short4
     if (L == 0) return;
     // eight blocks an SM at most: each adds its digit counts to the global ones once
     const long long runs = (L + EM_TB - 1) / EM_TB;
-    k_emit<<<(unsigned)std::min<long long>(runs, 152 * 8), EM_THREADS, 0, st>>>(
+    launch_chained(k_emit, (unsigned)std::min<long long>(runs, 152 * 8), EM_THREADS, 0, st,
         offs, zval_sorted, rect, views, n_views, n_entries, n_all, L, n_tiles, tkey, tval, passes, prep, dsz, d_n, d_L);
 }
 
@@ -316,6 +317,7 @@ void launch_emit(const uint32_t *offs, const uint32_t *zval_sorted, const short4
 // tiles keep the (0,0) the caller cleared them to.
 __global__ void k_tile_ranges(const uint32_t *__restrict__ key, long long L, const uint32_t *__restrict__ d_L,
                               uint2 *__restrict__ ranges) {
+    chain_begin();
     if (d_L) L = *d_L;
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < L; j += (long long)gridDim.x * blockDim.x) {
         const uint32_t k = key[j];
@@ -327,7 +329,7 @@ __global__ void k_tile_ranges(const uint32_t *__restrict__ key, long long L, con
 void launch_tile_ranges(const uint32_t *tkey_sorted, long long L, uint2 *ranges, cudaStream_t st,
                         const uint32_t *d_L) {
     if (L == 0) return;
-    k_tile_ranges<<<grid_for(L, 256), 256, 0, st>>>(tkey_sorted, L, d_L, ranges);
+    launch_chained(k_tile_ranges, grid_for(L, 256), 256, 0, st, tkey_sorted, L, d_L, ranges);
 }
 
 }  // namespace dgs

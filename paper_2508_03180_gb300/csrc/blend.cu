@@ -293,6 +293,7 @@ __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd(const ViewDesc 
                                                   float *__restrict__ out_rgb, float *__restrict__ out_rgb2,
                                                   float *__restrict__ out_D, int *__restrict__ out_nd) {
     __shared__ float4 s_rec[FSTAGE][kBatchF4];
+    chain_begin();
     blend_fwd_unit<KT, FWD_PPL, VAR>(blockIdx.x, views, n_views, ranges, cells, rec, bp, out_rgb, out_rgb2, out_D, out_nd,
                                 s_rec);
 }
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd_pull(const View
                                                        int *__restrict__ out_nd, const ChainSizes *__restrict__ dsz,
                                                        uint32_t *__restrict__ work) {
     __shared__ float4 s_rec[FSTAGE][kBatchF4];
+    chain_begin();
     const int n_views = dsz->n_views;
     const uint32_t units = (uint32_t)dsz->total_tiles * FWD_SUB;
     for (;;) {
@@ -348,8 +350,8 @@ void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const
     if (dsz) {
         // exactly the resident warps
 #define DGS_PULL(KV, VV)                                                                                     \
-        k_blend_fwd_pull<KV, VV><<<pull_grid<KV, VV>(total_tiles), WT, 0, st>>>(views, ranges, tile_cells, rec, bp, \
-                                                                               out_rgb, out_D, out_nd, dsz, work)
+        launch_chained(k_blend_fwd_pull<KV, VV>, pull_grid<KV, VV>(total_tiles), WT, 0, st, views, ranges, tile_cells, \
+                       rec, bp, out_rgb, out_D, out_nd, dsz, work)
         if (blend_variants(bp)) {
             switch (K_all) {
                 case 8: DGS_PULL(8, true); break;
@@ -368,8 +370,8 @@ void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const
     }
     const unsigned grid = (unsigned)total_tiles * FWD_SUB;
 #define DGS_FWD(KV, VV)                                                                                      \
-    k_blend_fwd<KV, VV><<<grid, WT, 0, st>>>(views, n_views, ranges, tile_cells, rec, bp, out_rgb, out_rgb2, out_D, \
-                                             out_nd)
+    launch_chained(k_blend_fwd<KV, VV>, grid, WT, 0, st, views, n_views, ranges, tile_cells, rec, bp, out_rgb, out_rgb2, \
+                   out_D, out_nd)
     if (blend_variants(bp)) {
         switch (K_all) {
             case 8: DGS_FWD(8, true); break;
@@ -906,6 +908,7 @@ void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, int K
     if (total_tiles == 0) return;
     const unsigned grid = (unsigned)total_tiles * BWD_SUB;
     const size_t smem = sizeof(float4) * bwd_smem_f4(K_all);
+    // (a plain launch: chained to its successor it took 0.5% longer on the 1M-Gaussian step)
 #define DGS_BWD(KV, VV)                                                                                          \
     do {                                                                                                        \
         if (g_cell_v)                                                                                           \

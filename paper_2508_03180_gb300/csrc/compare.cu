@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restri
                                                     const float4 *__restrict__ rec, BlendParams bp, float w_bg,
                                                     float *__restrict__ out_rgb, int *__restrict__ out_nd) {
     __shared__ float4 s_rec[FSTAGE][kBatchF4];
+    chain_begin();
     constexpr int NR = 2, NB = batch_cells(1);
     const int lane = threadIdx.x;
     const int tile = blockIdx.x / CSUB, sub = blockIdx.x % CSUB;
@@ -233,10 +234,10 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
     if (tiles > 0) {
         const unsigned grid = (unsigned)tiles * CSUB;
         if (wsr)
-            k_gauss_blend<false><<<grid, CT, 0, st>>>(dv, V, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
+            launch_chained(k_gauss_blend<false>, grid, CT, 0, st, dv, V, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
                                                       (const float4 *)ws.rec.p, bp, cfg.w_bg, out_img, nullptr);
         else
-            k_gauss_blend<true><<<grid, CT, 0, st>>>(dv, V, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
+            launch_chained(k_gauss_blend<true>, grid, CT, 0, st, dv, V, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
                                                      (const float4 *)ws.rec.p, bp, 0.f, out_img, out_nd);
     }
     CK(cudaGetLastError());

@@ -291,6 +291,36 @@ long long resident_ctas(const void *kernel, int threads);
 cudaError_t set_sort_fault(bool on);
 cudaError_t set_tc_fault(bool on);  // the tensor-core decode's completion wait runs out (DGS_FAULT_TC_WAIT)
 
+// Programmatic dependent launch: a kernel launched by launch_chained may begin while
+// its predecessor in the stream still runs, as soon as all of that one's blocks
+// have started, so its launch latency and block start-up overlap the
+// predecessor's tail (views: 256 x 256 134 -> 125 us, 1080p 488 -> 469, neural 720p
+// 330 -> 310).  Every such kernel calls chain_begin before it touches
+// global memory: it waits there until the predecessor has
+// completed and its writes are visible, and lets its own successor be launched.
+// Not within a captured graph, whose own edges are cheap already (a served burst
+// of eight requests: 881 us plain, 917 us chained).
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A &&...a) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &capture);
+    c.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, static_cast<P>(a)...);
+}
+
 // Clear the words of a BinPrep (all threads of the grid).
 __device__ __forceinline__ void prep_clear(const BinPrep &p, long long thread, long long threads) {
     for (long long i = thread; i < p.status_words; i += threads) p.status[i] = 0u;

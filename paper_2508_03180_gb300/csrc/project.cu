@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(128) k_project_fwd(const ViewDesc *__restrict_
                                                      SceneDev sc, const uint32_t *__restrict__ count,
                                                      const float *__restrict__ vview, BlendParams bp,
                                                      float4 *__restrict__ rec, float *__restrict__ g2d_zero) {
+    chain_begin();
     project_scene(views, n_views, slot, sc, count, vview, bp, rec, g2d_zero);
 }
 
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(128) k_project_fwd_table(const ViewDesc *__res
                                                            const float *__restrict__ vview, BlendParams bp,
                                                            float4 *__restrict__ rec,
                                                            const ChainSizes *__restrict__ dsz) {
+    chain_begin();
     const int n_views = dsz->n_views, n_scenes = dsz->n_scenes;
     for (int s = 0; s < n_scenes; ++s) {
         const SceneDev sc = scenes[s];
@@ -215,7 +217,7 @@ static int grid_for(long long n, int threads) {
 void launch_project_fwd(const ViewDesc *views, int n_views, int slot, const SceneDev &sc, const uint32_t *count,
                         const float *vview, const BlendParams &bp, float4 *rec, float *g2d_zero, cudaStream_t st) {
     if (sc.G == 0 || n_views == 0) return;
-    k_project_fwd<<<grid_for(sc.G, 128), 128, 0, st>>>(views, n_views, slot, sc, count, vview, bp, rec, g2d_zero);
+    launch_chained(k_project_fwd, grid_for(sc.G, 128), 128, 0, st, views, n_views, slot, sc, count, vview, bp, rec, g2d_zero);
 }
 
 void launch_cell_v_grad(const ViewDesc *views, int n_views, const SceneDev &sc, const float *gv, float *g_cell_v,
@@ -236,7 +238,7 @@ void launch_project_fwd_table(const ViewDesc *views, const SceneDev *scenes, lon
                               const float *vview, const BlendParams &bp, float4 *rec, cudaStream_t st,
                               const ChainSizes *dsz) {
     if (G_cap == 0) return;
-    k_project_fwd_table<<<grid_for(G_cap, 128), 128, 0, st>>>(views, scenes, count, vview, bp, rec, dsz);
+    launch_chained(k_project_fwd_table, grid_for(G_cap, 128), 128, 0, st, views, scenes, count, vview, bp, rec, dsz);
 }
 
 // a*b - c*d to about one rounding (Kahan's compensated form)
@@ -399,6 +401,7 @@ __global__ void __launch_bounds__(128) k_project_bwd_geom(const ViewDesc *__rest
                                                      float *__restrict__ g_scale,
                                                      float *__restrict__ g_log_scale, float *__restrict__ g_quat,
                                                      float *__restrict__ g_logit) {
+    chain_begin();
     const long long G = sc.G;
     const int K = sc.K;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < G; g += (long long)gridDim.x * blockDim.x) {
@@ -525,6 +528,7 @@ __global__ void __launch_bounds__(COL_T) k_project_bwd_colour(const ViewDesc *__
                                                               const float *__restrict__ g2d, float *__restrict__ g_mean,
                                                               float *__restrict__ g_sh) {
     __shared__ float s_acc[48 * COL_LD];  // dL/dk[c * 3 + ch] of thread t at [c * 3 + ch][t]
+    chain_begin();
     const long long G = sc.G;
     const int K = sc.K, C = (sc.sh_degree + 1) * (sc.sh_degree + 1), row = 3 * C;
     const int t = threadIdx.x;
@@ -630,10 +634,10 @@ void launch_project_bwd(const ViewDesc *views, int n_views, int slot, const Scen
                         const BlendParams &bp, const float *g2d, float *g_mean, float *g_scale, float *g_log_scale,
                         float *g_quat, float *g_logit, float *g_sh, cudaStream_t st) {
     if (sc.G == 0) return;
-    k_project_bwd_geom<<<grid_for(sc.G, 128), 128, 0, st>>>(views, n_views, slot, sc, count, bp, g2d, g_mean,
+    launch_chained(k_project_bwd_geom, grid_for(sc.G, 128), 128, 0, st, views, n_views, slot, sc, count, bp, g2d, g_mean,
                                                             g_scale, g_log_scale, g_quat, g_logit);
     if (g_mean || g_sh)
-        k_project_bwd_colour<<<grid_for(sc.G, 128), 128, 0, st>>>(views, n_views, slot, sc, count, g2d, g_mean, g_sh);
+        launch_chained(k_project_bwd_colour, grid_for(sc.G, 128), 128, 0, st, views, n_views, slot, sc, count, g2d, g_mean, g_sh);
 }
 
 }  // namespace dgs

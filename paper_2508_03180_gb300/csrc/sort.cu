@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_pass(uint32_t *__restrict__ k
     __shared__ uint32_t s_key[TILE], s_val[TILE];  // the partition in digit order
     __shared__ uint32_t s_part, s_cnt;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_begin();
     if (d_n) n = *d_n;
     const bool drop = d_live && pass == 0;
     if (d_live && pass > 0) n = *d_live;
@@ -282,12 +283,11 @@ static bool radix_passes(uint32_t *keys, uint32_t *vals, long long n, int passes
     const unsigned grid = (unsigned)std::min(parts, resident_ctas(kernel, RS_THREADS));
     for (int p = 0; p < passes; ++p) {
         if (small)
-            k_rs_pass<RS_ITEMS_SMALL><<<grid, RS_THREADS, 0, st>>>(keys, vals, s.keys_alt, s.vals_alt, n, d_n, d_live, p,
-                                                                  s.hist, skip, status[0], status[1], s.counters + p,
-                                                                  s.err);
+            launch_chained(k_rs_pass<RS_ITEMS_SMALL>, grid, RS_THREADS, 0, st, keys, vals, s.keys_alt, s.vals_alt, n, d_n,
+                           d_live, p, s.hist, skip, status[0], status[1], s.counters + p, s.err);
         else
-            k_rs_pass<RS_ITEMS><<<grid, RS_THREADS, 0, st>>>(keys, vals, s.keys_alt, s.vals_alt, n, d_n, d_live, p,
-                                                            s.hist, skip, status[0], status[1], s.counters + p, s.err);
+            launch_chained(k_rs_pass<RS_ITEMS>, grid, RS_THREADS, 0, st, keys, vals, s.keys_alt, s.vals_alt, n, d_n, d_live, p,
+                           s.hist, skip, status[0], status[1], s.counters + p, s.err);
     }
     if (!skip) return passes & 1;
     k_copy_pairs<<<152 * 2, 256, 0, st>>>(s.keys_alt, s.vals_alt, keys, vals, n, d_n, s.hist, passes);
@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_pair_offsets(const uint32_t *__r
     constexpr unsigned long long AGG = 1ull << 32, INC = 2ull << 32;
     __shared__ uint32_t s_warp[SC_THREADS / 32], s_part, s_excl;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_begin();
     if (d_all) n_all = *d_all;
     const long long n = d_n ? (long long)*d_n : n_all;
     const long long n_parts = (n + SC_TILE - 1) / SC_TILE;
@@ -428,8 +429,8 @@ void launch_pair_offsets(const uint32_t *idx, const uint32_t *count, long long n
     if (n == 0) return;
     const long long parts = (n + SC_TILE - 1) / SC_TILE;
     const unsigned grid = (unsigned)std::min(parts, resident_ctas((const void *)k_pair_offsets, SC_THREADS));
-    k_pair_offsets<<<grid, SC_THREADS, 0, st>>>(idx, count, n, d_all, d_n, offs, (unsigned long long *)scratch, counter,
-                                                small, slots, cap, dsz);
+    launch_chained(k_pair_offsets, grid, SC_THREADS, 0, st, idx, count, n, d_all, d_n, offs, (unsigned long long *)scratch,
+                   counter, small, slots, cap, dsz);
 }
 
 }  // namespace dgs
