@@ -141,7 +141,7 @@ Workspace::~Workspace() {
 }
 
 std::vector<DevBuf *> Workspace::all() {
-    return {&views, &scenes, &zkey, &zval, &rect, &depth, &count, &offs, &tkey, &tval, &ranges, &rec,
+    return {&views, &scenes, &zkey, &zval, &rect, &depth, &count, &offs, &tkey, &tval, &ranges, &order, &rec,
             &Dpix, &ndpix, &rgb, &g2d, &gstage, &sort_k, &sort_v, &sort_hist, &sort_status, &sort_ctr, &small, &scan, &sizes, &vview, &gvview, &dec};
 }
 
@@ -830,7 +830,8 @@ static dgs_status run_binning(dgs_ctx *ctx, Workspace &ws, cudaStream_t st, bool
     if ((s = ws.zkey.ensure(4 * n1)) || (s = ws.zval.ensure(4 * n1)) || (s = ws.rect.ensure(8 * n1)) ||
         (s = ws.depth.ensure(4 * n1)) || (s = ws.count.ensure(4 * n1)) || (s = ws.offs.ensure(4 * n1)) ||
         (s = ws.scan.ensure(4 * scan_scratch_words(n1))) || (s = ws.vview.ensure(4 * n1)) ||
-        (s = ws.ranges.ensure(8 * (size_t)std::max(1, ws.total_tiles))))
+        (s = ws.ranges.ensure(8 * (size_t)std::max(1, ws.total_tiles))) ||
+        (s = ws.order.ensure(4 * (size_t)std::max(1, ws.total_tiles))))
         return s;
     if ((s = ensure_sort_scratch(ws, n))) return s;
     // a device-sized chain sizes every buffer before its first launch, so no
@@ -893,6 +894,7 @@ static dgs_status run_binning(dgs_ctx *ctx, Workspace &ws, cudaStream_t st, bool
     {
         StageTimer t(pf, DGS_STAGE_TILE_RANGES, st);
         launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, st, d_L);
+        launch_tile_order((const uint2 *)ws.ranges.p, ws.total_tiles, (uint32_t *)ws.order.p, st);
     }
     CK(cudaGetLastError());
     if (device_sized) ws.async_pending = true;
@@ -991,7 +993,7 @@ dgs_status chain_forward(dgs_ctx *ctx, Workspace &ws, const std::vector<ChainVie
         int K_all = slots[0]->K;
         for (int k = 1; k < S; ++k)
             if (slots[k]->K != K_all) K_all = 0;
-        launch_blend_fwd(dv, V, ws.total_tiles, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
+        launch_blend_fwd(dv, V, ws.total_tiles, (const uint32_t *)ws.order.p, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
                          (const float4 *)ws.rec.p, bp, img, img2, (float *)ws.Dpix.p, (int *)ws.ndpix.p, K_all, st);
     }
     CK(cudaGetLastError());
@@ -1163,7 +1165,8 @@ extern "C" dgs_status dgs_render_backward(dgs_ctx *ctx, dgs_fwd_state *state, co
     }
     {
         StageTimer t(ctx->prof, DGS_STAGE_BLEND_BWD, st);
-        launch_blend_bwd((const ViewDesc *)ws.views.p, ws.V, ws.total_tiles, sc.K, (const uint2 *)ws.ranges.p,
+        launch_blend_bwd((const ViewDesc *)ws.views.p, ws.V, ws.total_tiles, (const uint32_t *)ws.order.p, sc.K,
+                         (const uint2 *)ws.ranges.p,
                          (const uint32_t *)ws.tval.p, (const float4 *)ws.rec.p, bp, (const float *)ws.rgb.p,
                          (const float *)ws.Dpix.p, (const int *)ws.ndpix.p, dl, (float *)ws.g2d.p, gv, st);
         if (gv) launch_cell_v_grad((const ViewDesc *)ws.views.p, ws.V, sc.dev(), gv, o_v, o_vsh, o_cc, st);

@@ -93,6 +93,7 @@ constexpr int fwd_minb(bool var) { return var ? 24 : 32; }  // (the variants spi
 // w_bg); without it the kernels are the paper's reading with no check left.
 template <int KT, int PPL, bool VAR>
 __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restrict__ views, int n_views,
+                                               const uint32_t *__restrict__ order,
                                                const uint2 *__restrict__ ranges, const uint32_t *__restrict__ cells,
                                                const float4 *__restrict__ rec, const BlendParams &bp,
                                                float *__restrict__ out_rgb, float *__restrict__ out_rgb2,
@@ -100,7 +101,7 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
                                                float4 (*s_rec)[kBatchF4]) {
     constexpr int ROWS = 2 * PPL, NSUB = kTile / ROWS;
     const int lane = threadIdx.x;
-    const int tile = unit / NSUB, sub = unit % NSUB;
+    const int tile = (int)order[unit / NSUB], sub = unit % NSUB;
     const int vi = find_view(views, n_views, tile);
     const ViewDesc &V = views[vi];
     const int local = tile - V.tile_base;
@@ -288,13 +289,14 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
 
 template <int KT, bool VAR>
 __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd(const ViewDesc *__restrict__ views, int n_views,
+                                                  const uint32_t *__restrict__ order,
                                                   const uint2 *__restrict__ ranges, const uint32_t *__restrict__ cells,
                                                   const float4 *__restrict__ rec, BlendParams bp,
                                                   float *__restrict__ out_rgb, float *__restrict__ out_rgb2,
                                                   float *__restrict__ out_D, int *__restrict__ out_nd) {
     __shared__ float4 s_rec[FSTAGE][kBatchF4];
     chain_begin();
-    blend_fwd_unit<KT, FWD_PPL, VAR>(blockIdx.x, views, n_views, ranges, cells, rec, bp, out_rgb, out_rgb2, out_D, out_nd,
+    blend_fwd_unit<KT, FWD_PPL, VAR>(blockIdx.x, views, n_views, order, ranges, cells, rec, bp, out_rgb, out_rgb2, out_D, out_nd,
                                 s_rec);
 }
 
@@ -305,6 +307,7 @@ __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd(const ViewDesc 
 // atomic per sub-tile: their rate is bounded by the blend work between them.
 template <int KT, bool VAR>
 __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd_pull(const ViewDesc *__restrict__ views,
+                                                       const uint32_t *__restrict__ order,
                                                        const uint2 *__restrict__ ranges,
                                                        const uint32_t *__restrict__ cells,
                                                        const float4 *__restrict__ rec, BlendParams bp,
@@ -320,7 +323,7 @@ __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd_pull(const View
         if (threadIdx.x == 0) u = atomicAdd(work, 1u);
         u = __shfl_sync(0xffffffffu, u, 0);
         if (u >= units) break;
-        blend_fwd_unit<KT, FWD_PPL, VAR>((int)u, views, n_views, ranges, cells, rec, bp, out_rgb, nullptr, out_D, out_nd,
+        blend_fwd_unit<KT, FWD_PPL, VAR>((int)u, views, n_views, order, ranges, cells, rec, bp, out_rgb, nullptr, out_D, out_nd,
                                     s_rec);
         __syncwarp();
     }
@@ -342,7 +345,7 @@ static unsigned pull_grid(int total_tiles) {
     return (unsigned)std::min<long long>((long long)total_tiles * FWD_SUB, per_grid);
 }
 
-void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const uint2 *ranges,
+void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const uint32_t *order, const uint2 *ranges,
                       const uint32_t *tile_cells, const float4 *rec, const BlendParams &bp, float *out_rgb,
                       float *out_rgb2, float *out_D, int *out_nd, int K_all, cudaStream_t st,
                       const ChainSizes *dsz, uint32_t *work) {
@@ -350,7 +353,7 @@ void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const
     if (dsz) {
         // exactly the resident warps
 #define DGS_PULL(KV, VV)                                                                                     \
-        launch_chained(k_blend_fwd_pull<KV, VV>, pull_grid<KV, VV>(total_tiles), WT, 0, st, views, ranges, tile_cells, \
+        launch_chained(k_blend_fwd_pull<KV, VV>, pull_grid<KV, VV>(total_tiles), WT, 0, st, views, order, ranges, tile_cells, \
                        rec, bp, out_rgb, out_D, out_nd, dsz, work)
         if (blend_variants(bp)) {
             switch (K_all) {
@@ -370,7 +373,7 @@ void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const
     }
     const unsigned grid = (unsigned)total_tiles * FWD_SUB;
 #define DGS_FWD(KV, VV)                                                                                      \
-    launch_chained(k_blend_fwd<KV, VV>, grid, WT, 0, st, views, n_views, ranges, tile_cells, rec, bp, out_rgb, out_rgb2, \
+    launch_chained(k_blend_fwd<KV, VV>, grid, WT, 0, st, views, n_views, order, ranges, tile_cells, rec, bp, out_rgb, out_rgb2, \
                    out_D, out_nd)
     if (blend_variants(bp)) {
         switch (K_all) {
@@ -607,6 +610,7 @@ __host__ __device__ constexpr int bwd_smem_f4(int K) {
 
 template <int KT, bool VAR, bool WV>
 __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *__restrict__ views, int n_views,
+                                                  const uint32_t *__restrict__ order,
                                                   const uint2 *__restrict__ ranges, const uint32_t *__restrict__ cells,
                                                   const float4 *__restrict__ rec, BlendParams bp,
                                                   const float *__restrict__ rgb, const float *__restrict__ Dpix,
@@ -614,7 +618,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
                                                   float *__restrict__ g2d, float *__restrict__ g_cell_v) {
     extern __shared__ float4 s_bwd[];
     const int lane = threadIdx.x;
-    const int tile = blockIdx.x / BWD_SUB, sub = blockIdx.x % BWD_SUB;
+    const int tile = (int)order[blockIdx.x / BWD_SUB], sub = blockIdx.x % BWD_SUB;
     const int vi = find_view(views, n_views, tile);
     const ViewDesc &V = views[vi];
     const int K = KT > 0 ? KT : V.K;
@@ -901,7 +905,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
 }
 
 // K_all: K of the chain's scene (compile-time loop for common values; sizes the shared memory)
-void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, int K_all, const uint2 *ranges,
+void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, const uint32_t *order, int K_all, const uint2 *ranges,
                       const uint32_t *tile_cells, const float4 *rec, const BlendParams &bp, const float *rgb,
                       const float *D, const int *nd, const float *dL_drgb, float *g2d, float *g_cell_v,
                       cudaStream_t st) {
@@ -912,10 +916,10 @@ void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, int K
 #define DGS_BWD(KV, VV)                                                                                          \
     do {                                                                                                        \
         if (g_cell_v)                                                                                           \
-            k_blend_bwd<KV, VV, true><<<grid, WT, smem, st>>>(views, n_views, ranges, tile_cells, rec, bp, rgb, D, nd, \
+            k_blend_bwd<KV, VV, true><<<grid, WT, smem, st>>>(views, n_views, order, ranges, tile_cells, rec, bp, rgb, D, nd, \
                                                               dL_drgb, g2d, g_cell_v);                          \
         else                                                                                                    \
-            k_blend_bwd<KV, VV, false><<<grid, WT, smem, st>>>(views, n_views, ranges, tile_cells, rec, bp, rgb, D, nd, \
+            k_blend_bwd<KV, VV, false><<<grid, WT, smem, st>>>(views, n_views, order, ranges, tile_cells, rec, bp, rgb, D, nd, \
                                                                dL_drgb, g2d, nullptr);                          \
     } while (0)
     if (blend_variants(bp)) {

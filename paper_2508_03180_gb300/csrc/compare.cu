@@ -35,6 +35,7 @@ constexpr int CSUB = kTile / CROWS;  // sub-tiles per tile
 // 1M Gaussians, 3.1M of them in tile lists twice (the whole call 992 -> 840 us).
 template <bool ALPHA>
 __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restrict__ views, int n_views,
+                                                    const uint32_t *__restrict__ order,
                                                     const uint2 *__restrict__ ranges,
                                                     const uint32_t *__restrict__ list,
                                                     const float4 *__restrict__ rec, BlendParams bp, float w_bg,
@@ -43,7 +44,7 @@ __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restri
     chain_begin();
     constexpr int NR = 2, NB = batch_cells(1);
     const int lane = threadIdx.x;
-    const int tile = blockIdx.x / CSUB, sub = blockIdx.x % CSUB;
+    const int tile = (int)order[blockIdx.x / CSUB], sub = blockIdx.x % CSUB;
     const ViewDesc &V = views[find_view(views, n_views, tile)];
     const int local = tile - V.tile_base;
     const int tx = local % V.Tx, ty = local / V.Tx;
@@ -189,7 +190,8 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
         (s = ws.zval.ensure(4 * n1)) || (s = ws.rect.ensure(8 * n1)) || (s = ws.count.ensure(4 * n1)) ||
         (s = ws.offs.ensure(4 * n1)) ||
         (s = ws.scan.ensure(4 * scan_scratch_words(n1))) || (s = ensure_sort_scratch(ws, n)) ||
-        (s = ws.rec.ensure(sizeof(float4) * kRecF4 * n1)) || (s = ws.ranges.ensure(8 * (size_t)std::max(1, tiles))))
+        (s = ws.rec.ensure(sizeof(float4) * kRecF4 * n1)) || (s = ws.ranges.ensure(8 * (size_t)std::max(1, tiles))) ||
+        (s = ws.order.ensure(4 * (size_t)std::max(1, tiles))))
         return s;
     if (ws.h_views_cap < (size_t)V) {
         if (ws.h_views) cudaFreeHost(ws.h_views);
@@ -231,13 +233,14 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
                 d_vis, nullptr);
     sort_tiles(ws, L, bits, nullptr, st);
     launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, st);
+    launch_tile_order((const uint2 *)ws.ranges.p, tiles, (uint32_t *)ws.order.p, st);
     if (tiles > 0) {
         const unsigned grid = (unsigned)tiles * CSUB;
         if (wsr)
-            launch_chained(k_gauss_blend<false>, grid, CT, 0, st, dv, V, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
+            launch_chained(k_gauss_blend<false>, grid, CT, 0, st, dv, V, (const uint32_t *)ws.order.p, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
                                                       (const float4 *)ws.rec.p, bp, cfg.w_bg, out_img, nullptr);
         else
-            launch_chained(k_gauss_blend<true>, grid, CT, 0, st, dv, V, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
+            launch_chained(k_gauss_blend<true>, grid, CT, 0, st, dv, V, (const uint32_t *)ws.order.p, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
                                                      (const float4 *)ws.rec.p, bp, 0.f, out_img, out_nd);
     }
     CK(cudaGetLastError());

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "dgs.h"
 
 namespace dgs {
@@ -142,6 +144,10 @@ void launch_emit(const uint32_t *offs, const uint32_t *zval_sorted, const short4
 void launch_tile_ranges(const uint32_t *tkey_sorted, long long L, uint2 *ranges, cudaStream_t st,
                         const uint32_t *d_L = nullptr);
 
+// order[i]: the tile that the blend kernels' i-th blocks take, longest lists first.
+void launch_tile_order(const uint2 *ranges, int n_tiles, uint32_t *order, cudaStream_t st,
+                       const ChainSizes *dsz = nullptr);
+
 // sort.cu
 struct SortScratch {
     uint32_t *keys_alt, *vals_alt;   // n each
@@ -242,12 +248,12 @@ void launch_project_bwd(const ViewDesc *views, int n_views, int slot, const Scen
                         float *g_log_scale, float *g_quat, float *g_logit, float *g_sh, cudaStream_t st);
 
 // blend.cu
-void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const uint2 *ranges,
+void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const uint32_t *order, const uint2 *ranges,
                       const uint32_t *tile_cells, const float4 *rec, const BlendParams &bp, float *out_rgb,
                       float *out_rgb2, float *out_D, int *out_nd, int K_all, cudaStream_t st,
                       const ChainSizes *dsz = nullptr, uint32_t *work = nullptr);
 // g_v_entry (nullable): dL/dv_n accumulated per (view, cell) entry [cell_base + cell].
-void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, int K, const uint2 *ranges,
+void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, const uint32_t *order, int K, const uint2 *ranges,
                       const uint32_t *tile_cells, const float4 *rec, const BlendParams &bp, const float *rgb,
                       const float *D, const int *nd, const float *dL_drgb, float *g2d, float *g_v_entry,
                       cudaStream_t st);
@@ -304,21 +310,36 @@ __device__ __forceinline__ void chain_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// cluster: CTAs per cluster, or 0 for a launch without clusters (a launch in clusters
+// of one is not the same: blocks of one warp then start more slowly).
+struct ClusterSize { unsigned n; };
 template <typename... P, typename... A>
-inline void launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A &&...a) {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
+inline void launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+                           ClusterSize cluster, A &&...a) {
+    cudaLaunchAttribute at[2] = {};
     cudaLaunchConfig_t c{};
     c.gridDim = dim3(grid);
     c.blockDim = dim3(threads);
     c.dynamicSmemBytes = smem;
     c.stream = st;
-    c.attrs = &at;
+    c.attrs = at;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(st, &capture);
-    c.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    if (capture == cudaStreamCaptureStatusNone) {
+        at[c.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[c.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster.n > 0) {
+        at[c.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[c.numAttrs].val.clusterDim.x = cluster.n;
+        at[c.numAttrs].val.clusterDim.y = at[c.numAttrs].val.clusterDim.z = 1;
+        ++c.numAttrs;
+    }
     cudaLaunchKernelEx(&c, kernel, static_cast<P>(a)...);
+}
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A &&...a) {
+    launch_chained(kernel, grid, threads, smem, st, ClusterSize{0}, std::forward<A>(a)...);
 }
 
 // Clear the words of a BinPrep (all threads of the grid).

@@ -85,7 +85,7 @@ struct Workspace {
     DevBuf views, scenes;
     DevBuf zkey, zval, rect, depth, count, offs;             // per (view, cell)
     DevBuf tkey, tval;                                       // per (tile, cell) pair
-    DevBuf ranges;                                           // per tile
+    DevBuf ranges, order;                                    // per tile
     DevBuf rec, g2d;                                         // per (view, Gaussian)
     DevBuf Dpix, ndpix, rgb;                                 // per pixel
     DevBuf gstage;                                           // backward staging

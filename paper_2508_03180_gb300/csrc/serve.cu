@@ -113,7 +113,7 @@ dgs_status plan_batch(dgs_ctx *ctx, const std::vector<PendingReq> &reqs, BatchPl
 long long slot_bytes(const ChainCaps &c) {
     const long long n = std::max(c.E, c.L);
     return (long long)sizeof(ViewDesc) * c.V + (long long)sizeof(SceneDev) * c.S + 32 * c.E + 4 * c.E / 1024 +
-           8 * n + 1024 * (n / 4096 + 1) + 8 * c.L + 8 * c.T + 48 * c.R + 20 * c.P +
+           8 * n + 1024 * (n / 4096 + 1) + 8 * c.L + 12 * c.T + 48 * c.R + 20 * c.P +
            (c.W > 0 ? 4 * c.W + 4LL * kDecF * c.R : 0);
 }
 
@@ -186,7 +186,7 @@ dgs_status fit_slot(dgs_ctx *ctx, ServeState &S, GraphSlot &g, const BatchPlan &
         (s = ws.zval.ensure(4 * c.E)) || (s = ws.rect.ensure(8 * c.E)) || (s = ws.depth.ensure(4 * c.E)) ||
         (s = ws.count.ensure(4 * c.E)) || (s = ws.offs.ensure(4 * c.E)) ||
         (s = ws.scan.ensure(4 * scan_scratch_words(c.E))) || (s = ensure_sort_scratch(ws, std::max(c.E, c.L))) ||
-        (s = ws.tkey.ensure(4 * c.L)) || (s = ws.tval.ensure(4 * c.L)) || (s = ws.ranges.ensure(8 * c.T)) ||
+        (s = ws.tkey.ensure(4 * c.L)) || (s = ws.tval.ensure(4 * c.L)) || (s = ws.ranges.ensure(8 * c.T)) || (s = ws.order.ensure(4 * c.T)) ||
         (s = ws.rec.ensure(sizeof(float4) * kRecF4 * c.R)) || (s = ws.Dpix.ensure(4 * c.P)) ||
         (s = ws.ndpix.ensure(4 * c.P)) || (s = ws.rgb.ensure(12 * c.P)) || (s = ws.vview.ensure(4 * c.E)) ||
         (c.W > 0 && ((s = ws.dec.ensure(sizeof(float) * kDecF * c.R)) || (s = ws.wpack.ensure(sizeof(float) * c.W)))))
@@ -248,6 +248,7 @@ dgs_status record_chain(dgs_ctx *ctx, Workspace &ws, const ChainCaps &c, const B
     radix_sort_counted((uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, c.L, bits, chain_sort_scratch(ws, 1), st, d_L,
                        nullptr, true);
     launch_tile_ranges((const uint32_t *)ws.tkey.p, c.L, (uint2 *)ws.ranges.p, st, d_L);
+    launch_tile_order((const uint2 *)ws.ranges.p, (int)c.T, (uint32_t *)ws.order.p, st, dsz);
     // neural scenes: the decode writes their records (slot k's samples of the
     // visible entries, counted on the device); the table projection skips them
     for (size_t k = 0; k < p.scenes.size(); ++k) {
@@ -259,7 +260,7 @@ dgs_status record_chain(dgs_ctx *ctx, Workspace &ws, const ChainCaps &c, const B
     }
     launch_project_fwd_table(dv, (const SceneDev *)ws.scenes.p, c.G, (const uint32_t *)ws.count.p,
                              (const float *)ws.vview.p, bp, (float4 *)ws.rec.p, st, dsz);
-    launch_blend_fwd(dv, c.V, (int)c.T, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
+    launch_blend_fwd(dv, c.V, (int)c.T, (const uint32_t *)ws.order.p, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
                      (const float4 *)ws.rec.p, bp, (float *)ws.rgb.p, nullptr, (float *)ws.Dpix.p, (int *)ws.ndpix.p,
                      p.K_all, st, dsz, small + kSmallWork);
     CKR(cudaMemcpyAsync(ws.h_small, small, 64, cudaMemcpyDeviceToHost, st));
