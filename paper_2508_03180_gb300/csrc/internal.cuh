@@ -304,10 +304,14 @@ cudaError_t set_tc_fault(bool on);  // the tensor-core decode's completion wait 
 // 330 -> 310).  Every such kernel calls chain_begin before it touches
 // global memory: it waits there until the predecessor has
 // completed and its writes are visible, and lets its own successor be launched.
+// A kernel before a blend only waits (chain_wait): blend blocks that are
+// placed while it still runs crowd on the SMs it has left, the longest lists
+// first (20,011 cells x 5, three 641 x 479 views: 850 us a step, 754 so).
 // Not within a captured graph, whose own edges are cheap already (a served burst
 // of eight requests: 881 us plain, 917 us chained).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_begin() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    chain_wait();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 // cluster: CTAs per cluster, or 0 for a launch without clusters (a launch in clusters

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(128) k_project_fwd(const ViewDesc *__restrict_
                                                      SceneDev sc, const uint32_t *__restrict__ count,
                                                      const float *__restrict__ vview, BlendParams bp,
                                                      float4 *__restrict__ rec, float *__restrict__ g2d_zero) {
-    chain_begin();
+    chain_wait();
     project_scene(views, n_views, slot, sc, count, vview, bp, rec, g2d_zero);
 }
 
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(128) k_project_fwd_table(const ViewDesc *__res
                                                            const float *__restrict__ vview, BlendParams bp,
                                                            float4 *__restrict__ rec,
                                                            const ChainSizes *__restrict__ dsz) {
-    chain_begin();
+    chain_wait();
     const int n_views = dsz->n_views, n_scenes = dsz->n_scenes;
     for (int s = 0; s < n_scenes; ++s) {
         const SceneDev sc = scenes[s];
