@@ -90,8 +90,12 @@ __device__ __forceinline__ bool rs_trivial(const uint32_t *hist, int q, long lon
 
 constexpr int RS_LOOK = 8;  // predecessors that a look-back reads at a time
 
+// A pass is latency more than rate: 5.6M pairs move 90 MB, 13 us at the copy rate, and
+// take 52 (61 with the values held in registers from the start and the look-back
+// before the reordering, 80 registers and three CTAs an SM; four at 64).
+
 template <int ITEMS>
-__global__ void __launch_bounds__(RS_THREADS) k_rs_pass(uint32_t *__restrict__ k0, uint32_t *__restrict__ v0,
+__global__ void __launch_bounds__(RS_THREADS, 4) k_rs_pass(uint32_t *__restrict__ k0, uint32_t *__restrict__ v0,
                                                         uint32_t *__restrict__ k1, uint32_t *__restrict__ v1,
                                                         long long n, const uint32_t *__restrict__ d_n,
                                                         const uint32_t *__restrict__ d_live, int pass,
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_pass(uint32_t *__restrict__ k
     __shared__ uint32_t s_key[TILE], s_val[TILE];  // the partition in digit order
     __shared__ uint32_t s_part, s_cnt;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    chain_begin();
+    chain_wait();
     if (d_n) n = *d_n;
     const bool drop = d_live && pass == 0;
     if (d_live && pass > 0) n = *d_live;
@@ -156,31 +160,41 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_pass(uint32_t *__restrict__ k
         status_next[part * 256 + tid] = 0u;
         const long long base = part * TILE + (long long)warp * WARP_ITEMS;
 
-        uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
+        uint32_t key[ITEMS], rank[ITEMS];
         unsigned live = 0;  // bit `it`: the item is there
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
             const long long idx = base + it * 32 + lane;
             const bool ok = idx < n;
             key[it] = ok ? kin[idx] : 0u;
-            val[it] = ok ? vin[idx] : 0u;
             live |= ok && !(drop && key[it] == 0xFFFFFFFFu) ? 1u << it : 0u;
         }
         const unsigned lt_mask = (1u << lane) - 1u;
-        // rank inside the warp, in item order (it, lane): stable
+        // rank inside the warp, in item order (it, lane): stable.  The lanes with an
+        // equal digit come from one ballot per bit: independent of one another and
+        // of the other items', where match.any is a serial instruction.
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
             const bool ok = (live >> it) & 1u;
-            const unsigned active = __ballot_sync(0xffffffffu, ok);
-            rank[it] = 0;
-            if (ok) {
-                const uint32_t d = (key[it] >> shift) & 255u;
-                const unsigned peers = __match_any_sync(active, d);
-                const uint32_t before = s_warp[warp][d];
-                rank[it] = before + __popc(peers & lt_mask);
-                __syncwarp(active);
-                if (lane == __ffs(peers) - 1) s_warp[warp][d] = before + __popc(peers);
+            unsigned peers = __ballot_sync(0xffffffffu, ok);
+            const uint32_t d = (key[it] >> shift) & 255u;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const bool bit = (d >> b) & 1u;
+                const unsigned m = __ballot_sync(0xffffffffu, bit);
+                peers &= bit ? m : ~m;
             }
+            rank[it] = peers;
+        }
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const bool ok = (live >> it) & 1u;
+            const unsigned peers = rank[it];
+            const uint32_t d = (key[it] >> shift) & 255u;
+            const uint32_t before = s_warp[warp][d];
+            __syncwarp();
+            if (ok && lane == __ffs(peers) - 1) s_warp[warp][d] = before + __popc(peers);
+            rank[it] = before + __popc(peers & lt_mask);
             __syncwarp();
         }
         __syncthreads();
@@ -202,6 +216,18 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_pass(uint32_t *__restrict__ k
         }
         s_local[d] = scan256(total);  // partition-local digit starts
         if (d == 255) s_cnt = s_local[255] + total;
+        __syncthreads();
+        // the partition in digit order in shared memory (which frees the registers and
+        // gives the predecessors time before the look-back)
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            if ((live >> it) & 1u) {
+                const uint32_t dg = (key[it] >> shift) & 255u;
+                const uint32_t lp = s_local[dg] + s_warp[warp][dg] + rank[it];
+                s_key[lp] = key[it];
+                s_val[lp] = vin[base + it * 32 + lane];
+            }
+        }
         if (part == 0) {
             s_base[d] = digit_base;
         } else {
@@ -232,18 +258,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_pass(uint32_t *__restrict__ k
             s_base[d] = digit_base + excl;
         }
         __syncthreads();
-        // the partition in digit order in shared memory, then out with
-        // consecutive threads on consecutive destinations within each digit
-#pragma unroll
-        for (int it = 0; it < ITEMS; ++it) {
-            if ((live >> it) & 1u) {
-                const uint32_t dg = (key[it] >> shift) & 255u;
-                const uint32_t lp = s_local[dg] + s_warp[warp][dg] + rank[it];
-                s_key[lp] = key[it];
-                s_val[lp] = val[it];
-            }
-        }
-        __syncthreads();
+        // out with consecutive threads on consecutive destinations within each digit
         const int cnt = (int)s_cnt;
         for (int i = tid; i < cnt; i += RS_THREADS) {
             const uint32_t k = s_key[i], dg = (k >> shift) & 255u;
@@ -347,7 +362,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_pair_offsets(const uint32_t *__r
     constexpr unsigned long long AGG = 1ull << 32, INC = 2ull << 32;
     __shared__ uint32_t s_warp[SC_THREADS / 32], s_part, s_excl;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    chain_begin();
+    chain_wait();
     if (d_all) n_all = *d_all;
     const long long n = d_n ? (long long)*d_n : n_all;
     const long long n_parts = (n + SC_TILE - 1) / SC_TILE;
