@@ -5,6 +5,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "internal.cuh"
 #include "sh.cuh"
@@ -159,10 +160,11 @@ void launch_cell_project(const ViewDesc *views, int n_views, const SceneDev *sce
 // entries; one thread's two binary searches were 40, most of a small view's 19 us
 // in here).  When at most EM_TB entries lie between them (always for the
 // depth-sorted entries, of which each owns a slot) their offsets are staged in
-// shared memory, otherwise (entries that own no slot interleaved, as in the
-// weighted-sum comparator's index order) they are searched in global memory.  A
-// thread finds the owner of the first of its eight consecutive slots and walks on from
-// there, one division for its tile, and writes the eight keys and cells as vectors.
+// shared memory with their first tile, row lengths and cell, otherwise
+// (entries that own no slot interleaved, as in the weighted-sum comparator's index
+// order) they are searched in global memory.  A thread finds the owner of the first
+// of its eight consecutive slots and walks on from there, with one division for the
+// first slot's tile, and writes the eight keys and cells as vectors.
 // Entries are in depth order, so the emitted sequence is (depth, cell)-ordered
 // within every tile; the stable tile sort keeps that order.  The keys' digits are
 // counted on the way, runs of equal digits of a thread at once.
@@ -191,12 +193,15 @@ __global__ void __launch_bounds__(EM_THREADS) k_emit(const uint32_t *__restrict_
                                                      int passes, BinPrep prep, const ChainSizes *__restrict__ dsz,
                                                      const uint32_t *__restrict__ d_n,
                                                      const uint32_t *__restrict__ d_L) {
-    __shared__ uint32_t s_off[EM_TB + 1];
+    // the run's entries: first slot (less j0), first tile, tiles per row | tiles of the
+    // view's row << 16, cell
+    __shared__ int s_off[EM_TB];
+    __shared__ uint32_t s_tile[EM_TB], s_wt[EM_TB], s_cell[EM_TB];
     __shared__ uint32_t s_hist[4][256];
     __shared__ long long s_own[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i < passes * 256; i += EM_THREADS) (&s_hist[0][0])[i] = 0u;
-    chain_begin();
+    chain_wait();
     prep_clear(prep, blockIdx.x * (long long)EM_THREADS + tid, (long long)gridDim.x * EM_THREADS);
     if (dsz) {
         n_views = dsz->n_views;
@@ -205,63 +210,76 @@ __global__ void __launch_bounds__(EM_THREADS) k_emit(const uint32_t *__restrict_
     }
     if (d_n) n_entries = *d_n;
     if (d_L) L = *d_L;
+    // (bounds: only a sort that gave up can leave an entry outside the arrays)
+    auto entry = [&](long long e, uint32_t &tile, uint32_t &wt, uint32_t &cell) {
+        const uint32_t vi = (uint32_t)min((long long)zval[e], n_all - 1);
+        int vlo = 0, vhi = n_views;  // view owning entry vi
+        while (vhi - vlo > 1) {
+            const int mid = (vlo + vhi) >> 1;
+            if (views[mid].cell_base <= (long long)vi) vlo = mid; else vhi = mid;
+        }
+        const ViewDesc &V = views[vlo];
+        const short4 r = rect[vi];
+        tile = (uint32_t)(V.tile_base + r.y * V.Tx + r.x);
+        wt = (uint32_t)(r.z - r.x + 1) | (uint32_t)V.Tx << 16;
+        cell = (uint32_t)((long long)vi - V.cell_base);
+    };
     for (long long j0 = blockIdx.x * (long long)EM_TB; j0 < L; j0 += (long long)gridDim.x * EM_TB) {
-        const long long j1 = min(j0 + (long long)EM_TB, L);  // this run: [j0, j1)
-        __syncthreads();  // s_off and s_own of the last run are read (and s_hist is clear)
+        const int run = (int)min((long long)EM_TB, L - j0);  // slots [j0, j0 + run)
+        __syncthreads();  // the last run's entries are read (and s_hist is clear)
         if (warp < 2) {
-            const long long o = warp_owner(offs, n_entries, warp == 0 ? j0 : j1 - 1, lane);
+            const long long o = warp_owner(offs, n_entries, warp == 0 ? j0 : j0 + run - 1, lane);
             if (lane == 0) s_own[warp] = o;
         }
         __syncthreads();
-        const long long e0 = s_own[0], ne = s_own[1] - e0 + 1;  // the run's owners are entries [e0, e0 + ne)
+        const long long e0 = s_own[0];
+        const int ne = (int)min(s_own[1] - e0 + 1, (long long)INT_MAX);  // the run's owners are entries [e0, e0 + ne)
         const bool staged = ne <= EM_TB;
         if (staged)
-            for (int i = tid; i < (int)ne; i += EM_THREADS) s_off[i] = offs[e0 + i];
+            for (int i = tid; i < ne; i += EM_THREADS) {
+                s_off[i] = (int)((long long)offs[e0 + i] - j0);
+                entry(e0 + i, s_tile[i], s_wt[i], s_cell[i]);
+            }
         __syncthreads();
-        const long long j = j0 + (long long)tid * EM_ITEMS;
-        if (j >= j1) continue;
-        auto off = [&](long long i) { return (long long)(staged ? s_off[i] : offs[e0 + i]); };
-        long long lo = 0, hi = ne;  // last i in [0, ne) with off(i) <= j
-        while (hi - lo > 1) {
-            const long long mid = (lo + hi) >> 1;
-            if (off(mid) <= j) lo = mid; else hi = mid;
+        const int js = tid * EM_ITEMS;
+        if (js >= run) continue;
+        auto off = [&](int i) { return staged ? s_off[i] : (int)((long long)offs[e0 + i] - j0); };
+        int own = 0, hi = ne;  // last i in [0, ne) with off(i) <= js
+        while (hi - own > 1) {
+            const int mid = (own + hi) >> 1;
+            if (off(mid) <= js) own = mid; else hi = mid;
         }
         uint32_t key[EM_ITEMS], cell[EM_ITEMS];
-        long long own = lo, next = -1;  // the current owner; its slots end before `next`
-        int x = 0, y = 0, x0 = 0, x1 = 0, Tx = 0, tile_base = 0;
-        uint32_t cellid = 0;
+        uint32_t tile = 0, wt = 1, cellid = 0;  // of the current owner
+        int next = js, x = 0;                   // its slots end before `next`; the slot's column
+        const long long j = j0 + js, j1 = j0 + run;
 #pragma unroll
         for (int i = 0; i < EM_ITEMS; ++i) {
-            const long long ji = j + i;
             key[i] = cell[i] = 0u;
-            if (ji < j1) {
-                if (ji >= next) {  // enter the owner of slot ji
+            if (js + i < run) {
+                if (js + i >= next) {  // enter the owner of this slot
                     if (i > 0)
-                        while (own + 1 < ne && off(own + 1) <= ji) ++own;
-                    next = own + 1 < ne ? off(own + 1) : j1;
-                    // (bounds: only a sort that gave up can leave an entry outside the arrays)
-                    const uint32_t vi = (uint32_t)min((long long)zval[e0 + own], n_all - 1);
-                    int vlo = 0, vhi = n_views;  // view owning entry vi
-                    while (vhi - vlo > 1) {
-                        const int mid = (vlo + vhi) >> 1;
-                        if (views[mid].cell_base <= (long long)vi) vlo = mid; else vhi = mid;
+                        while (own + 1 < ne && off(own + 1) <= js + i) ++own;
+                    if (staged) {
+                        tile = s_tile[own];
+                        wt = s_wt[own];
+                        cellid = s_cell[own];
+                    } else {
+                        entry(e0 + own, tile, wt, cellid);
                     }
-                    const ViewDesc &V = views[vlo];
-                    cellid = (uint32_t)((long long)vi - V.cell_base);
-                    const short4 r = rect[vi];
-                    const int w = r.z - r.x + 1, local = (int)(ji - off(own));
-                    x0 = r.x;
-                    x1 = r.z;
-                    y = r.y + local / w;
-                    x = x0 + local % w;
-                    Tx = V.Tx;
-                    tile_base = V.tile_base;
+                    x = 0;  // (an owner entered past the thread's first slot is entered at its first)
+                    if (i == 0) {
+                        const uint32_t local = (uint32_t)(js - off(own)), y = local / (wt & 0xffffu);
+                        x = (int)(local - y * (wt & 0xffffu));
+                        tile += y * (wt >> 16);
+                    }
+                    next = own + 1 < ne ? off(own + 1) : run;
                 }
-                key[i] = min((uint32_t)(tile_base + y * Tx + x), (uint32_t)(n_tiles - 1));
+                key[i] = min(tile + (uint32_t)x, (uint32_t)(n_tiles - 1));
                 cell[i] = cellid;
-                if (++x > x1) {
-                    x = x0;
-                    ++y;
+                if (++x == (int)(wt & 0xffffu)) {
+                    x = 0;
+                    tile += wt >> 16;
                 }
             }
         }
@@ -319,7 +337,7 @@ void launch_emit(const uint32_t *offs, const uint32_t *zval_sorted, const short4
 // tiles keep the (0,0) the caller cleared them to.
 __global__ void k_tile_ranges(const uint32_t *__restrict__ key, long long L, const uint32_t *__restrict__ d_L,
                               uint2 *__restrict__ ranges) {
-    chain_begin();
+    chain_wait();
     if (d_L) L = *d_L;
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < L; j += (long long)gridDim.x * blockDim.x) {
         const uint32_t k = key[j];
@@ -357,7 +375,7 @@ __global__ void __launch_bounds__(TO_THREADS) k_tile_order(const uint2 *__restri
     const int tid = threadIdx.x;
     if (tid < 128) s_cnt[tid] = 0u;
     __syncthreads();
-    chain_begin();
+    chain_wait();
     if (dsz) n_tiles = dsz->total_tiles;
     const int stride = ctas * TO_THREADS;
     auto sweep = [&](auto &&f) {
