@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd(const ViewDesc 
                                                   float *__restrict__ out_rgb, float *__restrict__ out_rgb2,
                                                   float *__restrict__ out_D, int *__restrict__ out_nd) {
     __shared__ float4 s_rec[FSTAGE][kBatchF4];
-    chain_begin();
+    chain_wait();
     blend_fwd_unit<KT, FWD_PPL, VAR>(blockIdx.x, views, n_views, order, ranges, cells, rec, bp, out_rgb, out_rgb2, out_D, out_nd,
                                 s_rec);
 }
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd_pull(const View
                                                        int *__restrict__ out_nd, const ChainSizes *__restrict__ dsz,
                                                        uint32_t *__restrict__ work) {
     __shared__ float4 s_rec[FSTAGE][kBatchF4];
-    chain_begin();
+    chain_wait();
     const int n_views = dsz->n_views;
     const uint32_t units = (uint32_t)dsz->total_tiles * FWD_SUB;
     for (;;) {
@@ -617,6 +617,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
                                                   const int *__restrict__ ndpix, const float *__restrict__ dL_drgb,
                                                   float *__restrict__ g2d, float *__restrict__ g_cell_v) {
     extern __shared__ float4 s_bwd[];
+    chain_wait();
     const int lane = threadIdx.x;
     const int tile = (int)order[blockIdx.x / BWD_SUB], sub = blockIdx.x % BWD_SUB;
     const int vi = find_view(views, n_views, tile);
@@ -912,15 +913,14 @@ void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, const
     if (total_tiles == 0) return;
     const unsigned grid = (unsigned)total_tiles * BWD_SUB;
     const size_t smem = sizeof(float4) * bwd_smem_f4(K_all);
-    // (a plain launch: chained to its successor it took 0.5% longer on the 1M-Gaussian step)
 #define DGS_BWD(KV, VV)                                                                                          \
     do {                                                                                                        \
         if (g_cell_v)                                                                                           \
-            k_blend_bwd<KV, VV, true><<<grid, WT, smem, st>>>(views, n_views, order, ranges, tile_cells, rec, bp, rgb, D, nd, \
-                                                              dL_drgb, g2d, g_cell_v);                          \
+            launch_chained(k_blend_bwd<KV, VV, true>, grid, WT, smem, st, views, n_views, order, ranges, tile_cells, \
+                           rec, bp, rgb, D, nd, dL_drgb, g2d, g_cell_v);                                        \
         else                                                                                                    \
-            k_blend_bwd<KV, VV, false><<<grid, WT, smem, st>>>(views, n_views, order, ranges, tile_cells, rec, bp, rgb, D, nd, \
-                                                               dL_drgb, g2d, nullptr);                          \
+            launch_chained(k_blend_bwd<KV, VV, false>, grid, WT, smem, st, views, n_views, order, ranges, tile_cells, \
+                           rec, bp, rgb, D, nd, dL_drgb, g2d, nullptr);                                         \
     } while (0)
     if (blend_variants(bp)) {
         switch (K_all) {

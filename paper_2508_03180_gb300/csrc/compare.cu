@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restri
                                                     const float4 *__restrict__ rec, BlendParams bp, float w_bg,
                                                     float *__restrict__ out_rgb, int *__restrict__ out_nd) {
     __shared__ float4 s_rec[FSTAGE][kBatchF4];
-    chain_begin();
+    chain_wait();
     constexpr int NR = 2, NB = batch_cells(1);
     const int lane = threadIdx.x;
     const int tile = (int)order[blockIdx.x / CSUB], sub = blockIdx.x % CSUB;

@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(128) k_decode_samples(const ViewDesc *__restri
                                                         SceneDev sc, const uint32_t *__restrict__ samples,
                                                         long long nsamp,
                                                         const uint32_t *__restrict__ d_n, float *__restrict__ srec) {
+    chain_wait();
     if (d_n) nsamp = min(nsamp, (long long)*d_n);  // the count on the device (capacity nsamp)
     const long long N = sc.N;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nsamp;
@@ -223,6 +224,7 @@ __global__ void __launch_bounds__(128) k_decode_samples(const ViewDesc *__restri
 // Every Gaussian's centre x_n + R(Q_n)(O_pos S_n) and Eq. 11 bound 1 - |O_pos|
 // (the same in every view), for the forward's epilogue.
 __global__ void __launch_bounds__(128) k_decode_centres(SceneDev sc, float4 *__restrict__ gc) {
+    chain_wait();
     const long long N = sc.N, G = sc.G;
     const int K = sc.K;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < G; g += (long long)gridDim.x * blockDim.x) {
@@ -288,6 +290,7 @@ __device__ void stage_samples(const MlpShape &S, float *sm, const SceneDev &sc, 
 // The packed weights in their shared-memory layouts (zero for padded hidden
 // units and outputs); one thread per packed float.
 __global__ void k_mlp_pack(const float *__restrict__ w, MlpShape S, float *__restrict__ pk) {
+    chain_wait();
     const int H4 = 4 * S.Hp, Rp = S.rb[4];
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < S.g_total; idx += gridDim.x * blockDim.x) {
         float v = 0.f;
@@ -495,6 +498,7 @@ __global__ void __launch_bounds__(256) k_decode(const ViewDesc *__restrict__ vie
                                                 float *__restrict__ dec, const float *__restrict__ vview,
                                                 BlendParams bp, float4 *__restrict__ rec,
                                                 float *__restrict__ g2d_zero) {
+    chain_wait();
     if (d_n) nsamp = min(nsamp, (long long)*d_n);  // the count on the device (capacity nsamp)
     extern __shared__ float4 smem4[];
     float *sm = reinterpret_cast<float *>(smem4);
@@ -602,6 +606,7 @@ static bool tc_fits(int F, int H, int K) {
 // The weight image: element e of a region holds the operand entry at its
 // core-matrix position (the inverse of tc::cm_off), hi or lo part.
 __global__ void k_mlp_pack_tc(const float *__restrict__ w, TcShape T, float *__restrict__ img) {
+    chain_wait();
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < T.g_total; idx += gridDim.x * blockDim.x) {
         float v = 0.f;
         bool lo = false;
@@ -716,6 +721,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_decode_tc(const ViewDesc *__r
                                                                float *__restrict__ dec, const float *__restrict__ vview,
                                                                BlendParams bp, float4 *__restrict__ rec,
                                                                float *__restrict__ g2d_zero, uint32_t *err) {
+    chain_wait();
     if (d_n) nsamp = min(nsamp, (long long)*d_n);  // the count on the device (capacity nsamp)
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) uint64_t mbar;
@@ -859,6 +865,7 @@ __global__ void __launch_bounds__(256) k_decode_bwd(SceneDev sc, MlpShape S, con
                                                         float *__restrict__ g_feat, float *__restrict__ g_offset,
                                                         float *__restrict__ rows, float *__restrict__ g_mlp,
                                                         CellGrads cg) {
+    chain_wait();
     if (d_n) nsamp = min(nsamp, (long long)*d_n);  // the count on the device (capacity nsamp)
     extern __shared__ float4 smem4[];
     float *sm = reinterpret_cast<float *>(smem4);
@@ -1354,9 +1361,9 @@ long long decode_scratch_floats(int F, int H, int K, long long nsamp, long long 
 static void decode_prep(const ViewDesc *views, int n_views, int slot, const SceneDev &sc, const MlpShape &S,
                         const uint32_t *samples, long long nsamp, const uint32_t *d_n, float *pk, float *srec,
                         cudaStream_t st) {
-    k_mlp_pack<<<(S.g_total + 255) / 256, 256, 0, st>>>(sc.mlp, S, pk);
+    launch_chained(k_mlp_pack, (S.g_total + 255) / 256, 256, 0, st, sc.mlp, S, pk);
     const long long b = std::min((nsamp + 127) / 128, 152LL * 16);
-    k_decode_samples<<<(unsigned)std::max(1LL, b), 128, 0, st>>>(views, n_views, slot, sc, samples, nsamp, d_n, srec);
+    launch_chained(k_decode_samples, (unsigned)std::max(1LL, b), 128, 0, st, views, n_views, slot, sc, samples, nsamp, d_n, srec);
 }
 
 void launch_decode(const ViewDesc *views, int n_views, int slot, const SceneDev &sc, const uint32_t *samples,
@@ -1367,15 +1374,15 @@ void launch_decode(const ViewDesc *views, int n_views, int slot, const SceneDev 
         const TcShape T = tc_shape(sc.F, sc.H, sc.K);
         float *img = scratch, *srec = scratch + up_to(T.g_total, 4);
         float4 *gc = reinterpret_cast<float4 *>(srec + nsamp * DINFO);
-        k_mlp_pack_tc<<<(T.g_total + 255) / 256, 256, 0, st>>>(sc.mlp, T, img);
+        launch_chained(k_mlp_pack_tc, (T.g_total + 255) / 256, 256, 0, st, sc.mlp, T, img);
         const long long b = std::min((nsamp + 127) / 128, 152LL * 16);
-        k_decode_samples<<<(unsigned)std::max(1LL, b), 128, 0, st>>>(views, n_views, slot, sc, samples, nsamp, d_nsamp,
+        launch_chained(k_decode_samples, (unsigned)std::max(1LL, b), 128, 0, st, views, n_views, slot, sc, samples, nsamp, d_nsamp,
                                                                      srec);
         const long long bg = std::min((sc.G + 127) / 128, 152LL * 16);
-        k_decode_centres<<<(unsigned)std::max(1LL, bg), 128, 0, st>>>(sc, gc);
+        launch_chained(k_decode_centres, (unsigned)std::max(1LL, bg), 128, 0, st, sc, gc);
         const long long tiles = (nsamp + TC_M - 1) / TC_M;
         const int grid = persistent_grid(k_decode_tc, TC_THREADS, (size_t)T.s_total, tiles);
-        k_decode_tc<<<grid, TC_THREADS, (size_t)T.s_total, st>>>(views, sc, T, img, srec, gc, nsamp, d_nsamp, dec,
+        launch_chained(k_decode_tc, grid, TC_THREADS, (size_t)T.s_total, st, views, sc, T, img, srec, gc, nsamp, d_nsamp, dec,
                                                                vview, bp, rec, g2d_zero, err);
         return;
     }
@@ -1384,16 +1391,16 @@ void launch_decode(const ViewDesc *views, int n_views, int slot, const SceneDev 
     float4 *gc = reinterpret_cast<float4 *>(srec + nsamp * DINFO);
     decode_prep(views, n_views, slot, sc, S, samples, nsamp, d_nsamp, pk, srec, st);
     const long long bg = std::min((sc.G + 127) / 128, 152LL * 16);
-    k_decode_centres<<<(unsigned)std::max(1LL, bg), 128, 0, st>>>(sc, gc);
+    launch_chained(k_decode_centres, (unsigned)std::max(1LL, bg), 128, 0, st, sc, gc);
     const size_t smem = sizeof(float) * (size_t)S.s_total;
     const long long tiles = (nsamp + S.M - 1) / S.M;
     if (S.HW == 4) {
         const int b = persistent_grid(k_decode<4>, 32 * S.W, smem, tiles);
-        k_decode<4><<<b, 32 * S.W, smem, st>>>(views, sc, S, pk, srec, gc, nsamp, d_nsamp, dec, vview, bp, rec,
+        launch_chained(k_decode<4>, b, 32 * S.W, smem, st, views, sc, S, pk, srec, gc, nsamp, d_nsamp, dec, vview, bp, rec,
                                                g2d_zero);
     } else {
         const int b = persistent_grid(k_decode<8>, 32 * S.W, smem, tiles);
-        k_decode<8><<<b, 32 * S.W, smem, st>>>(views, sc, S, pk, srec, gc, nsamp, d_nsamp, dec, vview, bp, rec,
+        launch_chained(k_decode<8>, b, 32 * S.W, smem, st, views, sc, S, pk, srec, gc, nsamp, d_nsamp, dec, vview, bp, rec,
                                                g2d_zero);
     }
 }
@@ -1411,7 +1418,7 @@ void launch_decode_bwd(const ViewDesc *views, int n_views, int slot, const Scene
 #define DGS_DBWD(HWV, FUSEV, CELLV, ROWS)                                                                      \
     do {                                                                                                      \
         const int b = persistent_grid(k_decode_bwd<HWV, FUSEV, CELLV>, 32 * S.W, smem, tiles);                \
-        k_decode_bwd<HWV, FUSEV, CELLV><<<b, 32 * S.W, smem, st>>>(sc, S, pk, srec, nsamp, d_nsamp, gdec,     \
+        launch_chained(k_decode_bwd<HWV, FUSEV, CELLV>, b, 32 * S.W, smem, st, sc, S, pk, srec, nsamp, d_nsamp, gdec,     \
                                                                    g_feat, g_offset, ROWS, g_mlp, cg);        \
     } while (0)
     if (wgrad_fused(S)) {

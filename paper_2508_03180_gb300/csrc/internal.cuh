@@ -297,23 +297,17 @@ long long resident_ctas(const void *kernel, int threads);
 cudaError_t set_sort_fault(bool on);
 cudaError_t set_tc_fault(bool on);  // the tensor-core decode's completion wait runs out (DGS_FAULT_TC_WAIT)
 
-// Programmatic dependent launch: a kernel launched by launch_chained may begin while
-// its predecessor in the stream still runs, as soon as all of that one's blocks
-// have started, so its launch latency and block start-up overlap the
-// predecessor's tail (views: 256 x 256 134 -> 125 us, 1080p 488 -> 469, neural 720p
-// 330 -> 310).  Every such kernel calls chain_begin before it touches
-// global memory: it waits there until the predecessor has
-// completed and its writes are visible, and lets its own successor be launched.
-// A kernel before a blend only waits (chain_wait): blend blocks that are
-// placed while it still runs crowd on the SMs it has left, the longest lists
-// first (20,011 cells x 5, three 641 x 479 views: 850 us a step, 754 so).
+// Programmatic dependent launch: a kernel launched by launch_chained is set up while
+// its predecessor in the stream still runs, which hides its launch latency (views:
+// 256 x 256 134 -> 125 us, 1080p 488 -> 469, neural 720p 330 -> 310).  Every such
+// kernel calls chain_wait before it touches global memory: it waits there until the
+// predecessor has completed and its writes are visible.  No kernel lets its successor
+// begin earlier than that: blocks placed while the predecessor's last ones run
+// crowd on the SMs it has left (with the longest tile lists first, ragged
+// training steps took 850 us instead of 750), and take shared memory that it needs.
 // Not within a captured graph, whose own edges are cheap already (a served burst
 // of eight requests: 881 us plain, 917 us chained).
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_begin() {
-    chain_wait();
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
 // cluster: CTAs per cluster, or 0 for a launch without clusters (a launch in clusters
 // of one is not the same: blocks of one warp then start more slowly).
 struct ClusterSize { unsigned n; };

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(LOSS_T) k_loss_l1(const float *__restrict__ rg
 
 __global__ void __launch_bounds__(LOSS_T) k_loss_final(const float *__restrict__ partial, int nb, float inv_n,
                                                        float *__restrict__ loss) {
+    chain_wait();
     __shared__ float s[LOSS_T / 32];
     float acc = 0.f;
     for (int i = threadIdx.x; i < nb; i += LOSS_T) acc += partial[i];
@@ -162,7 +163,7 @@ void launch_loss_l1(const float *rgb, const float *target, int64_t n, float *dL,
                     float *loss, cudaStream_t st) {
     const float inv_n = n > 0 ? 1.0f / (float)n : 0.f;
     k_loss_l1<<<nblocks, LOSS_T, 0, st>>>(rgb, target, n, inv_n, dL, partial);
-    k_loss_final<<<1, LOSS_T, 0, st>>>(partial, nblocks, inv_n, loss);
+    launch_chained(k_loss_final, 1, LOSS_T, 0, st, partial, nblocks, inv_n, loss);
 }
 
 }  // namespace dgs

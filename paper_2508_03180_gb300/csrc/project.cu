@@ -167,6 +167,7 @@ __global__ void __launch_bounds__(128) k_project_fwd_table(const ViewDesc *__res
 __global__ void k_cell_v_grad(const ViewDesc *__restrict__ views, int n_views, SceneDev sc,
                               const float *__restrict__ gv, float *__restrict__ g_cell_v, float *__restrict__ g_vsh,
                               float *__restrict__ g_center) {
+    chain_wait();
     const long long N = sc.N;
     const int Cv = sc.vsh ? (sc.v_sh_degree + 1) * (sc.v_sh_degree + 1) : 0;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
@@ -223,7 +224,7 @@ void launch_project_fwd(const ViewDesc *views, int n_views, int slot, const Scen
 void launch_cell_v_grad(const ViewDesc *views, int n_views, const SceneDev &sc, const float *gv, float *g_cell_v,
                         float *g_vsh, float *g_center, cudaStream_t st) {
     if (sc.N == 0 || (!g_cell_v && !g_vsh && !g_center)) return;
-    k_cell_v_grad<<<grid_for(sc.N, 128), 128, 0, st>>>(views, n_views, sc, gv, g_cell_v, g_vsh, g_center);
+    launch_chained(k_cell_v_grad, grid_for(sc.N, 128), 128, 0, st, views, n_views, sc, gv, g_cell_v, g_vsh, g_center);
 }
 
 void launch_gauss_bin(const ViewDesc *views, int n_views, const SceneDev &sc, const BlendParams &bp, bool wsr,
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(128) k_project_bwd_geom(const ViewDesc *__rest
                                                      float *__restrict__ g_scale,
                                                      float *__restrict__ g_log_scale, float *__restrict__ g_quat,
                                                      float *__restrict__ g_logit) {
-    chain_begin();
+    chain_wait();
     const long long G = sc.G;
     const int K = sc.K;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < G; g += (long long)gridDim.x * blockDim.x) {
@@ -478,6 +479,7 @@ __global__ void __launch_bounds__(128) k_project_bwd_neural(const ViewDesc *__re
                                                             SceneDev sc, const uint32_t *__restrict__ count,
                                                             BlendParams bp, const float *__restrict__ dec,
                                                             const float *__restrict__ g2d, float *__restrict__ gdec) {
+    chain_wait();
     const long long G = sc.G;
     const int K = sc.K;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < G; g += (long long)gridDim.x * blockDim.x) {
@@ -528,7 +530,7 @@ __global__ void __launch_bounds__(COL_T) k_project_bwd_colour(const ViewDesc *__
                                                               const float *__restrict__ g2d, float *__restrict__ g_mean,
                                                               float *__restrict__ g_sh) {
     __shared__ float s_acc[48 * COL_LD];  // dL/dk[c * 3 + ch] of thread t at [c * 3 + ch][t]
-    chain_begin();
+    chain_wait();
     const long long G = sc.G;
     const int K = sc.K, C = (sc.sh_degree + 1) * (sc.sh_degree + 1), row = 3 * C;
     const int t = threadIdx.x;
@@ -627,7 +629,7 @@ void launch_project_bwd_neural(const ViewDesc *views, int n_views, int slot, con
                                const BlendParams &bp, const float *dec, const float *g2d, float *gdec,
                                cudaStream_t st) {
     if (sc.G == 0) return;
-    k_project_bwd_neural<<<grid_for(sc.G, 128), 128, 0, st>>>(views, n_views, slot, sc, count, bp, dec, g2d, gdec);
+    launch_chained(k_project_bwd_neural, grid_for(sc.G, 128), 128, 0, st, views, n_views, slot, sc, count, bp, dec, g2d, gdec);
 }
 
 void launch_project_bwd(const ViewDesc *views, int n_views, int slot, const SceneDev &sc, const uint32_t *count,

@@ -8,6 +8,8 @@
   a valid outcome of the stopping rule (relative slack 1e-3 on T); the
   oracle's own counts may differ on at most 0.01% of pixels
 """
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -129,6 +131,20 @@ def test_cell_batches(rctx, K):
     sc = synth.make_scene(max(8, 900 // K), K, synth._box(-1, 1), 0.05, 0.4, 1, seed=40 + K)
     sc.g_logit[:] += 2.0
     _render_and_check(rctx, sc, [synth.small_camera(75, 50), synth.small_camera(64, 48)])
+
+
+@pytest.mark.parametrize("W,H", [(768, 512), (784, 512)])
+def test_sub_tile_sizes_give_the_same_image(rctx, W, H):
+    """1536 tiles, and one column of tiles more (the larger sub-tiles): the common
+    pixels of both images are equal bit for bit, and right."""
+    sc = synth.scene_small(n_cells=500)
+    sid = rctx.upload_scene(sc)
+    wide = synth.small_camera(784, 512)
+    cut = dataclasses.replace(wide, W=W, H=H)
+    a = rctx.render(sid, [wide])[0].view(3, 512, 784)[:, :, :W].clone()
+    b = rctx.render(sid, [cut])[0].view(3, H, W)
+    assert torch.equal(a, b)
+    rctx.release_scene(sid)
 
 
 def test_no_dilation_and_a_gaussian_of_no_extent():
