@@ -87,6 +87,14 @@ constexpr int FWD_PPL = 4;
 // exp2 of its negation is +0
 constexpr float kFar = 1e18f;
 constexpr int FWD_SUB = kTile / (2 * FWD_PPL);  // sub-tiles per tile
+// Up to this many tiles the forward takes 16x4 sub-tiles (two pixels per lane) instead:
+// with fewer than five 16x8 warps a scheduler, a view takes as long as its longest
+// list's chain of latencies, and the smaller sub-tile's list has fewer Gaussians in
+// reach (16x8 / 16x4, us: 256x256 of 2,048 x 8 46 / 31, 320x240 of 20,000 x 8 141 / 88,
+// 640x480 of 20,000 x 10 over three decades 71 / 59, 800x600 66 / 63); from about 2,500 tiles
+// its extra instructions count (1280x720 of 60,000 x 10 163 / 182, 1080p of 100,000 x 10
+// 279 / 342).  Per pixel both do the same operations in the same order.
+constexpr int kFewTiles = 1536;
 constexpr int fwd_minb(bool var) { return var ? 24 : 32; }  // (the variants spill at 64 registers)
 
 // VAR: the variant flags and background weight are live (dgs_config.flags,
@@ -287,7 +295,7 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
     }
 }
 
-template <int KT, bool VAR>
+template <int KT, int PPL, bool VAR>
 __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd(const ViewDesc *__restrict__ views, int n_views,
                                                   const uint32_t *__restrict__ order,
                                                   const uint2 *__restrict__ ranges, const uint32_t *__restrict__ cells,
@@ -296,7 +304,7 @@ __global__ void __launch_bounds__(WT, fwd_minb(VAR)) k_blend_fwd(const ViewDesc 
                                                   float *__restrict__ out_D, int *__restrict__ out_nd) {
     __shared__ float4 s_rec[FSTAGE][kBatchF4];
     chain_wait();
-    blend_fwd_unit<KT, FWD_PPL, VAR>(blockIdx.x, views, n_views, order, ranges, cells, rec, bp, out_rgb, out_rgb2, out_D, out_nd,
+    blend_fwd_unit<KT, PPL, VAR>(blockIdx.x, views, n_views, order, ranges, cells, rec, bp, out_rgb, out_rgb2, out_D, out_nd,
                                 s_rec);
 }
 
@@ -371,21 +379,26 @@ void launch_blend_fwd(const ViewDesc *views, int n_views, int total_tiles, const
 #undef DGS_PULL
         return;
     }
-    const unsigned grid = (unsigned)total_tiles * FWD_SUB;
-#define DGS_FWD(KV, VV)                                                                                      \
-    launch_chained(k_blend_fwd<KV, VV>, grid, WT, 0, st, views, n_views, order, ranges, tile_cells, rec, bp, out_rgb, out_rgb2, \
-                   out_D, out_nd)
+#define DGS_FWD(KV, PV, VV)                                                                                  \
+    launch_chained(k_blend_fwd<KV, PV, VV>, (unsigned)total_tiles * (kTile / (2 * PV)), WT, 0, st, views, n_views, order, \
+                   ranges, tile_cells, rec, bp, out_rgb, out_rgb2, out_D, out_nd)
     if (blend_variants(bp)) {
         switch (K_all) {
-            case 8: DGS_FWD(8, true); break;
-            case 10: DGS_FWD(10, true); break;
-            default: DGS_FWD(0, true); break;
+            case 8: DGS_FWD(8, FWD_PPL, true); break;
+            case 10: DGS_FWD(10, FWD_PPL, true); break;
+            default: DGS_FWD(0, FWD_PPL, true); break;
+        }
+    } else if (total_tiles <= kFewTiles) {
+        switch (K_all) {
+            case 8: DGS_FWD(8, 2, false); break;
+            case 10: DGS_FWD(10, 2, false); break;
+            default: DGS_FWD(0, 2, false); break;
         }
     } else {
         switch (K_all) {
-            case 8: DGS_FWD(8, false); break;
-            case 10: DGS_FWD(10, false); break;
-            default: DGS_FWD(0, false); break;
+            case 8: DGS_FWD(8, FWD_PPL, false); break;
+            case 10: DGS_FWD(10, FWD_PPL, false); break;
+            default: DGS_FWD(0, FWD_PPL, false); break;
         }
     }
 #undef DGS_FWD
