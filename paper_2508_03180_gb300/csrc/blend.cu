@@ -87,14 +87,16 @@ constexpr int FWD_PPL = 4;
 // exp2 of its negation is +0
 constexpr float kFar = 1e18f;
 constexpr int FWD_SUB = kTile / (2 * FWD_PPL);  // sub-tiles per tile
-// Up to this many tiles the forward takes 16x4 sub-tiles (two pixels per lane) instead:
-// with fewer than five 16x8 warps a scheduler, a view takes as long as its longest
+// Up to this many tiles the kernels take 16x4 sub-tiles (two pixels per lane) instead:
+// with fewer than eight 16x8 warps a scheduler, a view takes as long as its longest
 // list's chain of latencies, and the smaller sub-tile's list has fewer Gaussians in
-// reach (16x8 / 16x4, us: 256x256 of 2,048 x 8 46 / 31, 320x240 of 20,000 x 8 141 / 88,
-// 640x480 of 20,000 x 10 over three decades 71 / 59, 800x600 66 / 63); from about 2,500 tiles
-// its extra instructions count (1280x720 of 60,000 x 10 163 / 182, 1080p of 100,000 x 10
-// 279 / 342).  Per pixel both do the same operations in the same order.
-constexpr int kFewTiles = 1536;
+// reach (one view, 16x8 / 16x4, us: forward 256x256 of 2,048 x 8 46 / 31, 320x240 of
+// 20,000 x 8 141 / 88, 640x480 of 20,000 x 10 over three decades 71 / 59, 1024x576 of
+// 12,345 x 7 92 / 76; adjoint 124 / 79, 376 / 228, 185 / 145, and 960x540 186 / 159); at
+// 3,600 tiles its extra instructions count (1280x720 of 60,000 x 10: 163 / 182 and
+// 402 / 466; 20,011 x 5, 3,690 tiles: equal, and 353 / 360).  Per pixel both do the same
+// operations in the same order.
+constexpr int kFewTiles = 2304;
 constexpr int fwd_minb(bool var) { return var ? 24 : 32; }  // (the variants spill at 64 registers)
 
 // VAR: the variant flags and background weight are live (dgs_config.flags,
@@ -606,22 +608,33 @@ __device__ __forceinline__ int grad_slot(int j) { return j < 5 ? j : j + 1; }
 // per cell and sub-tile); two Gaussians per lane (half the factor loads): 5.62 ms,
 // its registers leave 16 warps an SM.
 constexpr int BWD_PPL = 4;
-constexpr int BWD_ROWS = 2 * BWD_PPL;
-constexpr int BWD_SUB = kTile / BWD_ROWS;  // sub-tiles per tile
 // Resident one-warp CTAs per SM the register budget is set for: 22 are what the
 // shared memory of K = 10 admits (80 registers; 20 at 96 registers is 4% slower
 // on the 1M-Gaussian step).  With dL/dv_n's sums 80 registers spill: 20 there
 // (0.43 against 0.47 ms on 20,011 cells x 5, three 641 x 479 views).
 constexpr int bwd_minb(bool wv) { return wv ? 20 : 22; }
 
-// float4s of shared memory: records [NSTAGE][3 K], G' rows [K][32] (a lane's
-// pixels q = 0..3), v T_n (e0, e1) and v T_n (e2, eD) [2][32] each, -v S_n
-// [32], and the Gaussian of every row (K ints)
-__host__ __device__ constexpr int bwd_smem_f4(int K) {
-    return NSTAGE * kRecF4 * K + WT * K + 4 * WT + WT + (K + 3) / 4;
+// float4s of shared memory: records [NSTAGE][3 K], G' rows [K][32] (a lane's PPL
+// pixels), v T_n (e0, e1) and v T_n (e2, eD) [PPL / 2][32] each, -v S_n
+// [32] (PPL), and the Gaussian of every row (K ints)
+__host__ __device__ constexpr int bwd_smem_f4(int K, int PPL) {
+    return NSTAGE * kRecF4 * K + WT * K * PPL / 4 + WT * PPL + WT * PPL / 4 + (K + 3) / 4;
 }
 
-template <int KT, bool VAR, bool WV>
+// A lane's pixels in shared memory, one pair per lane row: 16 or 8 bytes.
+template <int NR> struct RowPairs;
+template <> struct RowPairs<2> {
+    using T = float4;
+    static __device__ __forceinline__ T pack(const float2 (&v)[2]) { return make_float4(v[0].x, v[0].y, v[1].x, v[1].y); }
+    static __device__ __forceinline__ float2 row(T t, int rr) { return rr == 0 ? make_float2(t.x, t.y) : make_float2(t.z, t.w); }
+};
+template <> struct RowPairs<1> {
+    using T = float2;
+    static __device__ __forceinline__ T pack(const float2 (&v)[1]) { return v[0]; }
+    static __device__ __forceinline__ float2 row(T t, int) { return t; }
+};
+
+template <int KT, int PPL, bool VAR, bool WV>
 __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *__restrict__ views, int n_views,
                                                   const uint32_t *__restrict__ order,
                                                   const uint2 *__restrict__ ranges, const uint32_t *__restrict__ cells,
@@ -632,21 +645,22 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
     extern __shared__ float4 s_bwd[];
     chain_wait();
     const int lane = threadIdx.x;
-    const int tile = (int)order[blockIdx.x / BWD_SUB], sub = blockIdx.x % BWD_SUB;
+    constexpr int NR = PPL / 2, ROWS = 2 * PPL, NSUB = kTile / ROWS;  // rows per lane (pixel mapping as in the forward)
+    using Pairs = RowPairs<NR>;
+    const int tile = (int)order[blockIdx.x / NSUB], sub = blockIdx.x % NSUB;
     const int vi = find_view(views, n_views, tile);
     const ViewDesc &V = views[vi];
     const int K = KT > 0 ? KT : V.K;
     const int per = kRecF4 * K;
     float4 *const s_rec = s_bwd;                    // [NSTAGE][per]
-    float4 *const s_G = s_rec + NSTAGE * per;       // [K][WT]
-    float4 *const s_F01 = s_G + WT * K;             // [2][WT]
-    float4 *const s_F2D = s_F01 + 2 * WT;           // [2][WT]
-    float4 *const s_nS = s_F2D + 2 * WT;            // [WT]
+    typename Pairs::T *const s_G = reinterpret_cast<typename Pairs::T *>(s_rec + NSTAGE * per);  // [K][WT]
+    float4 *const s_F01 = reinterpret_cast<float4 *>(s_G + WT * K);  // [NR][WT]
+    float4 *const s_F2D = s_F01 + NR * WT;                           // [NR][WT]
+    typename Pairs::T *const s_nS = reinterpret_cast<typename Pairs::T *>(s_F2D + NR * WT);  // [WT]
     int *const s_k = reinterpret_cast<int *>(s_nS + WT);  // [K]
     const int local = tile - V.tile_base;
     const int tx = local % V.Tx, ty = local / V.Tx;
-    const float bx0 = (float)(tx * kTile), by0 = (float)(ty * kTile + BWD_ROWS * sub);
-    constexpr int PPL = BWD_PPL, NR = PPL / 2;  // rows per lane (pixel mapping as in the forward)
+    const float bx0 = (float)(tx * kTile), by0 = (float)(ty * kTile + ROWS * sub);
     int xs[2], ys[NR];
     float pxs[2], pys[NR];
 #pragma unroll
@@ -656,7 +670,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-        ys[r] = ty * kTile + BWD_ROWS * sub + lane_row(lane, r);
+        ys[r] = ty * kTile + ROWS * sub + lane_row(lane, r);
         pys[r] = (float)ys[r] + 0.5f;
     }
     const long long HW = (long long)V.W * V.H;
@@ -734,7 +748,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
         buf = buf == NSTAGE - 1 ? 0 : buf + 1;
         const float v = r[2].w;
         // the Gaussians that reach the sub-tile: row i of G' belongs to the i-th
-        const unsigned hits = __ballot_sync(0xffffffffu, lane < K && touches_rows(r[kRecF4 * lane], bx0, by0, (float)BWD_ROWS));
+        const unsigned hits = __ballot_sync(0xffffffffu, lane < K && touches_rows(r[kRecF4 * lane], bx0, by0, (float)ROWS));
         const int rows = __popc(hits);
         if ((hits >> lane) & 1u) s_k[__popc(hits & ((1u << lane) - 1u))] = lane;
         // With v <= 1 every 1 - v alpha is at least 1 - alpha_max, and the zero
@@ -757,7 +771,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
         const float amin = VAR && (bp.flags & DGS_FLAG_ALPHA_SKIP) ? 1.0f / 255.0f : 0.0f;
 #pragma unroll
         for (int rr = 0; rr < NR; ++rr) { X[rr] = make_float2(0.f, 0.f); P[rr] = make_float2(1.0f, 1.0f); }
-        float4 *row = s_G + lane;
+        typename Pairs::T *row = s_G + lane;
 #pragma unroll 1
         for (unsigned mask = hits; mask; mask &= mask - 1, row += WT) {
             const int k = __ffs(mask) - 1;
@@ -807,7 +821,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
                     gq[rr].y = n < nd[2 * rr + 1] ? gq[rr].y : 0.f;
                 }
             }
-            *row = make_float4(gq[0].x, gq[0].y, gq[1].x, gq[1].y);
+            *row = Pairs::pack(gq);
         }
         // per-pixel transmittance bookkeeping (S_n includes x_n; a pixel past its
         // last cell has T = S = 0), and the factors of pass 2.  The cell term of
@@ -834,7 +848,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
             nS[rr] = WV ? make_float2(-S[rr].x, -S[rr].y) : __fmul2_rn(make_float2(-v, -v), S[rr]);
         }
         float dv = dv2.x + dv2.y;
-        s_nS[lane] = make_float4(nS[0].x, nS[0].y, nS[1].x, nS[1].y);
+        s_nS[lane] = Pairs::pack(nS);
         __syncwarp();
         const uint32_t cellid = __ldg(cells + e);
         float *gbase = g2d + (V.rec_base + (long long)cellid * K) * kGradF;
@@ -847,7 +861,7 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
             const bool live = SPLIT > 1 || c + g < rows;
             const int i = live ? c + g : c;
             const int k = s_k[i];
-            const float4 *Gr = s_G + i * WT + w8;
+            const typename Pairs::T *Gr = s_G + i * WT + w8;
             const float4 r0 = r[3 * k], r1 = r[3 * k + 1], r2 = r[3 * k + 2];
             const float op = r1.w;
             const float py0 = by0 + 0.5f + (float)part;
@@ -855,16 +869,16 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
             a.dop = a.Y = a.Q = a.C0 = a.C1 = a.C2 = a.dv = make_float2(0.f, 0.f);
             auto sweep = [&](auto clamp) {
 #pragma unroll
-                for (int t = 0; t < 4 / SPLIT; ++t) {  // rows j and j + 4
+                for (int t = 0; t < 4 / SPLIT; ++t) {  // rows j and (with two rows per lane) j + 4
                     const int at = 8 * (SPLIT * t + part) + w8;
-                    const float4 g4 = Gr[at - w8], n4 = s_nS[at];
+                    const typename Pairs::T gp = Gr[at - w8], np = s_nS[at];
 #pragma unroll
                     for (int rr = 0; rr < NR; ++rr) {
                         const float4 fa = s_F01[rr * WT + at], fb = s_F2D[rr * WT + at];
                         pair_grad2<decltype(clamp)::value, WV>(
-                            a, rr == 0 ? make_float2(g4.x, g4.y) : make_float2(g4.z, g4.w), make_float2(fa.x, fa.y),
+                            a, Pairs::row(gp, rr), make_float2(fa.x, fa.y),
                             make_float2(fa.z, fa.w), make_float2(fb.x, fb.y), make_float2(fb.z, fb.w),
-                            rr == 0 ? make_float2(n4.x, n4.y) : make_float2(n4.z, n4.w),
+                            Pairs::row(np, rr),
                             (py0 + (float)(SPLIT * t + 4 * rr)) - r0.y, op, v, -v * op, r2, bp.alpha_max);
                     }
                 }
@@ -924,28 +938,34 @@ void launch_blend_bwd(const ViewDesc *views, int n_views, int total_tiles, const
                       const float *D, const int *nd, const float *dL_drgb, float *g2d, float *g_cell_v,
                       cudaStream_t st) {
     if (total_tiles == 0) return;
-    const unsigned grid = (unsigned)total_tiles * BWD_SUB;
-    const size_t smem = sizeof(float4) * bwd_smem_f4(K_all);
-#define DGS_BWD(KV, VV)                                                                                          \
+#define DGS_BWD(KV, PV, VV)                                                                                      \
     do {                                                                                                        \
+        const unsigned grid = (unsigned)total_tiles * (kTile / (2 * PV));                                       \
+        const size_t smem = sizeof(float4) * bwd_smem_f4(K_all, PV);                                            \
         if (g_cell_v)                                                                                           \
-            launch_chained(k_blend_bwd<KV, VV, true>, grid, WT, smem, st, views, n_views, order, ranges, tile_cells, \
+            launch_chained(k_blend_bwd<KV, PV, VV, true>, grid, WT, smem, st, views, n_views, order, ranges, tile_cells, \
                            rec, bp, rgb, D, nd, dL_drgb, g2d, g_cell_v);                                        \
         else                                                                                                    \
-            launch_chained(k_blend_bwd<KV, VV, false>, grid, WT, smem, st, views, n_views, order, ranges, tile_cells, \
+            launch_chained(k_blend_bwd<KV, PV, VV, false>, grid, WT, smem, st, views, n_views, order, ranges, tile_cells, \
                            rec, bp, rgb, D, nd, dL_drgb, g2d, nullptr);                                         \
     } while (0)
     if (blend_variants(bp)) {
         switch (K_all) {
-            case 8: DGS_BWD(8, true); break;
-            case 10: DGS_BWD(10, true); break;
-            default: DGS_BWD(0, true); break;
+            case 8: DGS_BWD(8, BWD_PPL, true); break;
+            case 10: DGS_BWD(10, BWD_PPL, true); break;
+            default: DGS_BWD(0, BWD_PPL, true); break;
+        }
+    } else if (total_tiles <= kFewTiles) {
+        switch (K_all) {
+            case 8: DGS_BWD(8, 2, false); break;
+            case 10: DGS_BWD(10, 2, false); break;
+            default: DGS_BWD(0, 2, false); break;
         }
     } else {
         switch (K_all) {
-            case 8: DGS_BWD(8, false); break;
-            case 10: DGS_BWD(10, false); break;
-            default: DGS_BWD(0, false); break;
+            case 8: DGS_BWD(8, BWD_PPL, false); break;
+            case 10: DGS_BWD(10, BWD_PPL, false); break;
+            default: DGS_BWD(0, BWD_PPL, false); break;
         }
     }
 #undef DGS_BWD

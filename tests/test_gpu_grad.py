@@ -169,17 +169,21 @@ def test_gradients_beyond_the_jacobian_clamp(rctx):
 
 
 @pytest.mark.parametrize("K", [1, 2, 3, 5, 6, 7, 8, 10, 13, 32])
-@pytest.mark.parametrize("opaque", [False, True])
-def test_gradients_per_cell_row_counts(rctx, K, opaque):
+@pytest.mark.parametrize("opaque,large", [(False, False), (True, False), (False, True), (True, True)])
+def test_gradients_per_cell_row_counts(rctx, K, opaque, large):
     """The adjoint's second pass takes a cell's Gaussians four at a time, the
     last one or two with more lanes each: every remainder, the compiled and the
     run-time K, with opacities below the alpha clamp and beyond it (their pixels
-    below the clamp keep a gradient), and with dL/dv_n requested and not."""
+    below the clamp keep a gradient), and with dL/dv_n requested and not.  large: a
+    second view, with nothing in it, takes the batch beyond 2304 tiles, where the
+    sub-tiles are 16x8 instead of 16x4."""
     sc = synth.make_scene(24, K, synth._box(-0.5, 0.5), 0.1, 0.4, 1, seed=100 + K)
     sc.cell_v[:] = np.random.default_rng(K).uniform(0.3, 1.0, sc.N).astype(np.float32)
     if opaque:
         sc.g_logit[::2] = 7.0  # sigma = 0.9991
     cams = synth.sphere_cameras(1, 3.0, 61, 43, seed0=9)
+    if large:
+        cams.append(synth.look_at((0.0, -3.0, 0.0), (0.0, -6.0, 0.0), 784, 768, 60.0))
     _, dl, gr, gs, _ = _grads(rctx, sc, cams, seed=K)
     ref, _ = _oracle_grads(sc, cams, dl, gs)
     names = (("g_mean", "mean"), ("g_scale", "scale"), ("g_quat", "quat"), ("g_logit", "logit"), ("g_sh", "sh"))

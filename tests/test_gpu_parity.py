@@ -133,16 +133,15 @@ def test_cell_batches(rctx, K):
     _render_and_check(rctx, sc, [synth.small_camera(75, 50), synth.small_camera(64, 48)])
 
 
-@pytest.mark.parametrize("W,H", [(768, 512), (784, 512)])
-def test_sub_tile_sizes_give_the_same_image(rctx, W, H):
-    """1536 tiles, and one column of tiles more (the larger sub-tiles): the common
-    pixels of both images are equal bit for bit, and right."""
+@pytest.mark.parametrize("W", [768, 784])
+def test_sub_tile_sizes_give_the_same_image(rctx, W):
+    """2304 tiles, and a column of tiles more (the larger sub-tiles): the common
+    pixels of both images are equal bit for bit."""
     sc = synth.scene_small(n_cells=500)
     sid = rctx.upload_scene(sc)
-    wide = synth.small_camera(784, 512)
-    cut = dataclasses.replace(wide, W=W, H=H)
-    a = rctx.render(sid, [wide])[0].view(3, 512, 784)[:, :, :W].clone()
-    b = rctx.render(sid, [cut])[0].view(3, H, W)
+    wide = synth.small_camera(784, 768)
+    a = rctx.render(sid, [wide])[0].view(3, 768, 784)[:, :, :W].clone()
+    b = rctx.render(sid, [dataclasses.replace(wide, W=W)])[0].view(3, 768, W)
     assert torch.equal(a, b)
     rctx.release_scene(sid)
 
