@@ -81,6 +81,10 @@ struct CellFeed {
 // 2,048 cells x 8 at 256 x 256, one warp a scheduler: 74 -> 46 us.  Weighting every
 // alpha by v_n T_n instead of the cell's sums (no sums to clear and add) takes
 // another 3%, but rounds N and D more often; 72 registers and 28 CTAs an SM: 2.00 ms.
+// Of 74 instructions per visited Gaussian then left, the minimum with alpha_max is
+// needed only where an opacity reaches it (a batch without one takes a copy of the
+// loop that has none), and offsets and row squares are formed in pairs: 1.95 -> 1.85 ms.
+// (In the adjoint's first pass neither pays: 5.10 -> 5.11 and 5.21 ms.)
 constexpr int FWD_PPL = 4;
 // an offset from the Gaussian's centre that no box reaches: s1 or s2 then
 // squares to at least ~1e18 (the record's L entries are far above 1e-9), and
@@ -133,6 +137,7 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
     const int K = KT > 0 ? KT : V.K;
     const uint32_t CB = batch_cells(K);
     const unsigned kmask = K == 32 ? 0xffffffffu : (1u << K) - 1u;
+    const unsigned kinv = (65535u + (unsigned)K) / (unsigned)K;  // l / K = l kinv >> 16 for l < 32
     const uint2 rg = ranges[tile];
 
     // A pixel is done once T < eps (eps >= 0): T is then not needed any more and holds,
@@ -171,9 +176,13 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
         // Gaussians whose box holds the whole sub-tile: no per-pixel test
         const unsigned full = VAR ? 0u : __ballot_sync(0xffffffffu, mine && covers_rows(rl, bx0, by0, (float)ROWS));
         const float amin = VAR && (bp.flags & DGS_FLAG_ALPHA_SKIP) ? 1.0f / 255.0f : 0.0f;
+        // an opacity below the clamp keeps every alpha there (G' <= 1, to the last
+        // bits): batches without a larger one in reach go without the minimum
+        const bool clamp = VAR || (hits & __ballot_sync(0xffffffffu, !(r[kRecF4 * lane + 1].w < 0.9999f * bp.alpha_max))) != 0u;
+        auto blend_batch = [&](auto with_clamp) {
         while (hits) {
             // the next cell with a Gaussian in reach: cell c of the batch, its Gaussians' lanes in mask
-            const int c = (__ffs(hits) - 1) / K;
+            const int c = KT > 0 ? (__ffs(hits) - 1) / K : (int)((unsigned)(__ffs(hits) - 1) * kinv >> 16);
             unsigned mask = hits & (kmask << (c * K));
             hits ^= mask;
             const float v = r[kRecF4 * (c * K) + 2].w;
@@ -187,11 +196,20 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
             for (; mask; mask &= mask - 1) {
                 const int k = __ffs(mask) - 1;
                 const float4 r0 = r[3 * k], r1 = r[3 * k + 1], r2 = r[3 * k + 2];
-                float dx[2], dy[NR];
-#pragma unroll
-                for (int c2 = 0; c2 < 2; ++c2) dx[c2] = pxs[c2] - r0.x;
-#pragma unroll
-                for (int rr = 0; rr < NR; ++rr) dy[rr] = pys[rr] - r0.y;
+                // offsets of the two columns, and of the rows (packed where there are two)
+                float dx[2], dy[NR], s22[NR];
+                {
+                    const float2 d = __fadd2_rn(make_float2(pxs[0], pxs[1]), make_float2(-r0.x, -r0.x));
+                    dx[0] = d.x;
+                    dx[1] = d.y;
+                }
+                if (NR == 2) {
+                    const float2 d = __fadd2_rn(make_float2(pys[0], pys[NR - 1]), make_float2(-r0.y, -r0.y));
+                    dy[0] = d.x;
+                    dy[NR - 1] = d.y;
+                } else {
+                    dy[0] = pys[0] - r0.y;
+                }
                 bool h[PPL];
                 if (VAR || !((full >> k) & 1u)) {  // (else every pixel of the sub-tile is in the box)
                     bool hx[2], hy[NR];
@@ -213,19 +231,24 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
                     }
                 }
                 const float2 pdx = __fmul2_rn(make_float2(r1.x, r1.x), make_float2(dx[0], dx[1]));
+                {
+                    const float2 s2 = __fmul2_rn(make_float2(r1.z, r1.z), make_float2(dy[0], dy[NR - 1]));
+                    const float2 q = __fmul2_rn(s2, s2);
+                    s22[0] = q.x;
+                    s22[NR - 1] = NR == 2 ? q.y : q.x;
+                }
 #pragma unroll
                 for (int rr = 0; rr < NR; ++rr) {
                     const float dyq = dy[rr];
-                    const float s2 = r1.z * dyq, s22 = s2 * s2;
                     const float2 s1 = __ffma2_rn(make_float2(r1.y, r1.y), make_float2(dyq, dyq), pdx);
-                    const float2 qd = __ffma2_rn(s1, s1, make_float2(s22, s22));
+                    const float2 qd = __ffma2_rn(s1, s1, make_float2(s22[rr], s22[rr]));
                     float2 al = __fmul2_rn(make_float2(r1.w, r1.w), make_float2(ex2_approx(-qd.x), ex2_approx(-qd.y)));
                     // a pixel the Gaussian does not reach (or, with the alpha skip, an
                     // alpha below 1/255) takes alpha 0: every update below leaves it unchanged
                     if (VAR) {
                         al.x = h[2 * rr] && al.x >= amin ? fminf(al.x, bp.alpha_max) : 0.f;
                         al.y = h[2 * rr + 1] && al.y >= amin ? fminf(al.y, bp.alpha_max) : 0.f;
-                    } else {
+                    } else if (decltype(with_clamp)::value) {
                         al.x = fminf(al.x, bp.alpha_max);
                         al.y = fminf(al.y, bp.alpha_max);
                     }
@@ -256,6 +279,8 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
                 T[2 * rr + 1] = d1 ? Tr.y : n1 ? end : Tn.y;
             }
         }
+        };
+        if (clamp) blend_batch(std::true_type{}); else blend_batch(std::false_type{});
         __syncwarp();  // every lane is done with s_rec[buf] before it is refilled
     }
     cp_async_wait<0>();  // copies of entries past an early stop land before the buffers are reused

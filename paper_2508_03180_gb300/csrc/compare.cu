@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "blend.cuh"
 #include "runtime.h"
@@ -32,7 +33,9 @@ constexpr int CSUB = kTile / CROWS;  // sub-tiles per tile
 //          is not above d_min.
 // Bound by instruction issue.  Two pixels per lane in scalar arithmetic, branches
 // per pixel and records fetched through registers took 617 us for one 1080p view of
-// 1M Gaussians, 3.1M of them in tile lists twice (the whole call 992 -> 840 us).
+// 1M Gaussians, 476 this way (the whole call 992 -> 840 us); without the minimum with
+// alpha_max where no opacity reaches it and with paired offsets the call went from
+// 788 to 762.
 template <bool ALPHA>
 __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restrict__ views, int n_views,
                                                     const uint32_t *__restrict__ order,
@@ -86,33 +89,39 @@ __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restri
         const bool mine = lane < feed.count(base, 1);
         const float4 rl = r[kRecF4 * lane];
         const unsigned full = __ballot_sync(0xffffffffu, mine && covers_rows(rl, bx0, by0, (float)CROWS));
-        for (unsigned mask = __ballot_sync(0xffffffffu, mine && touches_rows(rl, bx0, by0, (float)CROWS)); mask;
-             mask &= mask - 1) {
+        const unsigned hits = __ballot_sync(0xffffffffu, mine && touches_rows(rl, bx0, by0, (float)CROWS));
+        // (batches whose opacities are all below the clamp go without the minimum, as in the hybrid)
+        const bool clamp = (hits & __ballot_sync(0xffffffffu, !(r[kRecF4 * lane + 1].w < 0.9999f * bp.alpha_max))) != 0u;
+        auto blend_batch = [&](auto with_clamp) {
+        for (unsigned mask = hits; mask; mask &= mask - 1) {
             const int k = __ffs(mask) - 1;
             const float4 r0 = r[3 * k], r1 = r[3 * k + 1], r2 = r[3 * k + 2];
-            const float dx0 = px - r0.x, dx1 = (px + 8.f) - r0.x;
+            const float2 dx = __fadd2_rn(make_float2(px, px + 8.f), make_float2(-r0.x, -r0.x));
+            const float2 dy2 = __fadd2_rn(make_float2(py, py + 4.f), make_float2(-r0.y, -r0.y));
             bool h[2 * NR];  // the pixels that take the Gaussian
 #pragma unroll
             for (int q = 0; q < 2 * NR; ++q) h[q] = true;
             if (!((full >> k) & 1u)) {
-                const bool hx0 = fabsf(dx0) <= r0.z, hx1 = fabsf(dx1) <= r0.z;
+                const bool hx0 = fabsf(dx.x) <= r0.z, hx1 = fabsf(dx.y) <= r0.z;
 #pragma unroll
                 for (int rr = 0; rr < NR; ++rr) {
-                    const bool hy = fabsf((py + 4.f * rr) - r0.y) <= r0.w;
+                    const bool hy = fabsf(rr == 0 ? dy2.x : dy2.y) <= r0.w;
                     h[2 * rr] = hx0 && hy;
                     h[2 * rr + 1] = hx1 && hy;
                 }
             }
-            const float2 pdx = __fmul2_rn(make_float2(r1.x, r1.x), make_float2(dx0, dx1));
+            const float2 pdx = __fmul2_rn(make_float2(r1.x, r1.x), dx);
+            const float2 s2 = __fmul2_rn(make_float2(r1.z, r1.z), dy2), s22 = __fmul2_rn(s2, s2);
 #pragma unroll
             for (int rr = 0; rr < NR; ++rr) {
-                const float dy = (py + 4.f * rr) - r0.y, s2 = r1.z * dy, s22 = s2 * s2;
+                const float dy = rr == 0 ? dy2.x : dy2.y, q = rr == 0 ? s22.x : s22.y;
                 const float2 s1 = __ffma2_rn(make_float2(r1.y, r1.y), make_float2(dy, dy), pdx);
-                const float2 qd = __ffma2_rn(s1, s1, make_float2(s22, s22));
+                const float2 qd = __ffma2_rn(s1, s1, make_float2(q, q));
                 float2 al = __fmul2_rn(make_float2(r1.w, r1.w), make_float2(ex2_approx(-qd.x), ex2_approx(-qd.y)));
                 const bool a0 = h[2 * rr] && !(ALPHA && X[rr].x < eps), a1 = h[2 * rr + 1] && !(ALPHA && X[rr].y < eps);
-                al.x = a0 ? fminf(al.x, bp.alpha_max) : 0.f;
-                al.y = a1 ? fminf(al.y, bp.alpha_max) : 0.f;
+                if (decltype(with_clamp)::value) al = make_float2(fminf(al.x, bp.alpha_max), fminf(al.y, bp.alpha_max));
+                al.x = a0 ? al.x : 0.f;
+                al.y = a1 ? al.y : 0.f;
                 const float2 w = __fmul2_rn(ALPHA ? X[rr] : make_float2(r2.w, r2.w), al);
                 C0[rr] = __ffma2_rn(w, make_float2(r2.x, r2.x), C0[rr]);
                 C1[rr] = __ffma2_rn(w, make_float2(r2.y, r2.y), C1[rr]);
@@ -124,6 +133,8 @@ __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restri
                 }
             }
         }
+        };
+        if (clamp) blend_batch(std::true_type{}); else blend_batch(std::false_type{});
         __syncwarp();  // every lane is done with s_rec[buf] before it is refilled
     }
     cp_async_wait<0>();
