@@ -983,7 +983,8 @@ dgs_status chain_forward(dgs_ctx *ctx, Workspace &ws, const std::vector<ChainVie
         } else {
             StageTimer t(ctx->prof, DGS_STAGE_PROJECT_FWD, st);
             launch_project_fwd(dv, V, k, sd, (const uint32_t *)ws.count.p, (const float *)ws.vview.p, bp,
-                               (float4 *)ws.rec.p, grad_buffers ? (float *)ws.g2d.p : nullptr, st);
+                               (float4 *)ws.rec.p, grad_buffers ? (float *)ws.g2d.p : nullptr,
+                               (const uint32_t *)ws.small.p + kSmallVisible, ws.n_entries, st);
         }
     }
     float *img = out_img ? out_img : (float *)ws.rgb.p;

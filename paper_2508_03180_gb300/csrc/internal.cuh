@@ -185,8 +185,10 @@ void launch_pair_offsets(const uint32_t *idx, const uint32_t *count, long long n
 
 // project.cu  (one launch per distinct scene of the chain: views whose
 // scene_slot differs from `slot` are skipped)
+// visible: the chain's visible entries of n_entries (view, cell) entries, on the device
 void launch_project_fwd(const ViewDesc *views, int n_views, int slot, const SceneDev &sc, const uint32_t *count,
-                        const float *vview, const BlendParams &bp, float4 *rec, float *g2d_zero, cudaStream_t st);
+                        const float *vview, const BlendParams &bp, float4 *rec, float *g2d_zero,
+                        const uint32_t *visible, long long n_entries, cudaStream_t st);
 // dL/dv per cell from the per-(view, cell) values gv of views [0, n_views)
 // (all of scene sc): g_cell_v[n] = sum over views (nullable), and for a
 // view-dependent v_n g_vsh[n][lm] = sum over views of gv Y_lm(d) where the

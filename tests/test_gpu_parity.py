@@ -290,6 +290,23 @@ def test_update_from_arrays_at_any_alignment(rctx, n_cells, sh, offset):
     rctx.release_scene(oid)
 
 
+def test_sparse_projection_equals_dense(rctx):
+    """A scene of 2.5M Gaussians seen from street level, most cells culled (the
+    projection that lists the kept Gaussians first), and the same view beside others that
+    see all of it (the direct one): the same image bit for bit."""
+    sc = synth.make_scene(249_100, 10, synth._ground_plane, 0.05, 0.5, 0, seed=2)
+    cam = synth.street_cameras(1, 320, 192, seed0=3)[0]
+    far = [synth.look_at((0.0, -900.0, 300.0 + i), (0.0, 0.0, 0.0), 48, 32, 60.0) for i in range(3)]
+    sid = rctx.upload_scene(sc)
+    alone, _, st = rctx.render(sid, [cam], stats=True)
+    assert 0 < st.visible_cells < sc.N // 2
+    alone = alone.clone()
+    both, _, st = rctx.render(sid, [cam] + far, stats=True)
+    assert st.visible_cells > 2 * sc.N
+    assert torch.equal(both[:alone.numel()], alone)
+    rctx.release_scene(sid)
+
+
 def test_more_than_65536_tiles(rctx):
     """An odd number of tile-sort passes (17 bits of tile number)."""
     sc = synth.scene_small(n_cells=400)
