@@ -17,10 +17,10 @@ namespace dgs {
 // the array is aligned, turned in shared memory (odd row stride: no bank conflicts) and
 // written as runs of consecutive rows per plane.  Bound by HBM: the five arrays of
 // 1M Gaussians at SH 3 (472 MB read and written) took 220 us in five launches of
-// 32-row blocks, 148 us now.
+// 32-row blocks, 148 us this way with divisions in the index arithmetic and 130 without.
 constexpr int PL_T = 256, PL_ELEMS = 4096;
 __global__ void __launch_bounds__(PL_T) k_rows_to_planes(const PlaneCopies C) {
-    __shared__ float t[PL_ELEMS + PL_ELEMS / 2];  // rows x (cols | 1): widest for two columns
+    __shared__ __align__(16) float t[PL_ELEMS + PL_ELEMS / 2];  // rows x (cols | 1): widest for two columns
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int64_t task = blockIdx.x; task < C.tasks; task += gridDim.x) {
         int a = 0;
@@ -31,22 +31,31 @@ __global__ void __launch_bounds__(PL_T) k_rows_to_planes(const PlaneCopies C) {
         const int nr = (int)min((int64_t)tr, P.rows - r0), ne = nr * cols;
         const float *src = P.src + r0 * cols;
         const uint32_t magic = cols > 1 ? (uint32_t)(((1ull << 32) + cols - 1) / cols) : 0u;
-        auto put = [&](int i, float v) {  // i / cols by the exact reciprocal (i, cols < 2^16)
-            const int r = cols > 1 ? (int)__umulhi((uint32_t)i, magic) : i;
-            t[r * ld + (i - r * cols)] = v;
-        };
+        // i / cols by the exact reciprocal (i, cols < 2^16); element i belongs at i, or with
+        // an even row length (and the odd stride) at i + row
+        auto row = [&](uint32_t i) { return cols > 1 ? __umulhi(i, magic) : i; };
         const int n4 = ((uintptr_t)P.src & 15) == 0 ? ne / 4 : 0;  // (r0 * cols is a multiple of 32)
+        if (cols & 1) {
 #pragma unroll 4
-        for (int i = tid; i < n4; i += PL_T) {
-            const float4 v = reinterpret_cast<const float4 *>(src)[i];
-            put(4 * i, v.x); put(4 * i + 1, v.y); put(4 * i + 2, v.z); put(4 * i + 3, v.w);
+            for (int i = tid; i < n4; i += PL_T) reinterpret_cast<float4 *>(t)[i] = reinterpret_cast<const float4 *>(src)[i];
+            for (int i = 4 * n4 + tid; i < ne; i += PL_T) t[i] = src[i];
+        } else {
+#pragma unroll 4
+            for (int i = tid; i < n4; i += PL_T) {
+                const float4 v = reinterpret_cast<const float4 *>(src)[i];
+                t[4 * i + row(4 * i)] = v.x;
+                t[4 * i + 1 + row(4 * i + 1)] = v.y;
+                t[4 * i + 2 + row(4 * i + 2)] = v.z;
+                t[4 * i + 3 + row(4 * i + 3)] = v.w;
+            }
+            for (int i = 4 * n4 + tid; i < ne; i += PL_T) t[i + row(i)] = src[i];
         }
-        for (int i = 4 * n4 + tid; i < ne; i += PL_T) put(i, src[i]);
         __syncthreads();
         // warp w: 32-row groups of the planes, group-major
         const int groups = (nr + 31) / 32;
+#pragma unroll 4
         for (int u = warp; u < groups * cols; u += PL_T / 32) {
-            const int g = u / cols, c = u - g * cols, r = 32 * g + lane;
+            const int g = (int)row(u), c = u - g * cols, r = 32 * g + lane;
             if (r < nr) P.dst[c * P.stride + r0 + r] = t[r * ld + c];
         }
         __syncthreads();
