@@ -773,16 +773,13 @@ def forward_chain(streaming, prof, steps, px, stats, scene, cnt, peaks, fp32_tfl
     return out
 
 
-def launches_per_step(stats, device_sized=True):
-    # kernels of one fwd+bwd step: cell projection 1; depth sort 2 + 4 passes; gather 1; scan 3;
-    # emit 1; tile sort 2 + ceil(bits/8) passes; ranges 1; projection 1; blend 1; loss 2;
-    # blend adjoint 1; projection adjoint 2 (geometry, then colour); a render without stats keeps
-    # the pair count on the device: + the pair-count clamp 1 and the tile sort's copy-back 1
-    # (which decides on the device whether the result needs it)
+def launches_per_step(stats):
+    # kernels of one fwd+bwd step: cell projection 1; depth sort 4 passes; pair offsets 1; emit 1;
+    # tile sort ceil(bits/8) passes; ranges 1; tile order 1; projection 1; blend 1; loss 2; blend
+    # adjoint 1; projection adjoint 2 (geometry, then colour)
     tiles = int(stats.num_tiles)
     bits = max(1, math.ceil(math.log2(max(2, tiles))))
-    return (1 + (2 + 4) + 1 + 3 + 1 + (2 + math.ceil(bits / 8)) + 1 + 1 + 1 + 2 + 1 + 2
-            + (2 if device_sized else 0))
+    return 1 + 4 + 1 + 1 + math.ceil(bits / 8) + 1 + 1 + 1 + 1 + 2 + 1 + 2
 
 
 if __name__ == "__main__":

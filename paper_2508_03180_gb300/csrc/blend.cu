@@ -31,12 +31,14 @@ constexpr float LN2 = 0.6931471805599453f;
 // as its own pixels are done.  KT > 0 fixes K at compile time.
 constexpr int WT = 32;  // threads per work unit
 
-// Records reach shared memory by asynchronous copies (cp.async, 16 bytes a
-// lane, one to three per lane for a cell), three cells deep: the copy of
+// The adjoint's records reach shared memory by asynchronous copies (cp.async, 16 bytes
+// a lane, one to three per lane for a cell), three cells deep: the copy of
 // entry e + 2 is issued while entry e is blended, so neither registers nor a
 // wait on the load's latency are spent on staging.  Every iteration commits one
 // copy group (empty past the list's end) and waits for all but the two
 // newest, which are the next two entries' (cp_async16 and friends: internal.cuh).
+// (The forward takes its cells in batches: CellBatches.  In the adjoint batches
+// were no faster, 5.16 -> 5.19 ms with one buffer and 5.28 with two.)
 constexpr int NSTAGE = 3;
 
 // Issue the copy of the records of cell `id` (per float4s) into dst.
