@@ -248,7 +248,7 @@ def test_radix_sort_pairs_stable(rctx, n, bits):
     assert np.array_equal(kd.cpu().numpy(), k32.numpy()[order])
 
 
-@pytest.mark.parametrize("n", [2, 1023, 1024, 1025, 9 * 1024 + 1, 65536, 65537])
+@pytest.mark.parametrize("n", [2, 1023, 1024, 1025, 9 * 1024 + 1, 262_144, 262_145])
 def test_radix_sort_partition_edges(rctx, n):
     """Around a small partition, one look-back of eight partitions, and the
     size at which the partitions grow."""
