@@ -134,6 +134,7 @@ void DevBuf::release() {
 Workspace::~Workspace() {
     for (DevBuf *b : all()) b->release();
     if (h_small) cudaFreeHost(h_small);
+    if (h_chain) cudaFreeHost(h_chain);
     if (h_views) cudaFreeHost(h_views);
     if (h_scenes) cudaFreeHost(h_scenes);
     if (h_sizes) cudaFreeHost(h_sizes);
@@ -825,8 +826,6 @@ static dgs_status run_binning(dgs_ctx *ctx, Workspace &ws, cudaStream_t st, bool
     const long long n = ws.n_entries;
     const long long n1 = std::max(1LL, n);
     dgs_status s;
-    if ((s = ws.small.ensure(kSmallBytes))) return s;
-    CK(cudaMemsetAsync(ws.small.p, 0, kSmallBytes, st));
     if ((s = ws.zkey.ensure(4 * n1)) || (s = ws.zval.ensure(4 * n1)) || (s = ws.rect.ensure(8 * n1)) ||
         (s = ws.depth.ensure(4 * n1)) || (s = ws.count.ensure(4 * n1)) || (s = ws.offs.ensure(4 * n1)) ||
         (s = ws.scan.ensure(4 * scan_scratch_words(n1))) || (s = ws.vview.ensure(4 * n1)) ||
@@ -842,10 +841,10 @@ static dgs_status run_binning(dgs_ctx *ctx, Workspace &ws, cudaStream_t st, bool
         return s;
     uint32_t *small = (uint32_t *)ws.small.p;
     const uint32_t *d_vis = small + kSmallVisible;  // entries that survive culling: the depth sort keeps those
-    const ViewDesc *dv = (const ViewDesc *)ws.views.p;
+    const ViewDesc *dv = ws.d_views;
     {
         StageTimer t(pf, DGS_STAGE_CELL_PROJECT, st);
-        launch_cell_project(dv, V, (const SceneDev *)ws.scenes.p, n, (uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p,
+        launch_cell_project(dv, V, ws.d_scenes, n, (uint32_t *)ws.zkey.p, (uint32_t *)ws.zval.p,
                             (short4 *)ws.rect.p, (float *)ws.depth.p, (uint32_t *)ws.count.p, small + kSmallVisible,
                             (float *)ws.vview.p, ctx->cfg.flags, chain_prep(ws, 0, n, ws.total_tiles), st);
     }
@@ -936,23 +935,26 @@ dgs_status chain_forward(dgs_ctx *ctx, Workspace &ws, const std::vector<ChainVie
     ws.n_records = rec_base;
     const int S = (int)slots.size();
     dgs_status s;
-    if ((s = ws.views.ensure(sizeof(ViewDesc) * V)) || (s = ws.scenes.ensure(sizeof(SceneDev) * S))) return s;
-    if (ws.h_views_cap < (size_t)V) {
-        if (ws.h_views) cudaFreeHost(ws.h_views);
-        ws.h_views = nullptr;
-        CK(cudaMallocHost(&ws.h_views, sizeof(ViewDesc) * V));
-        ws.h_views_cap = V;
+    const size_t views_at = kSmallBytes, scenes_at = views_at + sizeof(ViewDesc) * V;
+    const size_t bytes = scenes_at + sizeof(SceneDev) * S;
+    static_assert(kSmallBytes % 16 == 0 && sizeof(ViewDesc) % 8 == 0, "descriptors follow the zeroed words");
+    if ((s = ws.small.ensure(bytes))) return s;
+    if (ws.h_chain_cap < bytes) {
+        if (ws.h_chain) cudaFreeHost(ws.h_chain);
+        ws.h_chain = nullptr;
+        ws.h_chain_cap = 0;
+        CK(cudaMallocHost(&ws.h_chain, bytes));
+        ws.h_chain_cap = bytes;
+        memset(ws.h_chain, 0, kSmallBytes);
     }
-    if (ws.h_scenes_cap < (size_t)S) {
-        if (ws.h_scenes) cudaFreeHost(ws.h_scenes);
-        ws.h_scenes = nullptr;
-        CK(cudaMallocHost(&ws.h_scenes, sizeof(SceneDev) * S));
-        ws.h_scenes_cap = S;
+    memcpy(ws.h_chain + views_at, ws.hviews.data(), sizeof(ViewDesc) * V);
+    for (int k = 0; k < S; ++k) {
+        const SceneDev sd = slots[k]->dev();
+        memcpy(ws.h_chain + scenes_at + sizeof(SceneDev) * k, &sd, sizeof(SceneDev));
     }
-    memcpy(ws.h_views, ws.hviews.data(), sizeof(ViewDesc) * V);
-    for (int k = 0; k < S; ++k) ws.h_scenes[k] = slots[k]->dev();
-    CK(cudaMemcpyAsync(ws.views.p, ws.h_views, sizeof(ViewDesc) * V, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(ws.scenes.p, ws.h_scenes, sizeof(SceneDev) * S, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(ws.small.p, ws.h_chain, bytes, cudaMemcpyHostToDevice, st));
+    ws.d_views = (const ViewDesc *)((const char *)ws.small.p + views_at);
+    ws.d_scenes = (const SceneDev *)((const char *)ws.small.p + scenes_at);
     if ((s = run_binning(ctx, ws, st, device_sized))) return s;
     const BlendParams bp = blend_params(ctx->cfg);
     const long long nrec = std::max(1LL, ws.n_records), px1 = std::max(1LL, px);
@@ -970,7 +972,7 @@ dgs_status chain_forward(dgs_ctx *ctx, Workspace &ws, const std::vector<ChainVie
         (grad_buffers && (s = ws.g2d.ensure(sizeof(float) * kGradF * nrec))) || (s = ws.Dpix.ensure(4 * px1)) ||
         (s = ws.ndpix.ensure(4 * px1)) || ((keep_rgb || !out_img) && (s = ws.rgb.ensure(12 * px1))))
         return s;
-    const ViewDesc *dv = (const ViewDesc *)ws.views.p;
+    const ViewDesc *dv = ws.d_views;
     for (int k = 0; k < S; ++k) {
         const SceneDev sd = slots[k]->dev();
         if (slots[k]->F > 0) {  // neural cells: decode the visible cells' Gaussians for every view first
@@ -1166,11 +1168,11 @@ extern "C" dgs_status dgs_render_backward(dgs_ctx *ctx, dgs_fwd_state *state, co
     }
     {
         StageTimer t(ctx->prof, DGS_STAGE_BLEND_BWD, st);
-        launch_blend_bwd((const ViewDesc *)ws.views.p, ws.V, ws.total_tiles, (const uint32_t *)ws.order.p, sc.K,
+        launch_blend_bwd(ws.d_views, ws.V, ws.total_tiles, (const uint32_t *)ws.order.p, sc.K,
                          (const uint2 *)ws.ranges.p,
                          (const uint32_t *)ws.tval.p, (const float4 *)ws.rec.p, bp, (const float *)ws.rgb.p,
                          (const float *)ws.Dpix.p, (const int *)ws.ndpix.p, dl, (float *)ws.g2d.p, gv, st);
-        if (gv) launch_cell_v_grad((const ViewDesc *)ws.views.p, ws.V, sc.dev(), gv, o_v, o_vsh, o_cc, st);
+        if (gv) launch_cell_v_grad(ws.d_views, ws.V, sc.dev(), gv, o_v, o_vsh, o_cc, st);
     }
     if (neural && (o_mlp || o_f || o_off || o_cc || o_ca || o_cq)) {
         if ((s = ws.gdec.ensure(sizeof(float) * kDecF * std::max(1LL, ws.n_records)))) return s;
@@ -1184,19 +1186,19 @@ extern "C" dgs_status dgs_render_backward(dgs_ctx *ctx, dgs_fwd_state *state, co
         float *m = o_mlp ? o_mlp : gscr, *f = o_f ? o_f : gscr + P, *off = o_off ? o_off : gscr + P + NF;
         {
             StageTimer t(ctx->prof, DGS_STAGE_PROJECT_BWD, st);
-            launch_project_bwd_neural((const ViewDesc *)ws.views.p, ws.V, 0, sc.dev(), (const uint32_t *)ws.count.p,
+            launch_project_bwd_neural(ws.d_views, ws.V, 0, sc.dev(), (const uint32_t *)ws.count.p,
                                       bp, (const float *)ws.dec.p, (const float *)ws.g2d.p, (float *)ws.gdec.p, st);
         }
         StageTimer t(ctx->prof, DGS_STAGE_DECODE_BWD, st);
         CK(cudaMemsetAsync(m, 0, sizeof(float) * P, st));
         CK(cudaMemsetAsync(f, 0, sizeof(float) * NF, st));
         CK(cudaMemsetAsync(off, 0, sizeof(float) * GO, st));
-        launch_decode_bwd((const ViewDesc *)ws.views.p, ws.V, 0, sc.dev(), (const uint32_t *)ws.zval.p, n_samp,
+        launch_decode_bwd(ws.d_views, ws.V, 0, sc.dev(), (const uint32_t *)ws.zval.p, n_samp,
                           (const uint32_t *)ws.small.p + kSmallVisible, (const float *)ws.gdec.p, m, f, off,
                           CellGrads{o_cc, o_ca, o_cq}, (float *)ws.wpack.p, st);
     } else if (!neural) {
         StageTimer t(ctx->prof, DGS_STAGE_PROJECT_BWD, st);
-        launch_project_bwd((const ViewDesc *)ws.views.p, ws.V, 0, sc.dev(), (const uint32_t *)ws.count.p, bp,
+        launch_project_bwd(ws.d_views, ws.V, 0, sc.dev(), (const uint32_t *)ws.count.p, bp,
                            (const float *)ws.g2d.p, o_mean, o_s, o_ls, o_q, o_lg, o_sh, st);
     }
     CK(cudaGetLastError());
@@ -1331,7 +1333,7 @@ extern "C" dgs_status dgs_state_counts(dgs_ctx *ctx, const dgs_fwd_state *state,
     unsigned long long *c = (unsigned long long *)ctx->aux.p;
     CK(cudaStreamWaitEvent(st, ws.done, 0));
     CK(cudaMemsetAsync(c, 0, 32, st));
-    launch_count_pairs((const ViewDesc *)ws.views.p, ws.V, ws.total_tiles, (const uint2 *)ws.ranges.p,
+    launch_count_pairs(ws.d_views, ws.V, ws.total_tiles, (const uint2 *)ws.ranges.p,
                        (const uint32_t *)ws.tval.p, (const float4 *)ws.rec.p, (const int *)ws.ndpix.p, c, st);
     CK(cudaGetLastError());
     unsigned long long h[4];

@@ -119,8 +119,8 @@ __device__ __forceinline__ void xform_s(const float R[9], const float t[3], floa
 // vview[entry]: v_n as rendered in that view (the scalar, or the clamped SH
 // value of a view-dependent v_n).
 // flags: dgs_config.flags (DGS_FLAG_NEAR_FULL changes the footprint of cells at the near plane).
-// The binning kernels also prepare their successors, so that a chain needs one
-// memset and no kernel that only counts: they add up the digit counts of
+// The binning kernels also prepare their successors, so that a chain needs no
+// memset of its own and no kernel that only counts: they add up the digit counts of
 // the sort that follows (hist, zeroed before) and clear the words listed here.
 struct BinPrep {
     uint32_t *hist;          // of the sort that follows: [passes][256]

@@ -30,8 +30,8 @@ constexpr int kSmallOverflow = 4; // L exceeded the pair capacity (captured chai
 constexpr int kSmallWork = 5;     // work counter of the pulling blend (captured chains)
 constexpr int kSmallTcErr = 6;    // a tensor-core product's completion wait gave up (decode)
 // and after its first 64 words what the binning kernels need zeroed, so that one
-// memset clears all of it: partition counters of the depth sort, the tile sort (4
-// each) and the offsets' scan, and the two sorts' digit counts
+// copy or memset clears all of it: partition counters of the depth sort, the tile sort
+// (4 each) and the offsets' scan, and the two sorts' digit counts
 constexpr int kSmallCounters = 64, kSmallHist = 128;
 constexpr size_t kSmallBytes = 4 * (kSmallHist + 2 * 4 * 256);
 constexpr PairSlots kPairSlots{kSmallTotal, kSmallPairs, kSmallOverflow, kSmallSortErr};
@@ -98,6 +98,12 @@ struct Workspace {
     DevBuf sizes;                 // ChainSizes of a captured chain
     uint32_t *h_small = nullptr;  // pinned mirror of `small`
     ChainSizes *h_sizes = nullptr;
+    // A render's chain keeps its view and scene descriptors behind `small`, and
+    // h_chain (pinned) holds zeros for `small` and the descriptors: one copy sets all of it.
+    const ViewDesc *d_views = nullptr;
+    const SceneDev *d_scenes = nullptr;
+    char *h_chain = nullptr;
+    size_t h_chain_cap = 0;
     ViewDesc *h_views = nullptr;
     size_t h_views_cap = 0;
     SceneDev *h_scenes = nullptr;
