@@ -104,21 +104,26 @@ __device__ __forceinline__ void proj_core(const ViewDesc &Vw, const GaussIn &p, 
     c.syy = fadd_s(fadd_s(fadd_s(fmul_s(c.V[3], c.T[3]), fmul_s(c.V[4], c.T[4])), fmul_s(c.V[5], c.T[5])), dilation);
 }
 
-// The 48-byte record of Gaussian p in view Vw (an invalid Gaussian, mean not
-// in front of the near plane, gets ext = -1 so no AABB test passes).  k: SH
-// coefficients, cv: the cell's v_n.  Returns c.valid; c keeps the view-space mean.
+// The 48-byte record of Gaussian p in view Vw.  A Gaussian that is not drawn gets
+// ext = -1, so no AABB test passes: its mean is not in front of the near plane, or its
+// projection is not a number (a zero quaternion, a NaN parameter, a screen covariance
+// beyond FP32).  The blends rely on it: they give a pixel outside the box an offset of
+// kFar in place of a branch, and that is alpha = 0 only where L is a number.  k: SH
+// coefficients, cv: the cell's v_n.  Returns whether it is drawn; c keeps the
+// view-space mean.
 template <bool DIRECT_RGB = false>
 __device__ __forceinline__ bool gauss_record(const ViewDesc &Vw, const GaussIn &p, const float (&k)[16][3],
                                              int sh_degree, float opac, float cv, const BlendParams &bp,
                                              ProjCore &c, float4 &r0, float4 &r1, float4 &r2,
                                              const float *rgb = nullptr) {
-    proj_core(Vw, p, bp.dilation, c);
-    if (!c.valid) {
+    auto not_drawn = [&] {
         r0 = make_float4(0.f, 0.f, -1.f, -1.f);
         r1 = make_float4(0.f, 0.f, 0.f, 0.f);
         r2 = make_float4(0.f, 0.f, 0.f, cv);
         return false;
-    }
+    };
+    proj_core(Vw, p, bp.dilation, c);
+    if (!c.valid) return not_drawn();
     const float mx = fadd_s(fmul_s(Vw.fx, c.x), Vw.cx);
     const float my = fadd_s(fmul_s(Vw.fy, c.y), Vw.cy);
     float ex, ey;
@@ -139,6 +144,8 @@ __device__ __forceinline__ bool gauss_record(const ViewDesc &Vw, const GaussIn &
     const ScreenCov sc2 = screen_cov(c, bp.dilation);
     const float ip = rsqrtf(sc2.syy * sc2.det);
     const float fp = sc2.syy * ip, fr = -sc2.sxy * ip, ft = rsqrtf(sc2.syy);
+    // (every term is >= 0 or not a number)
+    if (!(fabsf(mx) + fabsf(my) + ex + ey + fp + fabsf(fr) + ft >= 0.f)) return not_drawn();
     float col[3];
     if (DIRECT_RGB) {
         col[0] = rgb[0]; col[1] = rgb[1]; col[2] = rgb[2];
