@@ -224,8 +224,9 @@ __device__ __forceinline__ void blend_fwd_unit(int unit, const ViewDesc *__restr
                         for (int q = 0; q < PPL; ++q) h[q] = !(T[q] < bp.eps) && hx[q & 1] && hy[q >> 1];
                     } else {
                         // outside the box along a column or a row: an offset far off
-                        // the Gaussian, so exp2 gives alpha = +0 exactly (in-box pixels
-                        // compute as before; a done pixel's sums are not used)
+                        // the Gaussian, so exp2 gives alpha = +0 exactly (a done pixel
+                        // takes the cell's sums with weight 0: records are finite,
+                        // gauss_record)
 #pragma unroll
                         for (int c2 = 0; c2 < 2; ++c2) dx[c2] = hx[c2] ? dx[c2] : kFar;
 #pragma unroll

@@ -14,6 +14,8 @@
 // One thread per Gaussian reads its parameters once (SoA planes, coalesced)
 // and writes one 48-byte record per view, so a batch of views costs one pass
 // over the 236 B/Gaussian of parameters.
+#include <cfloat>
+
 #include "project.cuh"
 
 namespace dgs {
@@ -167,8 +169,9 @@ __global__ void __launch_bounds__(128) k_gauss_bin(const ViewDesc *__restrict__ 
             float4 r0, r1, r2;
             bool vis = gauss_record(Vw, p, k, sc.sh_degree, opac, cv, bp, c, r0, r1, r2);
             if (wsr) {
-                r2.w = tau > 0.f ? fmaxf(0.f, 1.f - c.t[2] / tau) * cv : cv;
-                vis = vis && r2.w > 0.f;
+                const float w = tau > 0.f ? fmaxf(0.f, 1.f - c.t[2] / tau) * cv : cv;
+                vis = vis && w > 0.f;
+                r2.w = fminf(w, FLT_MAX);  // (as the colours: 0 times it is 0)
             }
             short4 r = make_short4(-1, -1, -1, -1);
             if (vis) {

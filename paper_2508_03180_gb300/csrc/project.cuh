@@ -9,8 +9,9 @@
 namespace dgs {
 
 constexpr float KAPPA = 0.8493218002880191f;  // sqrt(log2(e) / 2), log2(e) = 1/ln 2
-
-
+// The largest colour of a record: the adjoint's products of a cell's 32 colours with
+// dL/dC / D stay finite down to D = 1e-10 at |dL/dC| of 100.
+constexpr float kMaxColour = 1e25f;
 
 struct GaussIn {
     float mean[3], scale[3], quat[4], logit;
@@ -108,9 +109,11 @@ __device__ __forceinline__ void proj_core(const ViewDesc &Vw, const GaussIn &p, 
 // ext = -1, so no AABB test passes: its mean is not in front of the near plane, or its
 // projection is not a number (a zero quaternion, a NaN parameter, a screen covariance
 // beyond FP32).  The blends rely on it: they give a pixel outside the box an offset of
-// kFar in place of a branch, and that is alpha = 0 only where L is a number.  k: SH
-// coefficients, cv: the cell's v_n.  Returns whether it is drawn; c keeps the
-// view-space mean.
+// kFar in place of a branch, and that is alpha = 0 only where L is a number.  For the
+// same reason colours are at most kMaxColour (a decoder's NaN too): an alpha or a weight
+// of 0 times a cell's colours is then 0, at pixels that a Gaussian does not reach and at those
+// finished before its cell.  k: SH coefficients, cv: the cell's v_n.  Returns whether it
+// is drawn; c keeps the view-space mean.
 template <bool DIRECT_RGB = false>
 __device__ __forceinline__ bool gauss_record(const ViewDesc &Vw, const GaussIn &p, const float (&k)[16][3],
                                              int sh_degree, float opac, float cv, const BlendParams &bp,
@@ -148,7 +151,8 @@ __device__ __forceinline__ bool gauss_record(const ViewDesc &Vw, const GaussIn &
     if (!(fabsf(mx) + fabsf(my) + ex + ey + fp + fabsf(fr) + ft >= 0.f)) return not_drawn();
     float col[3];
     if (DIRECT_RGB) {
-        col[0] = rgb[0]; col[1] = rgb[1]; col[2] = rgb[2];
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) col[ch] = fminf(rgb[ch], kMaxColour);
     } else {
         float d0 = p.mean[0] - Vw.eye[0], d1 = p.mean[1] - Vw.eye[1], d2 = p.mean[2] - Vw.eye[2];
         const float il = rsqrtf(d0 * d0 + d1 * d1 + d2 * d2);
@@ -160,7 +164,7 @@ __device__ __forceinline__ bool gauss_record(const ViewDesc &Vw, const GaussIn &
             float s = 0.5f;
 #pragma unroll
             for (int cidx = 0; cidx < 16; ++cidx) s += k[cidx][ch] * Y[cidx];
-            col[ch] = fmaxf(s, 0.0f);
+            col[ch] = fminf(fmaxf(s, 0.0f), kMaxColour);
         }
     }
     r0 = make_float4(mx, my, ex, ey);

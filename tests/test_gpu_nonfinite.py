@@ -1,7 +1,12 @@
-"""A Gaussian whose projection is not a number (a zero quaternion pads a cell with
-fewer than K Gaussians; a parameter of a diverging step is NaN) is not drawn: images and the
-other Gaussians' gradients are those of the same scene with it out of view, in
-every blend kernel."""
+"""Gaussians with undefined or infinite values stay within their own pixels.
+
+* A Gaussian whose projection is not a number (a zero quaternion pads a cell with
+  fewer than K Gaussians; a parameter of a diverging step is NaN) is not drawn: images and the
+  other Gaussians' gradients are those of the same scene with it out of view,
+  in every blend kernel.
+* A colour, or a weighted sum's weight, beyond FP32 leaves the pixels alone that it does
+  not reach: those outside the Gaussian's box and those finished before its cell.
+"""
 import copy
 
 import numpy as np
@@ -73,5 +78,73 @@ def test_undefined_gaussian_is_not_drawn(damage, opaque, flags, large):
             a, b = (g_got[k], g_want[k]) if k == "g_cell_v" else (g_got[k][live], g_want[k][live])
             # the same sums, added to by atomics in another order
             assert (a - b).norm() <= 1e-5 * b.norm(), k
+    finally:
+        ctx.close()
+
+
+def _flat_scene(n, logit, scale):
+    """n cells of one Gaussian each, one behind the other as seen from (0, -3, 0)."""
+    sc = synth.make_scene(n, 1, synth._box(-0.2, 0.2), 0.9, 1.0, 0, seed=5)
+    sc.cell_center[:] = [[0.0, 0.05 * i, 0.0] for i in range(n)]
+    sc.g_mean[:] = sc.cell_center
+    sc.g_scale[:] = scale
+    sc.g_logit[:] = logit
+    return sc
+
+
+@pytest.mark.parametrize("large", [False, True])
+def test_infinite_colour_behind_finished_pixels(large):
+    """Twelve opaque layers finish the pixels in the middle of the view; behind them, over all
+    of it, a Gaussian of infinite colour."""
+    sc = _flat_scene(13, 9.0, 1.0)
+    sc.g_scale[12] = 3.0
+    cams = [synth.small_camera(32, 16)] + ([EMPTY] if large else [])
+    ref = copy.deepcopy(sc)
+    sc.g_sh[12] = np.inf
+    ctx = Context()
+    try:
+        outs = []
+        for s in (ref, sc):
+            sid = ctx.upload_scene(s)
+            img, state, _ = ctx.render(sid, cams, want_state=True)
+            a = img[:3 * 16 * 32].reshape(3, 16, 32).clone()
+            ctx.release_state(state)
+            c = ctx.render_compare(sid, cams, "alpha")[0][:3 * 16 * 32].reshape(3, 16, 32).clone()
+            ctx.release_scene(sid)
+            outs.append((a, c))
+        for want, got in zip(*outs):
+            same = (got == want).all(0)
+            # finished pixels keep their colour, the others take the huge one
+            assert 0.1 < same.float().mean() < 0.9
+            assert (got[:, ~same] > 1e15).any(0).all()
+            assert not torch.isnan(got).any()
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("mode", ["hybrid", "alpha", "wsr", "weight"])
+def test_infinite_values_stay_within_the_box(mode):
+    """Two Gaussians, the nearer one over the middle of a one-tile view only."""
+    sc = _flat_scene(2, 0.0, 0.3)
+    sc.g_scale[1] = 2.0
+    cam = synth.small_camera(16, 16)
+    ref, none = copy.deepcopy(sc), copy.deepcopy(sc)
+    none.g_mean[0, 1] -= 10.0
+    if mode == "weight":
+        sc.cell_v[0] = np.inf
+    else:
+        sc.g_sh[0] = np.inf
+    ctx = Context()
+    try:
+        imgs = []
+        for s in (none, ref, sc):
+            sid = ctx.upload_scene(s)
+            img = ctx.render(sid, [cam])[0] if mode == "hybrid" else ctx.render_compare(
+                sid, [cam], "alpha" if mode == "alpha" else "wsr")[0]
+            imgs.append(img.reshape(3, 16, 16).clone())
+            ctx.release_scene(sid)
+        out = (imgs[0] == imgs[1]).all(0)  # the pixels that the nearer one does not reach
+        assert 0.2 < out.float().mean() < 0.9
+        assert torch.equal(imgs[2][:, out], imgs[0][:, out])
     finally:
         ctx.close()
