@@ -36,8 +36,11 @@ constexpr int CSUB = kTile / CROWS;  // sub-tiles per tile
 // 1M Gaussians, 476 this way (the whole call 992 -> 840 us); without the minimum with
 // alpha_max where no opacity reaches it and with paired offsets the call went from
 // 788 to 762.
-template <bool ALPHA>
-__global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restrict__ views, int n_views,
+// ONCE: eps > 1, where the first entry that reaches a pixel is also its last, even at an
+// alpha of 0, which leaves T at 1 (an instantiation of its own: the mask of such pixels
+// spills at the 64 registers of the others).
+template <bool ALPHA, bool ONCE = false>
+__global__ void __launch_bounds__(CT, ONCE ? 24 : 32) k_gauss_blend(const ViewDesc *__restrict__ views, int n_views,
                                                     const uint32_t *__restrict__ order,
                                                     const uint2 *__restrict__ ranges,
                                                     const uint32_t *__restrict__ list,
@@ -60,6 +63,7 @@ __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restri
     // X: T (alpha; below eps: done) or B (weighted sums), of the row pairs
     float2 C0[NR], C1[NR], C2[NR], X[NR];
     int n[2 * NR];
+    unsigned taken = 0u;  // ONCE: the pixels that took their entry
 #pragma unroll
     for (int rr = 0; rr < NR; ++rr) {
         C0[rr] = C1[rr] = C2[rr] = make_float2(0.f, 0.f);
@@ -118,7 +122,9 @@ __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restri
                 const float2 s1 = __ffma2_rn(make_float2(r1.y, r1.y), make_float2(dy, dy), pdx);
                 const float2 qd = __ffma2_rn(s1, s1, make_float2(q, q));
                 float2 al = __fmul2_rn(make_float2(r1.w, r1.w), make_float2(ex2_approx(-qd.x), ex2_approx(-qd.y)));
-                const bool a0 = h[2 * rr] && !(ALPHA && X[rr].x < eps), a1 = h[2 * rr + 1] && !(ALPHA && X[rr].y < eps);
+                const bool a0 = h[2 * rr] && !(ALPHA && X[rr].x < eps) && !(ONCE && (taken >> (2 * rr) & 1u));
+                const bool a1 = h[2 * rr + 1] && !(ALPHA && X[rr].y < eps) && !(ONCE && (taken >> (2 * rr) & 2u));
+                if (ONCE) taken |= ((a0 ? 1u : 0u) | (a1 ? 2u : 0u)) << (2 * rr);
                 if (decltype(with_clamp)::value) al = make_float2(fminf(al.x, bp.alpha_max), fminf(al.y, bp.alpha_max));
                 al.x = a0 ? al.x : 0.f;
                 al.y = a1 ? al.y : 0.f;
@@ -128,8 +134,8 @@ __global__ void __launch_bounds__(CT, 32) k_gauss_blend(const ViewDesc *__restri
                 C2[rr] = __ffma2_rn(w, make_float2(r2.z, r2.z), C2[rr]);
                 X[rr] = ALPHA ? __fadd2_rn(X[rr], make_float2(-w.x, -w.y)) : __fadd2_rn(X[rr], w);
                 if (ALPHA && out_nd) {
-                    if (a0 && X[rr].x < eps) n[2 * rr] = (int)(base + k + 1 - rg.x);
-                    if (a1 && X[rr].y < eps) n[2 * rr + 1] = (int)(base + k + 1 - rg.x);
+                    if (a0 && (ONCE || X[rr].x < eps)) n[2 * rr] = (int)(base + k + 1 - rg.x);
+                    if (a1 && (ONCE || X[rr].y < eps)) n[2 * rr + 1] = (int)(base + k + 1 - rg.x);
                 }
             }
         }
@@ -247,12 +253,13 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
     launch_tile_order((const uint2 *)ws.ranges.p, tiles, (uint32_t *)ws.order.p, st);
     if (tiles > 0) {
         const unsigned grid = (unsigned)tiles * CSUB;
-        if (wsr)
-            launch_chained(k_gauss_blend<false>, grid, CT, 0, st, dv, V, (const uint32_t *)ws.order.p, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
-                                                      (const float4 *)ws.rec.p, bp, cfg.w_bg, out_img, nullptr);
-        else
-            launch_chained(k_gauss_blend<true>, grid, CT, 0, st, dv, V, (const uint32_t *)ws.order.p, (const uint2 *)ws.ranges.p, (const uint32_t *)ws.tval.p,
-                                                     (const float4 *)ws.rec.p, bp, 0.f, out_img, out_nd);
+        auto blend = [&](auto kernel, float w_bg, int *nd) {
+            launch_chained(kernel, grid, CT, 0, st, dv, V, (const uint32_t *)ws.order.p, (const uint2 *)ws.ranges.p,
+                           (const uint32_t *)ws.tval.p, (const float4 *)ws.rec.p, bp, w_bg, out_img, nd);
+        };
+        if (wsr) blend(k_gauss_blend<false>, cfg.w_bg, nullptr);
+        else if (bp.eps > 1.0f) blend(k_gauss_blend<true, true>, 0.f, out_nd);
+        else blend(k_gauss_blend<true>, 0.f, out_nd);
     }
     CK(cudaGetLastError());
     return DGS_OK;

@@ -95,6 +95,43 @@ def test_alpha_blend_terminates(rctx):
         rctx.release_scene(sid)
 
 
+def _depth(sc, cam):
+    a = cam.as_array()
+    return sc.g_mean @ a[13:16] + a[18]
+
+
+def test_alpha_blend_with_eps_above_one():
+    """Every pixel then ends with the first entry that reaches it, also where that
+    entry's alpha is too small to change T: the entries behind it add nothing."""
+    from paper_2508_03180_gb300.renderer import Context
+    sc = synth.make_scene(40, 1, synth._box(-0.4, 0.4), 0.3, 0.6, 0, seed=12)
+    sc.g_logit[::2] = -40.0  # alpha <= 4e-18
+    cam = synth.small_camera(23, 13)
+    c = Context(eps=1.5)
+    try:
+        img, nd, _ = c.render_compare(c.upload_scene(sc), [cam], "alpha", want_ndone=True)
+        nd = nd.cpu().numpy().reshape(cam.H, cam.W)
+        opt = oracle.Options(eps=1.5)
+        pv = oracle.prepare_view(sc, cam.as_array(), opt)
+        mu, ext = pv["mu2f"], pv["extf"]
+        z = _depth(sc, cam)
+        order = np.argsort(z, kind="stable")
+        ys, xs = np.mgrid[0:cam.H, 0:cam.W].astype(np.float32) + np.float32(0.5)
+        inside = [(np.abs(xs - mu[g, 0]) <= ext[g, 0]) & (np.abs(ys - mu[g, 1]) <= ext[g, 1]) for g in order]
+        first = np.full((cam.H, cam.W), -1)
+        for i in range(len(order) - 1, -1, -1):
+            first[inside[i]] = order[i]
+        faint = (first >= 0) & (first % 2 == 0)
+        assert faint.mean() > 0.1 and (first % 2 == 1).mean() > 0.1
+        got = img.cpu().numpy().reshape(3, cam.H, cam.W)
+        # a faint first entry leaves the background (black), another one's colour shows
+        assert np.abs(got[:, faint]).max() <= 1e-15
+        assert (got[:, first % 2 == 1].max(0) > 0).all()
+        assert nd[first >= 0].min() >= 1 and nd[faint].mean() < sc.G / 2
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("tau,w_bg", [(float("inf"), 0.0), (3.0, 0.0), (3.2, 0.05)])
 def test_wsr_matches_oracle(rctx, tau, w_bg):
     scene = synth.scene_small(seed=3, sh_degree=3)
