@@ -121,12 +121,12 @@ def test_alpha_blend_with_eps_above_one():
         first = np.full((cam.H, cam.W), -1)
         for i in range(len(order) - 1, -1, -1):
             first[inside[i]] = order[i]
-        faint = (first >= 0) & (first % 2 == 0)
-        assert faint.mean() > 0.1 and (first % 2 == 1).mean() > 0.1
+        faint, clear = (first >= 0) & (first % 2 == 0), (first >= 0) & (first % 2 == 1)
+        assert faint.mean() > 0.1 and clear.mean() > 0.1
         got = img.cpu().numpy().reshape(3, cam.H, cam.W)
         # a faint first entry leaves the background (black), another one's colour shows
         assert np.abs(got[:, faint]).max() <= 1e-15
-        assert (got[:, first % 2 == 1].max(0) > 0).all()
+        assert (got[:, clear].max(0) > 0).all()
         assert nd[first >= 0].min() >= 1 and nd[faint].mean() < sc.G / 2
     finally:
         c.close()
