@@ -94,8 +94,10 @@ __global__ void __launch_bounds__(CT, ONCE ? 24 : 32) k_gauss_blend(const ViewDe
         const float4 rl = r[kRecF4 * lane];
         const unsigned full = __ballot_sync(0xffffffffu, mine && covers_rows(rl, bx0, by0, (float)CROWS));
         const unsigned hits = __ballot_sync(0xffffffffu, mine && touches_rows(rl, bx0, by0, (float)CROWS));
-        // (batches whose opacities are all below the clamp go without the minimum, as in the hybrid)
-        const bool clamp = (hits & __ballot_sync(0xffffffffu, !(r[kRecF4 * lane + 1].w < 0.9999f * bp.alpha_max))) != 0u;
+        // (batches whose opacities are all below the clamp go without the minimum, as in the
+        // hybrid; not without dilation, where a flat Gaussian's L is infinite: the minimum makes
+        // alpha_max of an exponent that is not a number)
+        const bool clamp = bp.dilation < 1e-12f || (hits & __ballot_sync(0xffffffffu, !(r[kRecF4 * lane + 1].w < 0.9999f * bp.alpha_max))) != 0u;
         auto blend_batch = [&](auto with_clamp) {
         for (unsigned mask = hits; mask; mask &= mask - 1) {
             const int k = __ffs(mask) - 1;

@@ -95,6 +95,29 @@ def test_alpha_blend_terminates(rctx):
         rctx.release_scene(sid)
 
 
+@pytest.mark.parametrize("mode", ["alpha", "wsr"])
+def test_flat_gaussian_without_dilation(mode):
+    """A needle seen obliquely: its screen covariance is singular and L infinite.  Where
+    L^T d is inf - inf the alpha is alpha_max, elsewhere 0."""
+    from paper_2508_03180_gb300.renderer import Context
+    sc = synth.make_scene(1, 1, synth._box(-0.1, 0.1), 1.0, 1.0, 0, seed=3)
+    sc.g_mean[:] = sc.cell_center[:] = 0.0
+    sc.g_scale[:] = [[0.5, 0.0, 0.0]]
+    sc.g_quat[:] = [[1.0, 0.0, 0.0, 0.0]]
+    sc.g_logit[:] = 0.0
+    sc.g_sh[:] = 1.0  # colour 0.5 + Y_00
+    cam = synth.look_at((0.0, -3.0, 0.0), (0.0, 0.0, 0.0), 32, 32, 60.0, up=(0.6, 0.0, 1.0))
+    c = Context(dilation=0.0)
+    try:
+        img = c.render_compare(c.upload_scene(sc), [cam], mode)[0].cpu().numpy().reshape(3, 32, 32)
+        assert np.isfinite(img).all()
+        col = 0.5 + 0.28209479177387814
+        want = {0.0, round(0.99 * col, 5)} if mode == "alpha" else {0.0, round(col, 5)}
+        assert set(np.unique(img.round(5).astype(np.float64).round(5))) == want
+    finally:
+        c.close()
+
+
 def _depth(sc, cam):
     a = cam.as_array()
     return sc.g_mean @ a[13:16] + a[18]
