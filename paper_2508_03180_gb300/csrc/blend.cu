@@ -830,9 +830,9 @@ __global__ void __launch_bounds__(WT, bwd_minb(WV)) k_blend_bwd(const ViewDesc *
                 const float2 qd = __ffma2_rn(s1, s1, make_float2(s22, s22));
                 float2 Gv = make_float2(ex2_approx(-qd.x), ex2_approx(-qd.y));
                 float2 rw = __fmul2_rn(make_float2(r1.w, r1.w), Gv);
-                if (VAR) {  // not reached (or alpha skipped as in the forward): G' = 0 leaves X and P as they are
-                    if (!(n < nd[2 * rr] && hx[0] && hy[rr]) || rw.x < amin) Gv.x = rw.x = 0.f;
-                    if (!(n < nd[2 * rr + 1] && hx[1] && hy[rr]) || rw.y < amin) Gv.y = rw.y = 0.f;
+                if (VAR) {  // not reached (or alpha skipped, or not a number, as in the forward): G' = 0 leaves X and P as they are
+                    if (!(n < nd[2 * rr] && hx[0] && hy[rr] && rw.x >= amin)) Gv.x = rw.x = 0.f;
+                    if (!(n < nd[2 * rr + 1] && hx[1] && hy[rr] && rw.y >= amin)) Gv.y = rw.y = 0.f;
                 }
                 gq[rr] = Gv;
                 const float2 al = make_float2(fminf(rw.x, bp.alpha_max), fminf(rw.y, bp.alpha_max));

@@ -82,6 +82,29 @@ def test_undefined_gaussian_is_not_drawn(damage, opaque, flags, large):
         ctx.close()
 
 
+def test_flat_gaussian_without_dilation():
+    """A needle seen obliquely: its screen covariance is singular, L infinite and its exponent
+    infinite or inf - inf.  The forward draws nothing of it, and the adjoint's replay agrees."""
+    sc = synth.make_scene(24, 2, synth._box(-0.5, 0.5), 0.1, 0.4, 0, seed=33)
+    needle = np.arange(1, sc.G, 6)
+    sc.g_scale[needle] = [[0.5, 0.0, 0.0]]
+    sc.g_quat[needle] = [[1.0, 0.0, 0.0, 0.0]]
+    ref = copy.deepcopy(sc)
+    ref.g_mean[needle, 1] = -3.0  # not in front of the near plane
+    cams = [synth.look_at((0.0, -3.0, 0.0), (0.0, 0.0, 0.0), 61, 43, 60.0, up=(0.6, 0.0, 1.0))]
+    ctx = Context(dilation=0.0)
+    try:
+        (got, _, _), g_got = _images(ctx, sc, cams)
+        (want, _, _), g_want = _images(ctx, ref, cams)
+        assert torch.equal(got, want) and (want > 0).float().mean() > 0.1
+        live = np.setdiff1d(np.arange(sc.G), needle)
+        for k in g_want:
+            a, b = (g_got[k], g_want[k]) if k == "g_cell_v" else (g_got[k][live], g_want[k][live])
+            assert (a - b).norm() <= 1e-5 * b.norm(), k
+    finally:
+        ctx.close()
+
+
 def _flat_scene(n, logit, scale):
     """n cells of one Gaussian each, one behind the other as seen from (0, -3, 0)."""
     sc = synth.make_scene(n, 1, synth._box(-0.2, 0.2), 0.9, 1.0, 0, seed=5)
