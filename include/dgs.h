@@ -599,15 +599,19 @@ dgs_status dgs_debug_check_guards(int64_t *n_checked);
  *                           run out of memory, without calling it: the call
  *                           returns DGS_ERR_OOM and the context stays usable.
  *   DGS_FAULT_SORT_WAIT     while count != 0, radix sorts launched on the
- *                           current device run with their first partition
- *                           withholding its digit counts and a poll limit of
- *                           1024, so the other partitions' look-back waits
- *                           run out: the kernels finish (every write stays
- *                           inside the sorted arrays), the order is
- *                           unspecified and dgs_sort_pairs /
- *                           dgs_sort_pairs_noalloc return DGS_ERR_TIMEOUT.
- *                           count = 0 switches it off.  Meanwhile call only
- *                           those two: a render would consume the order.
+ *                           current device (count = 2: the scans of the pair
+ *                           counts instead) run with their first partition
+ *                           withholding its counts and a poll limit of 1024,
+ *                           so the other partitions' look-back waits run out:
+ *                           the kernels finish (every write stays inside the
+ *                           arrays), the order is unspecified and
+ *                           dgs_sort_pairs / dgs_sort_pairs_noalloc return
+ *                           DGS_ERR_TIMEOUT.  A render shows the background
+ *                           and its chain reports DGS_ERR_TIMEOUT: from the
+ *                           call itself where that still synchronises after
+ *                           the wait, else once it is seen complete, from the
+ *                           next render or backward; a served request's
+ *                           result carries it.  count = 0 switches it off.
  *   DGS_FAULT_SERVE_WORKER  ctx's serving worker raises a host-side exception
  *                           the next time it admits requests; it catches it
  *                           at its top level, waits for its streams,

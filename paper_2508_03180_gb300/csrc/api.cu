@@ -761,7 +761,7 @@ std::unique_ptr<Workspace> acquire_ws(dgs_ctx *ctx, cudaStream_t st, dgs_status 
 }
 
 dgs_status observe_chain(dgs_ctx *ctx, Workspace &ws, bool wait) {
-    if (!ws.async_pending && !ws.check_tc) return DGS_OK;
+    if (!ws.async_pending && !ws.check_flags) return DGS_OK;
     if (wait) {
         CK(cudaEventSynchronize(ws.done));
     } else {
@@ -770,21 +770,22 @@ dgs_status observe_chain(dgs_ctx *ctx, Workspace &ws, bool wait) {
         if (q != cudaSuccess) return cuda_error(q, "a render's launch chain");
     }
     const uint32_t *h = ws.h_small;
-    if (ws.check_tc && h[kSmallTcErr]) {
+    if (h[kSmallTcErr]) {
         ctx->pending_status = DGS_ERR_TIMEOUT;
         ctx->pending_msg = "an earlier call's tensor-core completion wait gave up: its results are not valid";
     }
-    ws.check_tc = false;
+    if (h[kSmallSortErr]) {
+        ctx->pending_status = DGS_ERR_TIMEOUT;
+        ctx->pending_msg = "an earlier render's radix sort look-back wait gave up: its image and state are not valid";
+    }
+    ws.check_flags = false;
     if (!ws.async_pending) return DGS_OK;
     ws.async_pending = false;
     const long long L = h[kSmallTotal];
     ws.L = std::min(L, ws.L_cap);
     ws.n_vis = h[kSmallVisible];
     if (ws.total_tiles > 0) ctx->pairs_per_tile = std::max(ctx->pairs_per_tile, (double)L / ws.total_tiles);
-    if (h[kSmallSortErr]) {
-        ctx->pending_status = DGS_ERR_TIMEOUT;
-        ctx->pending_msg = "an earlier render's radix sort look-back wait gave up: its image and state are not valid";
-    } else if (h[kSmallOverflow]) {
+    if (h[kSmallOverflow] && !h[kSmallSortErr]) {
         ctx->pending_status = DGS_ERR_CAPACITY;
         ctx->pending_msg = "an earlier render's " + std::to_string(L) + " (tile, cell) pairs exceeded its capacity of " +
                            std::to_string(ws.L_cap) +
@@ -892,7 +893,8 @@ static dgs_status run_binning(dgs_ctx *ctx, Workspace &ws, cudaStream_t st, bool
     }
     {
         StageTimer t(pf, DGS_STAGE_TILE_RANGES, st);
-        launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, st, d_L);
+        launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, small + kSmallSortErr,
+                           device_sized ? nullptr : ws.h_small + kSmallSortErr, st, d_L);
         launch_tile_order((const uint2 *)ws.ranges.p, ws.total_tiles, (uint32_t *)ws.order.p, st);
     }
     CK(cudaGetLastError());
@@ -973,6 +975,7 @@ dgs_status chain_forward(dgs_ctx *ctx, Workspace &ws, const std::vector<ChainVie
         (s = ws.ndpix.ensure(4 * px1)) || ((keep_rgb || !out_img) && (s = ws.rgb.ensure(12 * px1))))
         return s;
     const ViewDesc *dv = ws.d_views;
+    bool decoded = false;
     for (int k = 0; k < S; ++k) {
         const SceneDev sd = slots[k]->dev();
         if (slots[k]->F > 0) {  // neural cells: decode the visible cells' Gaussians for every view first
@@ -981,7 +984,7 @@ dgs_status chain_forward(dgs_ctx *ctx, Workspace &ws, const std::vector<ChainVie
             launch_decode(dv, V, k, sd, (const uint32_t *)ws.zval.p, n_samp,
                           (const uint32_t *)ws.small.p + kSmallVisible, (float *)ws.dec.p, (float *)ws.wpack.p, (const float *)ws.vview.p, bp, (float4 *)ws.rec.p,
                           grad_buffers ? (float *)ws.g2d.p : nullptr, (uint32_t *)ws.small.p + kSmallTcErr, st);
-            ws.check_tc = true;
+            decoded = true;
         } else {
             StageTimer t(ctx->prof, DGS_STAGE_PROJECT_FWD, st);
             launch_project_fwd(dv, V, k, sd, (const uint32_t *)ws.count.p, (const float *)ws.vview.p, bp,
@@ -1000,8 +1003,10 @@ dgs_status chain_forward(dgs_ctx *ctx, Workspace &ws, const std::vector<ChainVie
                          (const float4 *)ws.rec.p, bp, img, img2, (float *)ws.Dpix.p, (int *)ws.ndpix.p, K_all, st);
     }
     CK(cudaGetLastError());
-    if (device_sized || ws.check_tc)  // the chain's sizes and flags, read once it has completed (observe_chain)
-        CK(cudaMemcpyAsync(ws.h_small, ws.small.p, 64, cudaMemcpyDeviceToHost, st));
+    // the chain's sizes and flags, read once it has completed (observe_chain); without either
+    // k_tile_ranges itself notes a tile sort that gave up in h_small
+    if (device_sized || decoded) CK(cudaMemcpyAsync(ws.h_small, ws.small.p, 64, cudaMemcpyDeviceToHost, st));
+    ws.check_flags = true;
     ws.stream = st;
     return DGS_OK;
 }
@@ -1420,7 +1425,7 @@ extern "C" dgs_status dgs_debug_inject_fault(dgs_ctx *ctx, int32_t kind, int32_t
             return DGS_OK;
         case DGS_FAULT_SORT_WAIT: {
             if (ctx) CK(cudaSetDevice(ctx->cfg.device));
-            CK(set_sort_fault(count != 0));
+            CK(set_sort_fault(count == 2 ? 2 : count != 0));
             return DGS_OK;
         }
         case DGS_FAULT_TC_WAIT: {

@@ -334,10 +334,18 @@ void launch_emit(const uint32_t *offs, const uint32_t *zval_sorted, const short4
 }
 
 // [start, end) of every non-empty tile from the tile-sorted keys; empty
-// tiles keep the (0,0) the caller cleared them to.
+// tiles keep the (0,0) the caller cleared them to -- and all tiles do if a wait of
+// the chain's sorts or of its scan gave up: slots that no pass wrote hold whatever
+// the buffer held, keys beyond the last tile and cells beyond the last cell.  With
+// empty lists no later kernel reads them.
 __global__ void k_tile_ranges(const uint32_t *__restrict__ key, long long L, const uint32_t *__restrict__ d_L,
-                              uint2 *__restrict__ ranges) {
+                              uint2 *__restrict__ ranges, const uint32_t *__restrict__ err,
+                              uint32_t *__restrict__ host_err) {
     chain_wait();
+    if (*err) {
+        if (host_err && blockIdx.x == 0 && threadIdx.x == 0) *host_err = 1u;
+        return;
+    }
     if (d_L) L = *d_L;
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < L; j += (long long)gridDim.x * blockDim.x) {
         const uint32_t k = key[j];
@@ -346,10 +354,10 @@ __global__ void k_tile_ranges(const uint32_t *__restrict__ key, long long L, con
     }
 }
 
-void launch_tile_ranges(const uint32_t *tkey_sorted, long long L, uint2 *ranges, cudaStream_t st,
-                        const uint32_t *d_L) {
+void launch_tile_ranges(const uint32_t *tkey_sorted, long long L, uint2 *ranges, const uint32_t *err, uint32_t *host_err,
+                        cudaStream_t st, const uint32_t *d_L) {
     if (L == 0) return;
-    launch_chained(k_tile_ranges, grid_for(L, 256), 256, 0, st, tkey_sorted, L, d_L, ranges);
+    launch_chained(k_tile_ranges, grid_for(L, 256), 256, 0, st, tkey_sorted, L, d_L, ranges, err, host_err);
 }
 
 // Tiles by descending list length (in steps of a quarter of a power of two), for

@@ -251,7 +251,8 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
                 (uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, (bits + 7) / 8, chain_prep(ws, 1, L, 0), st, nullptr,
                 d_vis, nullptr);
     sort_tiles(ws, L, bits, nullptr, st);
-    launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, st);
+    launch_tile_ranges((const uint32_t *)ws.tkey.p, L, (uint2 *)ws.ranges.p, small + kSmallSortErr,
+                       ws.h_small + kSmallSortErr, st);
     launch_tile_order((const uint2 *)ws.ranges.p, tiles, (uint32_t *)ws.order.p, st);
     if (tiles > 0) {
         const unsigned grid = (unsigned)tiles * CSUB;
@@ -264,6 +265,7 @@ dgs_status compare_chain(dgs_ctx *ctx, Workspace &ws, const Scene &sc, const std
         else blend(k_gauss_blend<true>, 0.f, out_nd);
     }
     CK(cudaGetLastError());
+    ws.check_flags = true;  // (a tile sort that gave up: k_tile_ranges notes it in h_small)
     return DGS_OK;
 }
 

@@ -141,8 +141,11 @@ void launch_emit(const uint32_t *offs, const uint32_t *zval_sorted, const short4
                  int n_views, long long n_entries, long long n_all, long long L, int n_tiles, uint32_t *tkey,
                  uint32_t *tval, int passes, const BinPrep &prep, cudaStream_t st, const ChainSizes *dsz,
                  const uint32_t *d_n, const uint32_t *d_L);
-void launch_tile_ranges(const uint32_t *tkey_sorted, long long L, uint2 *ranges, cudaStream_t st,
-                        const uint32_t *d_L = nullptr);
+// err: the chain's sort error word (the ranges stay empty if it is set); host_err
+// (nullable): pinned host memory where that is noted, for a chain whose words are not
+// copied back after its tile sort.
+void launch_tile_ranges(const uint32_t *tkey_sorted, long long L, uint2 *ranges, const uint32_t *err, uint32_t *host_err,
+                        cudaStream_t st, const uint32_t *d_L = nullptr);
 
 // order[i]: the tile that the blend kernels' i-th blocks take, longest lists first.
 void launch_tile_order(const uint2 *ranges, int n_tiles, uint32_t *order, cudaStream_t st,
@@ -296,7 +299,7 @@ int loss_l1_blocks(int64_t n);
 long long resident_ctas(const void *kernel, int threads);
 
 // Test-only: make the radix sort's look-back waits run out (see sort.cu).
-cudaError_t set_sort_fault(bool on);
+cudaError_t set_sort_fault(int which);  // 0 none, 1 sorts, 2 the pair-offset scan
 cudaError_t set_tc_fault(bool on);  // the tensor-core decode's completion wait runs out (DGS_FAULT_TC_WAIT)
 
 // Programmatic dependent launch: a kernel launched by launch_chained is set up while

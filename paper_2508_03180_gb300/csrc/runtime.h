@@ -121,7 +121,7 @@ struct Workspace {
     // on the device only (pair buffers sized L_cap), and L, n_vis and the
     // chain's flags are read from h_small once it has completed (observe_chain).
     bool async_pending = false;
-    bool check_tc = false;  // the chain ran tensor-core kernels: observe their wait flag once it completes
+    bool check_flags = false;  // a chain's wait flags are still to be observed once it completes
     long long L_cap = 0;
     dgs_status init();
     std::vector<DevBuf *> all();
@@ -282,9 +282,9 @@ std::unique_ptr<Workspace> acquire_ws(dgs_ctx *ctx, cudaStream_t st, dgs_status 
 // device memory (see observe_chain).
 dgs_status chain_forward(dgs_ctx *ctx, Workspace &ws, const std::vector<ChainView> &views, float *out_img,
                          bool keep_rgb, bool grad_buffers, cudaStream_t st, bool device_sized = false);
-// Read a device-sized chain's sizes and flags once it has completed (wait:
-// block until then; otherwise look only if it has).  A pair overflow or a
-// sort that gave up becomes ctx->pending_status.
+// Read a chain's flags, and a device-sized one's sizes, once it has completed (wait:
+// block until then; otherwise look only if it has).  A pair overflow or a wait
+// that gave up becomes ctx->pending_status.
 dgs_status observe_chain(dgs_ctx *ctx, Workspace &ws, bool wait);
 ViewDesc make_view(const dgs_camera &c, int tile_base, long long pix_base, int slot, const Scene &sc,
                    long long cell_base, long long rec_base);

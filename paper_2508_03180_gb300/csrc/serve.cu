@@ -247,7 +247,8 @@ dgs_status record_chain(dgs_ctx *ctx, Workspace &ws, const ChainCaps &c, const B
                 st, dsz, d_vis, d_L);
     radix_sort_counted((uint32_t *)ws.tkey.p, (uint32_t *)ws.tval.p, c.L, bits, chain_sort_scratch(ws, 1), st, d_L,
                        nullptr, true);
-    launch_tile_ranges((const uint32_t *)ws.tkey.p, c.L, (uint2 *)ws.ranges.p, st, d_L);
+    launch_tile_ranges((const uint32_t *)ws.tkey.p, c.L, (uint2 *)ws.ranges.p, small + kSmallSortErr, nullptr,
+                       st, d_L);
     launch_tile_order((const uint2 *)ws.ranges.p, (int)c.T, (uint32_t *)ws.order.p, st, dsz);
     // neural scenes: the decode writes their records (slot k's samples of the
     // visible entries, counted on the device); the table projection skips them

@@ -3,7 +3,8 @@ fault-injection calls, include/dgs.h):
 
 * a radix-sort look-back wait made to run out (the first partition withholds
   its counts, a short poll limit) ends the kernels, returns DGS_ERR_TIMEOUT,
-  and the same context then sorts and renders correctly;
+  and the same context then sorts and renders correctly; a render whose sorts or whose
+  scan of the pair counts gave up shows the background and reports it;
 * an injected device-allocation failure returns DGS_ERR_OOM from a scene
   upload and from a render, and the context stays usable;
 * a host-side fault in the serving worker completes every open request with
@@ -44,9 +45,11 @@ def _reference_image(scene, cams):
         ref.close()
 
 
-def test_sort_wait_runs_out_and_the_context_stays_usable():
+# 98 partitions of 1024 items, and of 3072: the others wait on the first
+@pytest.mark.parametrize("n", [100_003, 300_001])
+def test_sort_wait_runs_out_and_the_context_stays_usable(n):
     ctx = Context()
-    n, bits = 100_003, 32  # 33 partitions: 32 of them wait on the first
+    bits = 32
     g = torch.Generator().manual_seed(1)
     keys = torch.randint(0, 2 ** 31, (n,), generator=g, dtype=torch.int64).to(torch.int32)
     vals = torch.arange(n, dtype=torch.int32)
@@ -75,6 +78,102 @@ def test_sort_wait_runs_out_and_the_context_stays_usable():
         cams = [synth.small_camera(64, 48)]
         sid = ctx.upload_scene(scene)
         assert torch.equal(_render(ctx, sid, cams), _reference_image(scene, cams))
+    finally:
+        ctx.close()
+
+
+SORT, SCAN = 1, 2
+
+
+@pytest.mark.parametrize("which", [SORT, SCAN])
+@pytest.mark.parametrize("neural", [False, True])
+def test_render_whose_waits_ran_out_reports_it(which, neural):
+    """12,000 (view, cell) entries, several partitions of the depth sort and of the scan:
+    asynchronous renders and their backward, and a synchronising one."""
+    if neural:
+        sc = synth.neural_scene(n_cells=6000, K=10, F=32, H=32, seed=5)
+    else:
+        sc = synth.scene_small(n_cells=6000)
+    cams = [synth.small_camera(96, 64), synth.sphere_cameras(1, 3.0, 80, 60, seed0=4)[0]]
+    ctx = Context()
+    try:
+        sid = ctx.upload_scene(sc)
+        ref = _render(ctx, sid, cams)
+        g = dict(g_offset=torch.zeros(sc.G, 3, device="cuda")) if neural else dict(
+            g_mean=torch.zeros(sc.G, 3, device="cuda"))
+        L.dgs_debug_inject_fault(ctx.ctx, L.DGS_FAULT_SORT_WAIT, which)
+        try:
+            img, state, _ = ctx.render(sid, cams, want_state=True)
+            torch.cuda.synchronize()
+        finally:
+            L.dgs_debug_inject_fault(ctx.ctx, L.DGS_FAULT_SORT_WAIT, 0)
+        assert not img.any() and ref.any()  # the background
+        with pytest.raises(L.DgsError) as ei:
+            ctx.backward(state, torch.ones_like(img), g)
+        assert ei.value.code == L.DGS_ERR_TIMEOUT and "look-back" in str(ei.value)
+        ctx.release_state(state)
+        L.dgs_debug_inject_fault(ctx.ctx, L.DGS_FAULT_SORT_WAIT, which)
+        try:
+            with pytest.raises(L.DgsError) as ei:
+                ctx.render(sid, cams, stats=True)
+        finally:
+            L.dgs_debug_inject_fault(ctx.ctx, L.DGS_FAULT_SORT_WAIT, 0)
+        assert ei.value.code == L.DGS_ERR_TIMEOUT
+        assert torch.equal(_render(ctx, sid, cams), ref)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("tiles", ["one pass", "two passes"])
+def test_tile_sort_whose_wait_ran_out(tiles):
+    """300 cells (one partition of the depth sort) with many pairs: only the tile sort gives
+    up, after the host has read the pair count; comparators likewise."""
+    sc = synth.make_scene(300, 2, synth._box(-1, 1), 0.3, 0.6, 0, seed=6)
+    cams = [synth.small_camera(240, 240) if tiles == "one pass" else synth.small_camera(640, 480)]
+    ctx = Context()
+    try:
+        sid = ctx.upload_scene(sc)
+        calls = (lambda: ctx.render(sid, cams, stats=True)[0], lambda: ctx.render_compare(sid, cams, "wsr")[0],
+                 lambda: ctx.render_compare(sid, cams, "alpha")[0])
+        _, _, st = ctx.render(sid, cams, stats=True)
+        assert st.sort_length > 3 * 1024
+        for call in calls:
+            ref = call().clone()
+            assert ref.any()
+            L.dgs_debug_inject_fault(ctx.ctx, L.DGS_FAULT_SORT_WAIT, SORT)
+            try:
+                img = call()
+                torch.cuda.synchronize()
+            finally:
+                L.dgs_debug_inject_fault(ctx.ctx, L.DGS_FAULT_SORT_WAIT, 0)
+            assert not img.any()
+            with pytest.raises(L.DgsError) as ei:
+                ctx.render(sid, cams)
+            assert ei.value.code == L.DGS_ERR_TIMEOUT
+            assert torch.equal(call(), ref)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("which", [SORT, SCAN])
+def test_served_request_whose_waits_ran_out(which):
+    sc = synth.scene_small(n_cells=6000)
+    cam = synth.small_camera(96, 64)
+    ctx = Context()
+    try:
+        sid = ctx.upload_scene(sc)
+        ref = _render(ctx, sid, [cam])
+        ctx.serve_start(max_batch=2)
+        out = torch.ones(3 * 96 * 64, device="cuda")
+        for fault, status in ((0, L.DGS_OK), (which, L.DGS_ERR_TIMEOUT), (0, L.DGS_OK)):
+            L.dgs_debug_inject_fault(ctx.ctx, L.DGS_FAULT_SORT_WAIT, fault)
+            try:
+                r = ctx.poll(ctx.submit(sid, cam, out), 10_000_000)
+            finally:
+                L.dgs_debug_inject_fault(ctx.ctx, L.DGS_FAULT_SORT_WAIT, 0)
+            assert r is not None and r.status == status
+            torch.cuda.synchronize()
+            assert torch.equal(out.cpu(), ref if status == L.DGS_OK else torch.zeros_like(ref))
     finally:
         ctx.close()
 
