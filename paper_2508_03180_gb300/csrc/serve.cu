@@ -109,12 +109,13 @@ dgs_status plan_batch(dgs_ctx *ctx, const std::vector<PendingReq> &reqs, BatchPl
     return DGS_OK;
 }
 
-// Device bytes of a slot workspace with capacities c.
+// Device bytes of a slot workspace with capacities c (the buffers of fit_slot; the sort's
+// alternate arrays, two look-back arrays of 256 words per partition, counts and counters).
 long long slot_bytes(const ChainCaps &c) {
     const long long n = std::max(c.E, c.L);
-    return (long long)sizeof(ViewDesc) * c.V + (long long)sizeof(SceneDev) * c.S + 32 * c.E + 4 * c.E / 1024 +
-           8 * n + 1024 * (n / 4096 + 1) + 8 * c.L + 12 * c.T + 48 * c.R + 20 * c.P +
-           (c.W > 0 ? 4 * c.W + 4LL * kDecF * c.R : 0);
+    return (long long)sizeof(ViewDesc) * c.V + (long long)sizeof(SceneDev) * c.S + (long long)sizeof(ChainSizes) +
+           (long long)kSmallBytes + 32 * c.E + 4 * scan_scratch_words(c.E) + 8 * n + 2048 * sort_parts_for(n) + 4112 +
+           8 * c.L + 12 * c.T + 48 * c.R + 20 * c.P + (c.W > 0 ? 4 * c.W + 4LL * kDecF * c.R : 0);
 }
 
 long long grown(long long have, long long need) {

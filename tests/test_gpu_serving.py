@@ -149,6 +149,28 @@ def test_admission_respects_budget(scenes):
     c.close()
 
 
+def test_slot_size_counts_the_sort_scratch():
+    """A slot is sized for max_batch views of the largest resident scene if that fits its
+    share of the budget, else for its batch alone.  The share here would hold such a slot (327,680
+    entries) but for its look-back words, 512 KiB: the request on the larger scene needs
+    another capacity, and another graph."""
+    small, large = (synth.make_scene(n, 1, synth._box(-1, 1), 0.1, 0.2, 0, seed=4) for n in (60, 32768))
+    for s in (small, large):
+        s.cell_center[:, 1] -= 100.0  # behind the camera: no pairs
+    E = 8 * 32768 * 5 // 4
+    without = (32 + 8 + 48) * E + E // 256 + 20 * 5 * 2 * 256 + 8 * 1280
+    scenes = sum(4 * (11 + 11 + 3) * n * 9 // 8 for n in (60, 32768))
+    c = _ctx(hbm_budget_bytes=2 * (without + 300_000) + scenes)
+    ids = [c.upload_scene(s) for s in (small, large)]
+    c.serve_start(max_batch=8)
+    out = torch.zeros(3 * 16 * 16, device="cuda")
+    for sid in ids:
+        assert c.poll(c.submit(sid, synth.small_camera(16, 16), out), -1).status == 0
+    assert c.serve_stats()["graphs_captured"] == 2
+    assert not out.any()
+    c.close()
+
+
 def test_poll_timeout_and_errors(scenes):
     from paper_2508_03180_gb300 import _lib as L
     # a budget below one request: one chain in flight, one view per chain, so
