@@ -173,8 +173,6 @@ SortScratch sort_scratch_of(Workspace &ws) {
     s.status = (uint32_t *)ws.sort_status.p;
     s.counters = (uint32_t *)ws.sort_ctr.p;
     s.err = (uint32_t *)ws.small.p + kSmallSortErr;
-    s.cap_items = (long long)(ws.sort_k.cap / 4);
-    s.cap_parts = (long long)(ws.sort_status.cap / 2048);
     return s;
 }
 

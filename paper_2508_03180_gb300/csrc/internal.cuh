@@ -158,7 +158,6 @@ struct SortScratch {
     uint32_t *status;                // 2 * parts * 256 (alternate passes)
     uint32_t *counters;              // 4 (one per pass)
     uint32_t *err;                   // 1
-    long long cap_items, cap_parts;
 };
 long long sort_parts_for(long long n);
 // Stable LSD radix sort of (key, val) by the low `bits` bits.  Results end in
@@ -169,8 +168,8 @@ int radix_sort_pairs(uint32_t *keys, uint32_t *vals, long long n, int bits, cons
 // pass's sort_status_words(n) look-back words cleared already (BinPrep).  Returns
 // true if the result is in the alternate buffers.  d_n: the count in device memory,
 // n being the capacity.  d_live: items with key 0xFFFFFFFF, in no count, are left
-// out and *d_live remain.  skip_trivial: passes whose digit is 0 in every key are
-// skipped on the device, and the result is copied back (false returned).
+// out and *d_live remain.  skip_trivial (without d_live): passes whose digit is 0 in
+// every key are skipped on the device, and the result is copied back (false returned).
 bool radix_sort_counted(uint32_t *keys, uint32_t *vals, long long n, int bits, const SortScratch &s, cudaStream_t st,
                         const uint32_t *d_n, const uint32_t *d_live, bool skip_trivial);
 long long sort_status_words(long long n);

@@ -90,7 +90,8 @@ __device__ __forceinline__ uint32_t ld_volatile(const uint32_t *p) { return *(co
 // nothing; every pass then takes its input from the buffer the previous
 // non-trivial pass wrote, and the look-back arrays alternate over non-trivial
 // passes.  With d_live, pass 0 leaves out the items whose key is 0xFFFFFFFF (they are
-// not in the histograms), *d_live stay, and later passes sort those.
+// not in the histograms), *d_live stay, and later passes sort those; no pass is
+// skipped then (a skipped first pass would leave nothing out).
 __device__ __forceinline__ bool rs_trivial(const uint32_t *hist, int q, long long n) {
     return (long long)hist[256 * q] == n;
 }
@@ -124,10 +125,9 @@ __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_pass(uint32_t *__restrict_
     if (d_live && pass > 0) n = *d_live;
     int ord = pass;  // non-trivial passes before this one
     if (skip_trivial) {
-        const long long total = d_live ? (long long)*d_live : n;
-        if (rs_trivial(hist, pass, total)) return;
+        if (rs_trivial(hist, pass, n)) return;
         ord = 0;
-        for (int q = 0; q < pass; ++q) ord += rs_trivial(hist, q, total) ? 0 : 1;
+        for (int q = 0; q < pass; ++q) ord += rs_trivial(hist, q, n) ? 0 : 1;
     }
     const int shift = 8 * pass;
     const uint32_t *__restrict__ kin = (ord & 1) ? k1 : k0;
@@ -326,7 +326,7 @@ long long sort_status_words(long long n) {
 bool radix_sort_counted(uint32_t *keys, uint32_t *vals, long long n, int bits, const SortScratch &s, cudaStream_t st,
                         const uint32_t *d_n, const uint32_t *d_live, bool skip_trivial) {
     if (n <= 0 || bits <= 0) return false;
-    return radix_passes(keys, vals, n, (bits + 7) / 8, s, st, d_n, d_live, skip_trivial);
+    return radix_passes(keys, vals, n, (bits + 7) / 8, s, st, d_n, d_live, skip_trivial && !d_live);
 }
 
 int radix_sort_pairs(uint32_t *keys, uint32_t *vals, long long n, int bits, const SortScratch &s, cudaStream_t st) {

@@ -68,8 +68,6 @@ extern "C" dgs_status dgs_sort_pairs_noalloc(uint32_t *keys, uint32_t *vals, int
     sc.status = base + kOffStatus;
     sc.counters = base + kOffCounters;
     sc.err = base + kOffErr;
-    sc.cap_items = kMaxItems;
-    sc.cap_parts = kMaxParts;
     cudaStream_t st = (cudaStream_t)stream;
     // the array keeps the previous call's contents: the error flag starts at
     // zero here; histograms, counters and look-back words are cleared by the
