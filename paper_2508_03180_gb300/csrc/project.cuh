@@ -107,9 +107,9 @@ __device__ __forceinline__ void proj_core(const ViewDesc &Vw, const GaussIn &p, 
 
 // The 48-byte record of Gaussian p in view Vw.  A Gaussian that is not drawn gets
 // ext = -1, so no AABB test passes: its mean is not in front of the near plane, or its
-// projection is not a number (a zero quaternion, a NaN parameter, a screen covariance
-// beyond FP32).  The blends rely on it: they give a pixel outside the box an offset of
-// kFar in place of a branch, and that is alpha = 0 only where L is a number.  For the
+// projection or opacity is not a number (a zero quaternion, a NaN parameter, a screen
+// covariance beyond FP32).  The blends rely on it: they give a pixel outside the box an offset of
+// kFar in place of a branch, and that is alpha = 0 only where L and the opacity are numbers.  For the
 // same reason colours are at most kMaxColour (a decoder's NaN too): an alpha or a weight
 // of 0 times a cell's colours is then 0, at pixels that a Gaussian does not reach and at those
 // finished before its cell.  k: SH coefficients, cv: the cell's v_n.  Returns whether it
@@ -148,7 +148,7 @@ __device__ __forceinline__ bool gauss_record(const ViewDesc &Vw, const GaussIn &
     const float ip = rsqrtf(sc2.syy * sc2.det);
     const float fp = sc2.syy * ip, fr = -sc2.sxy * ip, ft = rsqrtf(sc2.syy);
     // (every term is >= 0 or not a number)
-    if (!(fabsf(mx) + fabsf(my) + ex + ey + fp + fabsf(fr) + ft >= 0.f)) return not_drawn();
+    if (!(fabsf(mx) + fabsf(my) + ex + ey + fp + fabsf(fr) + ft + fabsf(opac) >= 0.f)) return not_drawn();
     float col[3];
     if (DIRECT_RGB) {
 #pragma unroll

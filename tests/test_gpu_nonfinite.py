@@ -82,6 +82,28 @@ def test_undefined_gaussian_is_not_drawn(damage, opaque, flags, large):
         ctx.close()
 
 
+@pytest.mark.parametrize("cfg", [dict(), dict(dilation=0.0), dict(flags=2)])
+def test_undefined_opacity_is_not_drawn(cfg):
+    """(By the hybrid renderer; the comparators take alpha_max within the box.)"""
+    sc = synth.make_scene(24, 4, synth._box(-0.5, 0.5), 0.1, 0.4, 0, seed=37)
+    bad = np.arange(3, sc.G, 8)
+    ref = copy.deepcopy(sc)
+    ref.g_mean[bad, 1] = -3.0  # not in front of the near plane
+    sc.g_logit[bad] = np.nan
+    ctx = Context(**cfg)
+    try:
+        (got, alpha, wsr), g_got = _images(ctx, sc, [CAM])
+        (want, _, _), g_want = _images(ctx, ref, [CAM])
+        assert torch.equal(got, want) and want.any()
+        assert torch.isfinite(alpha).all() and torch.isfinite(wsr).all()
+        live = np.setdiff1d(np.arange(sc.G), bad)
+        for k in g_want:
+            a, b = (g_got[k], g_want[k]) if k == "g_cell_v" else (g_got[k][live], g_want[k][live])
+            assert (a - b).norm() <= 1e-5 * b.norm(), k
+    finally:
+        ctx.close()
+
+
 def test_flat_gaussian_without_dilation():
     """A needle seen obliquely: its screen covariance is singular, L infinite and its exponent
     infinite or inf - inf.  The forward draws nothing of it, and the adjoint's replay agrees."""
