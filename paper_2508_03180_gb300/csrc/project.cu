@@ -167,9 +167,7 @@ __global__ void __launch_bounds__(128) k_gauss_bin(const ViewDesc *__restrict__ 
             const ViewDesc &Vw = views[v];
             ProjCore c;
             float4 r0, r1, r2;
-            // (the comparators' blend tests every pixel: a NaN opacity is alpha_max within the box there)
-            bool vis = gauss_record(Vw, p, k, sc.sh_degree, opac == opac ? opac : 0.f, cv, bp, c, r0, r1, r2);
-            r1.w = opac;
+            bool vis = gauss_record<false, true>(Vw, p, k, sc.sh_degree, opac, cv, bp, c, r0, r1, r2);
             if (wsr) {
                 const float w = tau > 0.f ? fmaxf(0.f, 1.f - c.t[2] / tau) * cv : cv;
                 vis = vis && w > 0.f;

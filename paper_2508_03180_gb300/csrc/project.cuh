@@ -114,7 +114,9 @@ __device__ __forceinline__ void proj_core(const ViewDesc &Vw, const GaussIn &p, 
 // of 0 times a cell's colours is then 0, at pixels that a Gaussian does not reach and at those
 // finished before its cell.  k: SH coefficients, cv: the cell's v_n.  Returns whether it
 // is drawn; c keeps the view-space mean.
-template <bool DIRECT_RGB = false>
+// EACH_PIXEL: for the comparators, whose blend tests every pixel (an opacity that is not a
+// number is drawn, and makes alpha_max within the box).
+template <bool DIRECT_RGB = false, bool EACH_PIXEL = false>
 __device__ __forceinline__ bool gauss_record(const ViewDesc &Vw, const GaussIn &p, const float (&k)[16][3],
                                              int sh_degree, float opac, float cv, const BlendParams &bp,
                                              ProjCore &c, float4 &r0, float4 &r1, float4 &r2,
@@ -148,7 +150,7 @@ __device__ __forceinline__ bool gauss_record(const ViewDesc &Vw, const GaussIn &
     const float ip = rsqrtf(sc2.syy * sc2.det);
     const float fp = sc2.syy * ip, fr = -sc2.sxy * ip, ft = rsqrtf(sc2.syy);
     // (every term is >= 0 or not a number)
-    if (!(fabsf(mx) + fabsf(my) + ex + ey + fp + fabsf(fr) + ft + fabsf(opac) >= 0.f)) return not_drawn();
+    if (!(fabsf(mx) + fabsf(my) + ex + ey + fp + fabsf(fr) + ft + (EACH_PIXEL ? 0.f : fabsf(opac)) >= 0.f)) return not_drawn();
     float col[3];
     if (DIRECT_RGB) {
 #pragma unroll
