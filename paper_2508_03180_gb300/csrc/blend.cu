@@ -11,7 +11,8 @@
 // order of k (Eq. 12's inner sums and product commute).
 //
 // GB300 mapping: one one-warp CTA per 16x8 half of a 16x16 tile, four
-// pixels per lane in packed pairs (f32x2 arithmetic).  The 48-byte records of
+// pixels per lane in packed pairs (f32x2 arithmetic), or per 16x4 quarter, two
+// pixels per lane, where there are few tiles (kFewTiles).  The 48-byte records of
 // the cells' Gaussians are copied into the warp's shared memory asynchronously,
 // ahead of their use, and broadcast from there to the warp's 128 pixels.
 #include <algorithm>
@@ -496,13 +497,12 @@ void launch_count_pairs(const ViewDesc *views, int n_views, int total_tiles, con
 //     dL/dv_n   = T_n (dN.A_n + dD B_n) - S_n sum_k alpha_k / (1 - v alpha_k)
 // then alpha = sigma G' (unless clamped) and G' = exp(-q/2).
 //
-// Same work unit as the forward (one warp per 16x8 sub-tile, four pixels per
-// lane).  Per cell, the warp replays its pixels keeping G' of the Gaussians
-// that reach the sub-tile in warp-private shared memory, updates S and T,
-// then for each such Gaussian sums its pixels' nine screen-space gradient
-// terms across the warp with a transposed shuffle tree (each step halves the
-// values a lane carries) and adds the totals to global memory (one atomic
-// add per value per sub-tile).
+// Same work unit as the forward (one warp per sub-tile).  Per cell, the warp
+// replays its pixels keeping G' of the Gaussians that reach the sub-tile in
+// warp-private shared memory and updates S and T; then groups of eight lanes take
+// a Gaussian each and sum its nine screen-space gradient terms over the
+// sub-tile's pixels, and the totals are added to global memory (one
+// atomic add per value per sub-tile): see k_blend_bwd.
 
 // Sums of eight per-lane values over the eight lanes of a group (lanes that
 // differ in bits 0..2): three halving steps (offsets 4, 2, 1) in which each

@@ -35,7 +35,10 @@ constexpr int CSUB = kTile / CROWS;  // sub-tiles per tile
 // per pixel and records fetched through registers took 617 us for one 1080p view of
 // 1M Gaussians, 476 this way (the whole call 992 -> 840 us); without the minimum with
 // alpha_max where no opacity reaches it and with paired offsets the call went from
-// 788 to 762.
+// 788 to 762.  Small views gain as well, though the scalar form's sub-tiles were 16x4
+// (alpha-blending / weighted sums, us a call: 320x240 of 20,000 x 8 421 -> 299 / 744 -> 469,
+// 640x480 of 20,000 x 10 over three decades 367 -> 255 / 288 -> 212, 160x120 of 2,048 x 8
+// 389 -> 233 / 319 -> 216); packed 16x4 sub-tiles are not measured.
 // ONCE: eps > 1, where the first entry that reaches a pixel is also its last, even at an
 // alpha of 0, which leaves T at 1 (an instantiation of its own: the mask of such pixels
 // spills at the 64 registers of the others).

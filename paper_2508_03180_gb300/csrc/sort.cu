@@ -1,10 +1,11 @@
 // Stable LSD radix sort of (uint32 key, uint32 value) pairs, 8-bit digits,
-// one "onesweep" pass per digit: every CTA ranks a 3072-item partition
-// locally, then learns the global offset of each digit from its predecessors
-// through decoupled look-back (Merrill & Garland single-pass prefix scan,
-// applied per digit as in Adinets & Merrill's Onesweep), and writes the
-// partition out through shared memory in digit order (coalesced runs).  The digit
-// histograms of all passes come from one upfront read of the keys.
+// one "onesweep" pass per digit: every CTA ranks a partition (3072 items, or 1024 in
+// small sorts) locally, reorders it by digit in shared memory, learns the global
+// offset of each digit from its predecessors through decoupled look-back (Merrill &
+// Garland single-pass prefix scan, applied per digit as in Adinets & Merrill's
+// Onesweep), and writes coalesced runs.  The digit counts of all passes are there
+// beforehand: a render's kernels count the keys that they write (BinPrep), and
+// radix_sort_pairs reads its keys once for them.
 //
 // Sec. IV-B sorts the cell sequence with a radix sort; its cost grows with
 // the sequence length, which is why the sort runs over cells, not Gaussians
