@@ -342,11 +342,12 @@ __global__ void k_tile_ranges(const uint32_t *__restrict__ key, long long L, con
                               uint2 *__restrict__ ranges, const uint32_t *__restrict__ err,
                               uint32_t *__restrict__ host_err) {
     chain_wait();
-    if (*err) {
+    const uint32_t gave_up = *err;  // (requested together with the count)
+    if (d_L) L = *d_L;
+    if (gave_up) {
         if (host_err && blockIdx.x == 0 && threadIdx.x == 0) *host_err = 1u;
         return;
     }
-    if (d_L) L = *d_L;
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < L; j += (long long)gridDim.x * blockDim.x) {
         const uint32_t k = key[j];
         if (j == 0 || key[j - 1] != k) ranges[k].x = (uint32_t)j;
