@@ -13,7 +13,9 @@
  *     rendering); across cells the weights w_n = v_n T_n^cell follow
  *     alpha-blending style transmittance, and blending halts once T^cell
  *     drops below eps (Sec. V, Eq. 12-14).  A Gaussian is skipped at a pixel
- *     outside its screen AABB (Sec. VI-A).
+ *     outside its screen AABB (Sec. VI-A).  One whose projection or opacity
+ *     is not a number (a zero quaternion, a NaN parameter) is not drawn;
+ *     colours are held to 1e25.
  *   * render_backward is the adjoint of that image with respect to every
  *     Gaussian parameter (the paper trains through this renderer, Sec. VI).
  *
